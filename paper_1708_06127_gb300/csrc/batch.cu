@@ -546,10 +546,18 @@ static void engine_setup(Engine& E, int K, const viecut_opts& o) {
   E.list_nois.ensure_n<int32_t>(K);
   E.sideK.ensure_n<unsigned char>((int64_t)K * kDenseMax);
   E.noiCurK.ensure_n<int32_t>((int64_t)kSMs * kNoiDenseBlocksPerSM * kDenseMax);  // per dense-step block
-  VC_CUDA(cudaMemsetAsync(E.phase.p, 0, sizeof(int) * K, E.stream));
+  // Slots nothing joined yet are visited by the per-slot kernels too (first, did and nv
+  // say what to skip): every array starts from zero, and every phase from kBGone, in the
+  // engine's own stream order.
+  for (Buf* b : {&E.phase, &E.level, &E.run, &E.any, &E.changed, &E.contracted, &E.first, &E.did, &E.best_kind,
+                 &E.trace_len, &E.nv, &E.nv_new, &E.nnz, &E.n_start, &E.lam, &E.best_vertex, &E.argmin, &E.dmin,
+                 &E.obase, &E.norig, &E.n1, &E.noi_base, &E.vbase, &E.vbase_new, &E.gkey, &E.seed, &E.gact,
+                 &E.summary, &E.list_noid, &E.list_nois})
+    VC_CUDA(cudaMemsetAsync(b->p, 0, b->cap, E.stream));
   {
-    std::vector<int> gone(K, kBGone);
-    VC_CUDA(cudaMemcpy(E.phase.p, gone.data(), sizeof(int) * K, cudaMemcpyHostToDevice));
+    const std::vector<int> gone(K, kBGone);
+    VC_CUDA(cudaMemcpyAsync(E.phase.p, gone.data(), sizeof(int) * K, cudaMemcpyHostToDevice, E.stream));
+    VC_CUDA(cudaStreamSynchronize(E.stream));  // the host vector goes out of scope
   }
   VC_CUDA(cudaMallocHost(&E.h_summary, sizeof(int) * kSummaryInts));
   E.ws = new Workspace;
