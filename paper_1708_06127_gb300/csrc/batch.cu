@@ -30,6 +30,7 @@ namespace vc {
 enum BPhase { kBLP = 0, kBPRA = 1, kBPRB = 2, kBNoiS = 3, kBNoiD = 4, kBDone = 5, kBGone = 6 };
 constexpr int kBTraceCap = 512;
 constexpr int kSummaryInts = 16;
+constexpr int kSides = kNoiClasses + 1;  // streams of the exact-step phases
 
 // Device arrays of the per-graph state (K graphs).
 struct BState {
@@ -41,8 +42,10 @@ struct BState {
   unsigned long long* seed;
   unsigned char* gact;
   TraceStep* trace;
-  int* summary;  // [0..6] phase counts, [7] max n among NOI_D graphs, [8] contract or drop count
-  int32_t *list_noid, *list_nois;
+  // [0..6] phase counts, [7] max n among NOI_D graphs, [8] contract or drop count, [9] listed
+  // NOI_D graphs, [12..15] listed NOI_S graphs by size class
+  int* summary;
+  int32_t *list_noid, *list_nois;  // list_nois: K entries per size class
 };
 
 // ---------------------------------------------------------------- union setup
@@ -237,8 +240,8 @@ __global__ void b_summary_k(int K, BState S) {
       atomicMax(&S.summary[7], (int)S.nv[g]);
       S.noi_base[g] = S.vbase[g];
     } else if (ph == kBNoiS) {
-      S.list_nois[atomicAdd(&S.summary[10], 1)] = g;
-      atomicMax(&S.summary[11], (int)S.nv[g]);
+      const int cls = noi_class(S.nv[g]);
+      S.list_nois[cls * K + atomicAdd(&S.summary[12 + cls], 1)] = g;
     }
   }
 }
@@ -483,10 +486,11 @@ struct Engine {
   Buf gidA, gidB;
   int32_t* gid = nullptr;
   Buf vact, sideK, noiM, noiCurK, noiQ;
-  // the exact-step phases run on their own stream beside the other phases of a
-  // super-step (they touch only their graphs' vertices and state)
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // the exact-step phases run on streams of their own (sparse rounds by size class, then
+  // the dense step) beside the other phases of a super-step (they touch only their graphs'
+  // vertices and state)
+  cudaStream_t side[kSides] = {};
+  cudaEvent_t ev_fork = nullptr, ev_join[kSides] = {};
   Buf om0, oc1, os1;  // per original vertex
   int64_t ocap = 0;
   Workspace* ws = nullptr;
@@ -496,8 +500,10 @@ struct Engine {
     delete ws;
     if (h_summary) cudaFreeHost(h_summary);
     if (ev_fork) cudaEventDestroy(ev_fork);
-    if (ev_join) cudaEventDestroy(ev_join);
-    if (side) cudaStreamDestroy(side);
+    for (int i = 0; i < kSides; ++i) {
+      if (ev_join[i]) cudaEventDestroy(ev_join[i]);
+      if (side[i]) cudaStreamDestroy(side[i]);
+    }
     if (own_stream && stream) cudaStreamDestroy(stream);
   }
   BState state() {
@@ -528,9 +534,11 @@ static void engine_setup(Engine& E, int K, const viecut_opts& o) {
     VC_CUDA(cudaStreamCreateWithFlags(&E.stream, cudaStreamNonBlocking));
     E.own_stream = true;
   }
-  VC_CUDA(cudaStreamCreateWithFlags(&E.side, cudaStreamNonBlocking));
   VC_CUDA(cudaEventCreateWithFlags(&E.ev_fork, cudaEventDisableTiming));
-  VC_CUDA(cudaEventCreateWithFlags(&E.ev_join, cudaEventDisableTiming));
+  for (int i = 0; i < kSides; ++i) {
+    VC_CUDA(cudaStreamCreateWithFlags(&E.side[i], cudaStreamNonBlocking));
+    VC_CUDA(cudaEventCreateWithFlags(&E.ev_join[i], cudaEventDisableTiming));
+  }
   for (Buf* b : {&E.phase, &E.level, &E.run, &E.any, &E.changed, &E.contracted, &E.first, &E.did, &E.best_kind,
                  &E.trace_len})
     b->ensure_n<int>(K);
@@ -543,7 +551,7 @@ static void engine_setup(Engine& E, int K, const viecut_opts& o) {
   E.trace.ensure_n<TraceStep>((int64_t)K * kBTraceCap);
   E.summary.ensure_n<int>(kSummaryInts);
   E.list_noid.ensure_n<int32_t>(K);
-  E.list_nois.ensure_n<int32_t>(K);
+  E.list_nois.ensure_n<int32_t>((int64_t)kNoiClasses * K);
   E.sideK.ensure_n<unsigned char>((int64_t)K * kDenseMax);
   E.noiCurK.ensure_n<int32_t>((int64_t)kSMs * kNoiDenseBlocksPerSM * kDenseMax);  // per dense-step block
   // Slots nothing joined yet are visited by the per-slot kernels too (first, did and nv
@@ -612,13 +620,14 @@ static bool engine_step(Engine& E) {
   // beside label propagation and Padberg-Rinaldi on the others; buffers grow first (a
   // reallocation waits for the device)
   const bool exact = cnt[kBNoiS] > 0 || cnt[kBNoiD] > 0;
+  bool forked[kSides];
+  for (int i = 0; i < kSides; ++i) forked[i] = i < kNoiClasses ? cnt[12 + i] > 0 : cnt[kBNoiD] > 0;
   if (exact) {
     long long* M = nullptr;
     int64_t mcap = 0;
     int blocks = 0;
     if (cnt[kBNoiS] > 0) {
       W.noi_r.ensure_n<long long>(noi_round_scratch(G.n));
-      W.noi_seen.ensure_n<int>(G.n);
       E.noiQ.ensure_n<int32_t>(G.n);
     }
     if (cnt[kBNoiD] > 0) {
@@ -629,16 +638,23 @@ static bool engine_step(Engine& E) {
       M = E.noiM.ensure_n<long long>(2 * mcap * blocks);
     }
     VC_CUDA(cudaEventRecord(E.ev_fork, s));
-    VC_CUDA(cudaStreamWaitEvent(E.side, E.ev_fork, 0));
-    if (cnt[kBNoiS] > 0)
-      noi_round_batch(G, S.list_nois, cnt[10], S.vbase, S.nv, S.lam, W.noi_r.as<long long>(),
-                      W.noi_seen.as<int>(), E.noiQ.as<int32_t>(), F, S.changed, cnt[11], E.side);
+    // the largest graphs first: their chains are the longest
+    for (int cls = kNoiClasses - 1; cls >= 0; --cls) {
+      if (cnt[12 + cls] == 0) continue;
+      cudaStream_t t = E.side[cls];
+      VC_CUDA(cudaStreamWaitEvent(t, E.ev_fork, 0));
+      noi_round_batch(G, S.list_nois + (int64_t)cls * K, cnt[12 + cls], S.vbase, S.nv, S.lam,
+                      W.noi_r.as<long long>(), E.noiQ.as<int32_t>(), F, S.changed, cls, t);
+      VC_CUDA(cudaEventRecord(E.ev_join[cls], t));
+    }
     if (cnt[kBNoiD] > 0) {
+      cudaStream_t t = E.side[kNoiClasses];
+      VC_CUDA(cudaStreamWaitEvent(t, E.ev_fork, 0));
       BatchNoi bn{S.lam, S.best_kind, S.nv, S.nnz, S.dmin, S.argmin, S.trace_len, S.trace, kBTraceCap, S.level};
       noi_dense_batch(G, S.list_noid, cnt[kBNoiD], S.vbase, S.nv, M, mcap, blocks, E.noiCurK.as<int32_t>(),
-                      E.sideK.as<unsigned char>(), bn, E.side);
+                      E.sideK.as<unsigned char>(), bn, t);
+      VC_CUDA(cudaEventRecord(E.ev_join[kNoiClasses], t));
     }
-    VC_CUDA(cudaEventRecord(E.ev_join, E.side));
   }
   BatchCtx bc;
   bc.gid = E.gid;
@@ -674,7 +690,8 @@ static bool engine_step(Engine& E) {
     pr_partners(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), s);
     pr_pass_b(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), W.st(), F, nullptr, s, &bc);
   }
-  if (exact) VC_CUDA(cudaStreamWaitEvent(s, E.ev_join, 0));
+  for (int i = 0; i < kSides; ++i)
+    if (forked[i]) VC_CUDA(cudaStreamWaitEvent(s, E.ev_join[i], 0));
   b_decide_k<<<gK, 256, 0, s>>>(K, S);
   count_launch();
   read_summary(E);

@@ -73,7 +73,7 @@ struct Workspace {
   cudaStream_t s = nullptr;
   // vertex-sized
   Buf deg, labA, labB, map0, cidT, cur1, side1, flags, rank, cnt, pos, scan64, scan32, hv;
-  Buf partner, pw, parent, slist, rlist, mlist, blist, glist, bl1, bcounts, noi_r, noi_seen;
+  Buf partner, pw, parent, slist, rlist, mlist, blist, glist, bl1, bcounts, noi_r;
   // entry-sized
   Buf tmpK, tmpV, cmpK, cmpV;
   // pair-sized

@@ -284,8 +284,8 @@ void noi_dense(const GraphView& g, long long* M0, long long* M1, int32_t* curK, 
 // Scratch of a sparse exact-step round (r of noi_round_sparse / noi_round_batch), in
 // int64 entries, for a graph (or union) of n vertices: attachments, then chunk bounds.
 inline int64_t noi_round_scratch(int64_t n) { return 2 * n + 64; }
-void noi_round_sparse(const GraphView& g, const DevState* st, long long* r, int* seen,
-                      int32_t* parent, int32_t* labels, int* changed, cudaStream_t s);
+void noi_round_sparse(const GraphView& g, const DevState* st, long long* r, int32_t* parent, int32_t* labels,
+                      int* changed, cudaStream_t s);
 
 // Per-graph result arrays of a batch's exact step (indexed by graph; trace holds
 // trace_cap steps per graph).
@@ -309,9 +309,14 @@ constexpr int kNoiDenseBlocksPerSM = 4;
 void noi_dense_batch(const GraphView& u, const int32_t* list, int count, const long long* vbase, const long long* nv,
                      long long* M, int64_t mcap, int blocks, int32_t* curK, unsigned char* sideK, const BatchNoi& bn,
                      cudaStream_t s);
-// One sparse round for each listed graph; labels and gchanged written per graph.
-// max_n: the largest listed graph (its state then fits in shared memory; 0 = unknown)
+// One sparse round for each listed graph of size class cls; labels and gchanged written
+// per graph.  The classes (2048, 4096, 8192 vertices, more) hold a block's shared memory
+// to its graph's size: a block's time is a chain of dependent steps, so blocks in flight
+// per SM count.
+constexpr int kNoiClasses = 4;
+__host__ __device__ constexpr int noi_class_max(int cls) { return cls == kNoiClasses - 1 ? 0x7fffffff : 2048 << cls; }
+__host__ __device__ constexpr int noi_class(long long n) { return n <= 2048 ? 0 : n <= 4096 ? 1 : n <= 8192 ? 2 : 3; }
 void noi_round_batch(const GraphView& u, const int32_t* list, int count, const long long* vbase, const long long* nv,
-                     const long long* glam, long long* r, int* seen, int32_t* parent, int32_t* labels,
-                     int* gchanged, int max_n, cudaStream_t s);
+                     const long long* glam, long long* r, int32_t* parent, int32_t* labels, int* gchanged, int cls,
+                     cudaStream_t s);
 }  // namespace vc

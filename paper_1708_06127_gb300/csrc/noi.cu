@@ -10,9 +10,11 @@
 #include <limits.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
 #include <string>
-#include <unordered_map>
+#include <type_traits>
+#include <utility>
 
 #include "kernels.cuh"
 #include "viecut.h"
@@ -61,6 +63,265 @@ __device__ __forceinline__ int warp_argmax_unseen(const long long* r, const int*
   return bx;
 }
 
+// ------------------------------------------------------------ a round as closures
+// Call a vertex "low" when it is visited with attachment r < max(lambda-hat, 1).  When a
+// low vertex u is visited every unvisited r is at most r(u), so no unvisited vertex has
+// reached lambda-hat; the vertices visited after u up to the next low vertex are then
+// exactly the closure of u: the smallest set R holding u such that every vertex outside R
+// and outside the earlier runs has fewer than lambda-hat of weight into the vertices
+// visited so far.  Adding a vertex only raises the weights into the set, so the closure
+// does not depend on the order in which its vertices are added, and neither do the
+// attachments of the vertices left afterwards; the next low vertex (the largest r, ties
+// to the smallest id) is therefore the same as in the maximum-adjacency order.  The round
+// unites every x, y with r(y) >= lambda-hat once x's edge is added; each such pair lies
+// within one run, and every vertex of a run is joined to the vertex whose edge raised it
+// to lambda-hat (visited inside the run), so the round's components are the runs and the
+// union-find with smallest-id roots labels each run with its smallest id.
+//
+// So a round needs the exact order only to pick each run's first vertex (an argmax over
+// the vertices not yet taken); a run then grows level by level, the block relaxing all
+// vertices of a level at once, a warp per list (a level of few vertices splits its lists
+// over the warps).  The time is a chain of dependent steps -- a level waits for its lists
+// (one L2 access), its shared-memory additions and one barrier -- so what counts is the
+// cost of a step: the state of the graph sits in shared memory (attachments, queue, list
+// offsets), and r holds the attachment less lam = max(lambda-hat, 1): a vertex is taken
+// exactly when its r is not negative (an untaken one stays below lam; a run's first vertex
+// is raised to 0 when it is chosen), so that one addition tests, raises and takes, and
+// the untaken vertex of largest attachment holds the largest r read as unsigned.
+//
+// Measured (RHG n = 8191, average degree 32, unit weights: 612 runs, 2174 levels): 1.66 ms a
+// round, about 1400 cycles a level (450 of them the lists' L2 access) and 1100 a choice,
+// against 4.47 ms for one warp over the same state.  8 and 4 warps take 1.70 and 2.05 ms;
+// lists prefetched into L1 when a vertex is first touched, the same time.
+//
+// Vertices are local ids of the graph [lo, lo + n).
+struct NoiShared {
+  int cnt[3];     // vertices taken in a level, by level modulo 3
+  int runmin[2];  // smallest id of a run, by run modulo 2
+  unsigned long long red_v[32];
+  int red_i[32];
+};
+
+// The state in shared memory.  R = int serves graphs in which lam x entries stays below
+// 2^31: weights are cut to lam (which crosses it as the weight itself does), so no sum
+// wraps.  kOff: the list offsets are kept too (they are read from goff otherwise).
+template <typename RT, typename OT, bool kOff>
+struct ClosureSmem {
+  using R = RT;
+  using O = OT;
+  static constexpr bool kBounds = false;
+  R* r;  // 16-byte aligned, a multiple of 4 entries (0, as taken, past n)
+  OT* soff;
+  uint16_t* queue;
+  const int64_t* goff;  // the graph's offsets
+  int64_t e0;           // its first entry
+  __device__ __forceinline__ void init(int n, R lam) const {
+    const int T = blockDim.x;
+    for (int k = threadIdx.x; k < ((n + 3) & ~3); k += T) r[k] = k < n ? -lam : 0;
+    if (kOff)
+      for (int k = threadIdx.x; k <= n; k += T) soff[k] = (OT)(goff[k] - e0);
+  }
+  __device__ __forceinline__ OT beg(int x) const { return kOff ? soff[x] : (OT)(__ldg(goff + x) - e0); }
+  __device__ __forceinline__ OT end(int x) const { return kOff ? soff[x + 1] : (OT)(__ldg(goff + x + 1) - e0); }
+};
+
+// The state in global memory (graphs beyond the shared-memory size), read past the L1
+// cache, which the atomic operations do not update.  cmax[c] bounds the unsigned values
+// of chunk c's 32 vertices that are untaken from above (0: all taken).
+struct ClosureGlobal {
+  using R = long long;
+  using O = int64_t;
+  static constexpr bool kBounds = true;
+  R* r;
+  unsigned long long* cmax;
+  int32_t* queue;
+  const int64_t* goff;
+  int64_t e0;
+  __device__ __forceinline__ void init(int n, R lam) const {
+    const int T = blockDim.x;
+    for (int k = threadIdx.x; k < n; k += T) __stcg(r + k, -lam);
+    for (int k = threadIdx.x; k < ((n + 31) >> 5); k += T) __stcg(cmax + k, (unsigned long long)-lam);
+  }
+  __device__ __forceinline__ int64_t beg(int x) const { return __ldg(goff + x) - e0; }
+  __device__ __forceinline__ int64_t end(int x) const { return __ldg(goff + x + 1) - e0; }
+};
+
+__device__ __forceinline__ unsigned warp_max_r(unsigned x) { return __reduce_max_sync(0xffffffffu, x); }
+__device__ __forceinline__ unsigned long long warp_max_r(unsigned long long x) {
+  const unsigned hi = (unsigned)(x >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)x : 0u);
+  return ((unsigned long long)mh << 32) | ml;
+}
+
+// The largest v of the block and the smallest i holding it (i >= 0), in every thread.
+// One barrier; red_v and red_i may be written again after the next one.
+template <int NW, typename R>
+__device__ __forceinline__ int block_argmax(R v, int i, R* top, NoiShared& sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const R wv = warp_max_r(v);
+  const unsigned wi = __reduce_min_sync(0xffffffffu, v == wv ? (unsigned)i : 0xffffffffu);
+  if (lane == 0) {
+    sh.red_v[wid] = wv;
+    sh.red_i[wid] = (int)wi;
+  }
+  __syncthreads();
+  const R bv = lane < NW ? (R)((volatile unsigned long long*)sh.red_v)[lane] : (R)0;
+  const unsigned bi = lane < NW ? (unsigned)((volatile int*)sh.red_i)[lane] : 0xffffffffu;
+  *top = warp_max_r(bv);
+  return (int)__reduce_min_sync(0xffffffffu, bv == *top ? bi : 0xffffffffu);
+}
+
+// lam x entries (and the offsets) below 2^31: 32-bit values do not wrap.
+__device__ __forceinline__ bool noi_fits32(long long lam, int64_t entries) {
+  return lam < INT_MAX && entries < INT_MAX && (lam > 1 ? lam : 1) * entries < INT_MAX;
+}
+
+// Shared-memory additions of either width (the 64-bit one is declared unsigned).
+__device__ __forceinline__ int noi_add(int* p, int x) { return atomicAdd(p, x); }
+__device__ __forceinline__ long long noi_add(long long* p, long long x) {
+  return (long long)atomicAdd((unsigned long long*)p, (unsigned long long)x);
+}
+
+constexpr int kNoiUnroll = 4;  // rows of a list in flight per warp while relaxing
+
+// One round by a block of NW warps (a power of two), one graph at a time.  put(x, m)
+// receives every vertex x with the smallest id m of its run.  Returns, in every thread,
+// whether some run holds two or more vertices.  Ends with a barrier.
+template <int NW, typename WT, typename ST, typename PUT>
+__device__ __forceinline__ bool noi_closure_block(int32_t lo, int n, const int32_t* __restrict__ adj,
+                                                  const WT* __restrict__ w, long long lam_in, const ST& S,
+                                                  NoiShared& sh, PUT put) {
+  using R = typename ST::R;
+  using U = typename std::make_unsigned<R>::type;
+  using OT = typename ST::O;
+  using QT = typename std::remove_pointer<decltype(ST::queue)>::type;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  const R lam = (R)(lam_in > 1 ? lam_in : 1);  // weights >= 1: a first addition crosses any bound below 1
+  const int64_t e0 = S.e0;
+  S.init(n, lam);
+  if (tid < 3) sh.cnt[tid] = 0;
+  if (tid < 2) sh.runmin[tid] = INT_MAX;
+  __syncthreads();
+  int qt = 0, lev = 0, run = 0;  // taken so far, levels so far modulo 3, runs so far modulo 2
+  bool unites = false;
+  while (qt < n) {
+    // the run's first vertex: the untaken vertex of largest r, ties to the smallest id
+    int u;
+    if constexpr (!ST::kBounds) {
+      // every thread reads its vertices, four at a time; the best four again at the end
+      U bv = 0, top;
+      int bk = tid * 4;
+      auto four = [&](int k, U* x) {
+#pragma unroll
+        for (int q = 0; q < (int)sizeof(R) / 4; ++q) ((uint4*)x)[q] = ((const uint4*)(S.r + k))[q];
+      };
+      for (int k = tid * 4; k < n; k += NW * 128) {
+        U x[4];
+        four(k, x);
+        const U m = max(max(x[0], x[1]), max(x[2], x[3]));
+        if (m > bv) { bv = m; bk = k; }
+      }
+      if (bv) {  // the first of the four (bk is in range: a thread without vertices has bv = 0)
+        U x[4];
+        four(bk, x);
+        bk += x[0] == bv ? 0 : x[1] == bv ? 1 : x[2] == bv ? 2 : 3;
+      }
+      u = block_argmax<NW>(bv, bk, &top, sh);
+    } else {
+      // the chunk of largest bound (ties: the lower chunk), read exactly; a stale bound (its
+      // vertex was taken) is lowered and the choice made again
+      for (;;) {
+        U bv = 0, top;
+        int bc = 0;
+        for (int c = tid; c < ((n + 31) >> 5); c += NW * 32) {
+          const U m = __ldcg(S.cmax + c);
+          if (m > bv) { bv = m; bc = c; }
+        }
+        const int uc = block_argmax<NW>(bv, bc, &top, sh), k = uc * 32 + lane;
+        const R x = k < n ? __ldcg(S.r + k) : 0;
+        const U rv = x < 0 ? (U)x : 0;
+        const U best = warp_max_r(rv);
+        u = uc * 32 + __ffs(__ballot_sync(0xffffffffu, rv == best)) - 1;
+        if (best == top) break;
+        __syncthreads();  // every warp has read the bounds and its copy of the choice
+        if (tid == 0) __stcg(S.cmax + uc, best);
+        __syncthreads();
+      }
+    }
+    // every warp has read the values: the barrier of the choice lies between
+    if (ST::kBounds) __syncthreads();
+    if (tid == 0) {
+      S.r[u] = 0;
+      S.queue[qt] = (QT)u;
+      sh.runmin[run ^ 1] = INT_MAX;  // the last run's, read before this run's first barrier
+    }
+    const int rs = qt;
+    int qh = qt++;
+    while (qh < qt) {
+      const int cnt = qt - qh;
+      int* got = &sh.cnt[lev];
+      lev = lev == 2 ? 0 : lev + 1;
+      if (tid == 0) sh.cnt[lev] = 0;  // last read two barriers ago
+      // a warp per list, or (fewer lists than warps) P warps per list on interleaved rows
+      const int lg = cnt >= NW ? 31 - __clz(NW) : 32 - __clz(cnt - 1);
+      const int P = NW >> lg, part = wid >> lg;
+      for (int i = wid & ((1 << lg) - 1); i < cnt; i += NW) {
+        const int x = qh == rs ? u : (int)S.queue[qh + i];
+        const OT beg = S.beg(x), len = S.end(x) - beg;
+        const int32_t* a = adj + e0 + beg;
+        for (OT row = (OT)part * 32; row < len; row += P * kNoiUnroll * 32) {
+          int y[kNoiUnroll];
+          R c[kNoiUnroll];
+#pragma unroll
+          for (int q = 0; q < kNoiUnroll; ++q) {
+            const OT e = row + q * P * 32 + lane;
+            y[q] = -1;
+            c[q] = 0;
+            if (e < len) {
+              y[q] = __ldg(a + e) - lo;
+              const long long x64 = ldw(w, e0 + beg + e);
+              c[q] = (sizeof(R) == 4 && x64 > (long long)lam) ? lam : (R)x64;
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < kNoiUnroll; ++q) {
+            if (row + q * P * 32 >= len) break;  // the same in every lane
+            bool join = false;
+            if (y[q] >= 0) {
+              const R old = noi_add(&S.r[y[q]], c[q]), now = old + c[q];
+              join = old < 0 && now >= 0;  // the addition that crosses lam takes the vertex
+              if constexpr (ST::kBounds)
+                if (now < 0) atomicMax(&S.cmax[y[q] >> 5], (U)now);
+            }
+            const unsigned b = __ballot_sync(0xffffffffu, join);
+            if (b) {
+              int at = 0;
+              if (lane == 0) at = atomicAdd(got, __popc(b));
+              if (join) atomicMin(&sh.runmin[run], y[q]);
+              at = qt + __shfl_sync(0xffffffffu, at, 0) + __popc(b & below);
+              if (join) S.queue[at] = (QT)y[q];
+            }
+          }
+        }
+      }
+      __syncthreads();
+      qh = qt;
+      qt += *(volatile int*)got;
+    }
+    if (qt - rs == 1) {
+      if (tid == 0) put(u, u);
+    } else {
+      const int m = min(u, *(volatile int*)&sh.runmin[run]);
+      for (int i = rs + tid; i < qt; i += NW * 32) put((int)S.queue[i], m);
+      unites = true;
+    }
+    run ^= 1;
+  }
+  __syncthreads();
+  return unites;
+}
+
 // Where one graph's exact-step results go: its bound, best-side kind, shape and
 // trace (fields of DevState for single runs, per-graph arrays for batches).
 struct NoiIO {
@@ -76,13 +337,18 @@ struct NoiIO {
   int level;
 };
 
-// All rounds on one graph of n <= kDenseMax vertices, by one block, on a dense matrix.
+// All rounds on one graph of n <= kDenseMax vertices, by one block.  The first round runs
+// on the lists (a closure level touches its vertices' entries, not whole matrix rows), and
+// the matrix that the later rounds work on is built from the lists for the contracted
+// graph alone, which is several times smaller; it sits in the block's dynamic shared
+// memory (scap entries at dyn) when it fits there, else in M0 / M1.
 // The graph's vertices are [base, base + n) of the CSR (off points at its first row).
 template <typename WT>
 __device__ __forceinline__ void noi_dense_body(int n, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                                               const WT* __restrict__ w, int32_t base, long long* M0, long long* M1,
-                                               int32_t* curK, unsigned char* sideK, const NoiIO& io) {
-  __shared__ long long r[kDenseMax];
+                                               const WT* __restrict__ w, int32_t base, long long* dyn, int scap,
+                                               long long* M0, long long* M1, int32_t* curK, unsigned char* sideK,
+                                               const NoiIO& io) {
+  __shared__ __align__(16) long long r[kDenseMax];
   __shared__ int seen[kDenseMax];
   __shared__ int parent[kDenseMax];
   __shared__ int root[kDenseMax];
@@ -91,20 +357,30 @@ __device__ __forceinline__ void noi_dense_body(int n, const int64_t* __restrict_
   __shared__ long long red_d[kNoiThreads / 32];
   __shared__ int red_v[kNoiThreads / 32];
   __shared__ long long red_c[kNoiThreads / 32];
-  __shared__ int s_x, s_stop, s_improved, s_nk2, s_arg, s_qt;
+  __shared__ int s_stop, s_improved, s_nk2, s_arg, s_qt;
+  __shared__ int64_t s_off[kDenseMax + 1];
+  __shared__ uint16_t s_queue[kDenseMax];
+  __shared__ NoiShared s_noi;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   constexpr int T = kNoiThreads;
   int nk = n;
-  long long* M = M0;
-  long long* Mn = M1;
-  for (int i = tid; i < nk * nk; i += T) M[i] = 0;
+  long long* M = nullptr;   // the current matrix (null: the first round, on the lists)
+  long long* Mn = nullptr;  // where the next one goes
   for (int k = tid; k < n; k += T) curK[k] = k;
-  __syncthreads();
-  for (int v = tid; v < nk; v += T)
-    for (int64_t e = off[v]; e < off[v + 1]; ++e) M[v * nk + (adj[e] - base)] += (long long)w[e];
   __syncthreads();
   while (nk > 1) {
     const long long lam = *io.lam;
+    if (!M) {
+      const int64_t e0 = off[0];
+      auto put = [&](int x, int m) { root[x] = m; };
+      if (noi_fits32(lam, off[n] - e0)) {
+        const ClosureSmem<int, int64_t, true> S{(int*)r, s_off, s_queue, off, e0};
+        noi_closure_block<kNoiThreads / 32>(base, nk, adj, w, lam, S, s_noi, put);
+      } else {
+        const ClosureSmem<long long, int64_t, true> S{r, s_off, s_queue, off, e0};
+        noi_closure_block<kNoiThreads / 32>(base, nk, adj, w, lam, S, s_noi, put);
+      }
+    } else {
     for (int k = tid; k < nk; k += T) { r[k] = 0; seen[k] = 0; parent[k] = k; }
     __syncthreads();
     if (nk <= kNoiWarpMax) {
@@ -131,7 +407,7 @@ __device__ __forceinline__ void noi_dense_body(int n, const int64_t* __restrict_
       }
       __syncthreads();
     } else {
-      // the round as closures (see noi_closure_warp below): each run's first vertex is the
+      // the round as closures (see noi_closure_block above): each run's first vertex is the
       // untaken vertex of largest r (ties: smallest id); the run then grows level by
       // level, every thread relaxing matrix entries of the level's vertices, and takes
       // its smallest id as the label of all its vertices (rr holds the taken vertices)
@@ -183,6 +459,7 @@ __device__ __forceinline__ void noi_dense_body(int n, const int64_t* __restrict_
       for (int k = tid; k < nk; k += T) root[k] = sfind(parent, k);
       __syncthreads();
     }
+    }
     // roots -> ranks (every root is the minimum of its component)
     {
       int flag = (tid < nk && root[tid] == tid) ? 1 : 0;  // nk <= T
@@ -205,18 +482,35 @@ __device__ __forceinline__ void noi_dense_body(int n, const int64_t* __restrict_
     }
     const int nk2 = s_nk2;
     if (nk2 == nk) break;  // no contraction (cannot happen while lambda-hat <= min degree)
+    // the next matrix: beside the current one, or over the one before it (which was larger)
+    long long* prev = M;
+    if (!M) Mn = nk2 * nk2 <= scap ? dyn : M0;
+    else if (!Mn) Mn = nk2 * nk2 + (M == dyn ? nk * nk : 0) <= scap ? dyn + (M == dyn ? nk * nk : 0) : M1;
     for (int i = tid; i < nk2 * nk2; i += T) Mn[i] = 0;
+    for (int k = tid; k < nk; k += T) parent[k] = rr[root[k]];  // every vertex's new id
     __syncthreads();
-    for (int i = tid; i < nk * nk; i += T) {
-      long long c = M[i];
-      if (c != 0) {
-        int a = rr[root[i / nk]], b = rr[root[i % nk]];
-        if (a != b) atomicAdd((unsigned long long*)&Mn[a * nk2 + b], (unsigned long long)c);
+    if (!M) {
+      // a warp per list
+      for (int v = wid; v < nk; v += T / 32) {
+        const int a = parent[v];
+        for (int64_t e = off[v] + lane; e < off[v + 1]; e += 32) {
+          const int b = parent[adj[e] - base];
+          if (a != b) atomicAdd((unsigned long long*)&Mn[a * nk2 + b], (unsigned long long)w[e]);
+        }
+      }
+    } else {
+      for (int i = tid; i < nk * nk; i += T) {
+        const long long c = M[i];
+        if (c != 0) {
+          const int a = parent[i / nk], b = parent[i % nk];
+          if (a != b) atomicAdd((unsigned long long*)&Mn[a * nk2 + b], (unsigned long long)c);
+        }
       }
     }
-    for (int k = tid; k < n; k += T) curK[k] = rr[root[curK[k]]];
+    for (int k = tid; k < n; k += T) curK[k] = parent[curK[k]];
     __syncthreads();
-    { long long* t = M; M = Mn; Mn = t; }
+    M = Mn;
+    Mn = prev;
     nk = nk2;
     // degrees, minimum with smallest argmin, and entry count of the contracted graph
     long long bd = LLONG_MAX, cnt = 0;
@@ -280,39 +574,38 @@ __global__ void __launch_bounds__(kNoiThreads) noi_dense_k(int n, const int64_t*
                                                            const int32_t* __restrict__ adj, const WT* __restrict__ w,
                                                            long long* M0, long long* M1, int32_t* curK,
                                                            unsigned char* sideK, DevState* st, TraceStep* trace,
-                                                           int trace_cap, int level, int in_smem) {
-  // small kernels keep the first round's matrix in shared memory (a round reads one
-  // matrix row per scan step; shared memory answers in a few cycles); later rounds
-  // are smaller and alternate between it and the global one
+                                                           int trace_cap, int level, int scap) {
   extern __shared__ __align__(16) long long noi_dyn[];
-  if (in_smem) M0 = noi_dyn;
   NoiIO io{&st->lambda_hat, &st->best_kind, &st->n, &st->nnz, &st->dmin, &st->argmin, &st->trace_len,
            trace, trace_cap, level};
-  noi_dense_body<WT>(n, off, adj, w, 0, M0, M1, curK, sideK, io);
+  noi_dense_body<WT>(n, off, adj, w, 0, noi_dyn, scap, M0, M1, curK, sideK, io);
 }
 
-constexpr int kNoiSmemMaxN = 160;  // 160^2 x 8 B = 200 KiB of shared memory
+// Matrix entries in dynamic shared memory: a contracted graph of at most 150 vertices
+// (beside the body's own arrays, below the 227 KB of a block).
+constexpr int kNoiDenseSmem = 150 * 150;
+
+// Opts a kernel into its dynamic shared memory, once per kernel and device.
+template <typename F>
+static void noi_set_smem(F kfn, size_t bytes) {
+  static std::mutex mu;
+  static std::map<std::pair<const void*, int>, bool> ready;
+  int dev = 0;
+  VC_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  bool& done = ready[{(const void*)kfn, dev}];
+  if (!done) VC_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  done = true;
+}
 
 template <typename WT>
 static void noi_dense_launch(const GraphView& g, long long* M0, long long* M1, int32_t* curK, unsigned char* sideK,
                              DevState* st, TraceStep* trace, int trace_cap, int level, cudaStream_t s) {
-  static std::mutex mu;
-  static std::unordered_map<int, bool> ready;  // per device: the shared-memory limit was raised
   const int n = (int)g.n;
-  const bool small = n <= kNoiSmemMaxN;
-  const size_t smem = small ? sizeof(long long) * (size_t)n * n : 0;
-  if (small) {
-    int dev = 0;
-    VC_CUDA(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lk(mu);
-    if (!ready[dev]) {
-      VC_CUDA(cudaFuncSetAttribute(noi_dense_k<WT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(sizeof(long long) * kNoiSmemMaxN * kNoiSmemMaxN)));
-      ready[dev] = true;
-    }
-  }
-  noi_dense_k<WT><<<1, kNoiThreads, smem, s>>>(n, g.off, g.adj, (const WT*)g.w, M0, M1, curK, sideK, st, trace,
-                                               trace_cap, level, small ? 1 : 0);
+  const int scap = std::min(n * n, kNoiDenseSmem);
+  noi_set_smem(noi_dense_k<WT>, sizeof(long long) * kNoiDenseSmem);
+  noi_dense_k<WT><<<1, kNoiThreads, sizeof(long long) * scap, s>>>(n, g.off, g.adj, (const WT*)g.w, M0, M1, curK,
+                                                                   sideK, st, trace, trace_cap, level, scap);
   count_launch();
   VC_CHECK_LAUNCH();
 }
@@ -324,14 +617,18 @@ void noi_dense(const GraphView& g, long long* M0, long long* M1, int32_t* curK, 
 }
 
 // Batches: a persistent grid pulls the listed graphs; each block solves one at a time
-// with its own matrices (mcap entries each).
+// with its own matrices (mcap entries each; those of at most 60 vertices in the 28 KB of
+// shared memory that four blocks per SM would leave each).
+constexpr int kNoiDenseBatchSmem = 60 * 60;
 template <typename WT>
 __global__ void __launch_bounds__(kNoiThreads) noi_dense_batch_k(const int32_t* __restrict__ list, int count,
                                                                  const int64_t* __restrict__ off,
                                                                  const int32_t* __restrict__ adj,
                                                                  const WT* __restrict__ w, const long long* vbase,
                                                                  const long long* nv, long long* M, int64_t mcap,
-                                                                 int32_t* curK, unsigned char* sideK, BatchNoi bn) {
+                                                                 int32_t* curK, unsigned char* sideK, BatchNoi bn,
+                                                                 int scap) {
+  extern __shared__ __align__(16) long long noi_dyn[];
   long long* M0 = M + (int64_t)blockIdx.x * 2 * mcap;
   long long* M1 = M0 + mcap;
   int32_t* ck = curK + (int64_t)blockIdx.x * kDenseMax;
@@ -340,7 +637,7 @@ __global__ void __launch_bounds__(kNoiThreads) noi_dense_batch_k(const int32_t* 
     const int32_t base = (int32_t)vbase[g];
     NoiIO io{bn.lam + g, bn.best_kind + g, bn.n_out + g, bn.nnz_out + g, bn.dmin + g, bn.argmin + g,
              bn.trace_len + g, bn.trace + (int64_t)g * bn.trace_cap, bn.trace_cap, bn.level[g]};
-    noi_dense_body<WT>((int)nv[g], off + base, adj, w, base, M0, M1, ck, sideK + (int64_t)g * kDenseMax, io);
+    noi_dense_body<WT>((int)nv[g], off + base, adj, w, base, noi_dyn, scap, M0, M1, ck, sideK + (int64_t)g * kDenseMax, io);
     __syncthreads();
   }
 }
@@ -349,12 +646,14 @@ void noi_dense_batch(const GraphView& u, const int32_t* list, int count, const l
                      long long* M, int64_t mcap, int blocks, int32_t* curK, unsigned char* sideK, const BatchNoi& bn,
                      cudaStream_t s) {
   if (count <= 0) return;
+  const size_t smem = sizeof(long long) * kNoiDenseBatchSmem;
   if (u.wbytes == 4)
-    noi_dense_batch_k<int32_t><<<blocks, kNoiThreads, 0, s>>>(list, count, u.off, u.adj, (const int32_t*)u.w, vbase,
-                                                               nv, M, mcap, curK, sideK, bn);
+    noi_dense_batch_k<int32_t><<<blocks, kNoiThreads, smem, s>>>(list, count, u.off, u.adj, (const int32_t*)u.w, vbase,
+                                                                 nv, M, mcap, curK, sideK, bn, kNoiDenseBatchSmem);
   else
-    noi_dense_batch_k<long long><<<blocks, kNoiThreads, 0, s>>>(list, count, u.off, u.adj, (const long long*)u.w,
-                                                                 vbase, nv, M, mcap, curK, sideK, bn);
+    noi_dense_batch_k<long long><<<blocks, kNoiThreads, smem, s>>>(list, count, u.off, u.adj, (const long long*)u.w,
+                                                                   vbase, nv, M, mcap, curK, sideK, bn,
+                                                                   kNoiDenseBatchSmem);
   count_launch();
   VC_CHECK_LAUNCH();
 }
@@ -417,335 +716,98 @@ __device__ __forceinline__ void noi_round_body(int64_t lo, int64_t hi, const int
   __syncthreads();
 }
 
-// ---- the same round by one warp, as closures.  Call a vertex "low" when it is visited
-// with attachment r < max(lambda-hat, 1).  When a low vertex u is visited every
-// unvisited r is at most r(u), so no unvisited vertex has reached lambda-hat; the
-// vertices visited after u up to the next low vertex are then exactly the closure of
-// u: the smallest set R holding u such that every vertex outside R and outside the
-// earlier runs has fewer than lambda-hat of weight into the vertices visited so far.
-// Adding a vertex only raises the weights into the set, so the closure does not depend
-// on the order in which its vertices are added, and neither do the attachments of the
-// vertices left afterwards; the next low vertex (the largest r, ties to the smallest
-// id) is therefore the same as in the maximum-adjacency order.  The round unites every
-// x, y with r(y) >= lambda-hat once x's edge is added; each such pair lies within one
-// run, and every vertex of a run is joined to the vertex whose edge raised it to
-// lambda-hat (visited inside the run), so the round's components are the runs and the
-// union-find with smallest-id roots labels each run with its smallest id.
-//
-// So a round needs the exact order only to pick each run's first vertex (an argmax
-// over the vertices not yet taken); a run then grows level by level, the warp relaxing
-// up to 32 queued vertices at once: their lists are laid end to end over the lanes, a
-// vertex whose attachment reaches lambda-hat joins the queue, and the run's labels are
-// written when it stops growing.  queue (n entries from lo) holds the vertices in the
-// order they were taken.
+// ---- the same round as closures, a block per graph
+// Shared memory of a graph of at most ncap vertices: 32-bit values, list offsets and
+// queue, or 64-bit values and queue.  16,384 vertices take 160 KB of a block's 227.
+constexpr int kNoiSmemRoundMaxN = 16384;
+__host__ __device__ constexpr size_t noi_round_smem(int ncap) { return (size_t)((ncap + 3) & ~3) * 10 + 16; }
 
-// argmax over the warp of (val, -idx) for val >= 0 (val < 0: no candidate); returns
-// idx, or -1 if no lane has a candidate; *best = the value.
-__device__ __forceinline__ int warp_argmax_vi(long long val, int idx, long long* best) {
-  const unsigned long long u = (unsigned long long)(val + 1);  // 0 = none
-  const unsigned hi = (unsigned)(u >> 32), lo = (unsigned)u;
-  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-  const unsigned long long mu = ((unsigned long long)mh << 32) | ml;
-  const unsigned wi = __reduce_min_sync(0xffffffffu, (u == mu && u != 0) ? (unsigned)idx : 0xffffffffu);
-  *best = (long long)mu - 1;
-  return mu == 0 ? -1 : (int)wi;
-}
-
-// Taken flags of a round: an int per vertex at v - sb (global memory, where graphs of a
-// union sit side by side), or a bit per vertex of the graph [lo, lo + n) in words the
-// warp owns (shared memory).  claim(v) takes v and returns whether it was not taken
-// yet: a vertex joins a queue at most once, whatever the weights.
-struct WordSeen {
-  int* p;
-  int64_t sb;
-  __device__ __forceinline__ void clear(int64_t lo, int64_t n, int lane) const {
-    for (int64_t k = lane; k < n; k += 32) p[lo + k - sb] = 0;
-  }
-  __device__ __forceinline__ bool test(int64_t v) const { return ((volatile int*)p)[v - sb] != 0; }
-  __device__ __forceinline__ bool claim(int64_t v) const { return atomicExch(&p[v - sb], 1) == 0; }
-};
-struct BitSeen {
-  unsigned* bits;
-  int64_t lo;
-  __device__ __forceinline__ void clear(int64_t, int64_t n, int lane) const {
-    for (int64_t k = lane; k < ((n + 31) >> 5); k += 32) bits[k] = 0;
-  }
-  __device__ __forceinline__ bool test(int64_t v) const {
-    return (((volatile unsigned*)bits)[(v - lo) >> 5] >> ((v - lo) & 31)) & 1u;
-  }
-  __device__ __forceinline__ bool claim(int64_t v) const {
-    const unsigned bit = 1u << ((v - lo) & 31);
-    return (atomicOr(&bits[(v - lo) >> 5], bit) & bit) == 0u;
-  }
-};
-
-constexpr int kNoiUnroll = 4;  // list entries in flight per lane while relaxing
-
-// One round over the graph [lo, lo + n) (ids global: labels, queue and the lists use
-// them); r holds vertex v at v - sb, queue the n taken vertices from lo (at q - qb for
-// place q: qb = 0 for a queue over the whole id range, lo for the graph's own array).
-// Writes every vertex's label; returns, in every lane, whether some run holds two or
-// more vertices (the round unites).
-template <typename WT, typename SEEN>
-__device__ __forceinline__ bool noi_closure_warp(int64_t lo, int64_t n, const int64_t* __restrict__ off,
-                                                 const int32_t* __restrict__ adj, const WT* __restrict__ w,
-                                                 long long lam, long long* r, int64_t sb, SEEN seen,
-                                                 long long* cmax, int32_t* queue, int64_t qb, int32_t* labels) {
-  const int lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
-  const int64_t nc = (n + 31) >> 5;
-  for (int64_t k = lane; k < n; k += 32) r[lo + k - sb] = 0;
-  for (int64_t c = lane; c < nc; c += 32) cmax[c] = 0;
-  seen.clear(lo, n, lane);
-  __syncwarp();
-  int32_t* q = queue + (lo - qb);  // q[i]: the i-th taken vertex
-  int64_t qt = 0, qh = 0;          // taken / relaxed so far (the same in every lane)
-  bool unites = false;
-  while (qt < n) {
-    // the run's first vertex: the untaken vertex of largest r, ties to the smallest id.
-    // cmax[c] bounds the attachments of chunk c's untaken vertices from above (raised
-    // with every relaxation; a taken vertex may leave it stale): the chunk of largest
-    // bound (ties: lower chunk) is checked exactly, and a stale bound is lowered and the
-    // choice made again.  A bound that holds is the largest attachment left.
-    int u;
-    for (;;) {
-      long long bv = -1;
-      int bc = -1;
-      for (int64_t c = lane; c < nc; c += 32) {
-        const long long m = cmax[c];
-        if (m > bv) { bv = m; bc = (int)c; }
-      }
-      long long bound, best;
-      const int C = warp_argmax_vi(bv, bc, &bound);
-      const int64_t k = (int64_t)C * 32 + lane;
-      const long long rv = (k < n && !seen.test(lo + k)) ? r[lo + k - sb] : -1;
-      const int xl = warp_argmax_vi(rv, (int)k, &best);
-      if (best == bound) {
-        u = xl;
-        break;
-      }
-      if (lane == 0) cmax[C] = best;  // -1: every vertex of the chunk is taken
-      __syncwarp();
-    }
-    const int64_t rs = qt;
-    int32_t runmin = (int32_t)(lo + u);
-    if (lane == 0) {
-      q[qt] = runmin;
-      seen.claim(lo + u);
-    }
-    ++qt;
-    __syncwarp();
-    while (qh < qt) {
-      // up to 32 taken vertices at once, their lists end to end over the lanes
-      const int cnt = (int)(qt - qh < 32 ? qt - qh : 32);
-      int64_t fb = 0, deg = 0;
-      if (lane < cnt) {
-        const int32_t x = q[qh + lane];
-        fb = __ldg(off + x);
-        deg = __ldg(off + x + 1) - fb;
-      }
-      qh += cnt;
-      int64_t incl = deg;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int64_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const int64_t total = __shfl_sync(0xffffffffu, incl, 31);
-      const int64_t excl = incl - deg;  // where lane j's list starts in the laid-out lists
-      for (int64_t p0 = 0; p0 < total; p0 += 32 * kNoiUnroll) {
-        int32_t y[kNoiUnroll];
-        long long c[kNoiUnroll];
-#pragma unroll
-        for (int i = 0; i < kNoiUnroll; ++i) {
-          const int64_t p = p0 + lane + 32 * i;
-          // the list holding place p: the last lane j whose list starts at or before p
-          int j = 0;
-#pragma unroll
-          for (int step = 16; step > 0; step >>= 1) {
-            const int t = j + step;
-            const int64_t ex = __shfl_sync(0xffffffffu, excl, t & 31);
-            if (t < cnt && ex <= p) j = t;
-          }
-          const int64_t e = __shfl_sync(0xffffffffu, fb, j) + (p - __shfl_sync(0xffffffffu, excl, j));
-          y[i] = -1;
-          c[i] = 0;
-          if (p < total) {
-            y[i] = __ldg(adj + e);
-            c[i] = (long long)__ldg(w + e);
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < kNoiUnroll; ++i) {
-          bool join = false;
-          if (y[i] >= 0 && !seen.test(y[i])) {
-            const long long ry =
-                (long long)atomicAdd((unsigned long long*)&r[y[i] - sb], (unsigned long long)c[i]) + c[i];
-            atomicMax(&cmax[(y[i] - lo) >> 5], ry);
-            // the addition that first leaves r(y) >= lambda-hat: the one that crosses it,
-            // or (lambda-hat <= 0) the first one
-            join = ry >= lam && (ry - c[i] < lam || ry - c[i] <= 0);
-          }
-          join = join && seen.claim(y[i]);
-          const unsigned b = __ballot_sync(0xffffffffu, join);
-          if (join) q[qt + __popc(b & below)] = y[i];
-          qt += __popc(b);
-          const unsigned m = __reduce_min_sync(0xffffffffu, join ? (unsigned)y[i] : 0xffffffffu);
-          if (m != 0xffffffffu && (int32_t)m < runmin) runmin = (int32_t)m;
-          __syncwarp();
-        }
-      }
-    }
-    for (int64_t i = rs + lane; i < qt; i += 32) labels[q[i]] = runmin;
-    if (qt - rs > 1) unites = true;
-    __syncwarp();
-  }
-  return unites;
-}
-
-// The round with the graph's state (attachments, taken flags and queue) in shared
-// memory.  One warp per block.
-constexpr int kNoiSmemRoundMaxN = 16384;  // 16384 x 12.375 B < 227 KB
-__host__ __device__ constexpr size_t noi_round_smem(int ncap) {
-  return (size_t)ncap * 12 + ((size_t)ncap / 32 + 1) * 12 + 16;
-}
-
-template <typename WT>
-__global__ void __launch_bounds__(32) noi_round_smem_k(int64_t n, const int64_t* __restrict__ off,
-                                                       const int32_t* __restrict__ adj, const WT* __restrict__ w,
-                                                       const DevState* st, int32_t* labels, int* changed) {
+// The listed graphs (list null: the one graph of n1 vertices with bound st->lambda_hat),
+// a block at a time each.  Graphs of at most ncap vertices keep their state in shared
+// memory; the others in r (values at the vertex), cmax (chunk bounds) and queue.
+template <typename WT, int NW>
+__global__ void __launch_bounds__(NW * 32) noi_round_k(
+    const int32_t* __restrict__ list, int count, int64_t n1, const DevState* st, const long long* __restrict__ vbase,
+    const long long* __restrict__ nv, const long long* __restrict__ glam, const int64_t* __restrict__ off,
+    const int32_t* __restrict__ adj, const WT* __restrict__ w, long long* r, unsigned long long* cmax,
+    int32_t* queue, int32_t* __restrict__ labels, int* changed, int ncap) {
   extern __shared__ __align__(16) unsigned char noi_rs[];
-  long long* r = (long long*)noi_rs;
-  long long* cmax = r + n;
-  int32_t* queue = (int32_t*)(cmax + n / 32 + 1);
-  unsigned* seen = (unsigned*)(queue + n);
-  const bool any =
-      noi_closure_warp<WT>(0, n, off, adj, w, st->lambda_hat, r, 0, BitSeen{seen, 0}, cmax, queue, 0, labels);
-  if (any && threadIdx.x == 0) atomicOr(changed, 1);
-}
-
-// Above the shared-memory size: the same round on global arrays.
-template <typename WT>
-__global__ void __launch_bounds__(32) noi_round_k(int64_t n, const int64_t* __restrict__ off,
-                                                  const int32_t* __restrict__ adj, const WT* __restrict__ w,
-                                                  const DevState* st, long long* r, int* seen,
-                                                  int32_t* queue, int32_t* labels, int* changed) {
-  // r holds n attachments, then the chunk bounds
-  const bool any =
-      noi_closure_warp<WT>(0, n, off, adj, w, st->lambda_hat, r, 0, WordSeen{seen, 0}, r + n, queue, 0, labels);
-  if (any && threadIdx.x == 0) atomicOr(changed, 1);
-}
-
-template <typename WT>
-static void noi_round_launch(const GraphView& g, const DevState* st, long long* r, int* seen,
-                             int32_t* queue, int32_t* labels, int* changed, cudaStream_t s) {
-  if (g.n <= kNoiSmemRoundMaxN) {
-    static std::mutex mu;
-    static std::unordered_map<int, bool> ready;  // per device: the shared-memory limit was raised
-    {
-      int dev = 0;
-      VC_CUDA(cudaGetDevice(&dev));
-      std::lock_guard<std::mutex> lk(mu);
-      if (!ready[dev]) {
-        VC_CUDA(cudaFuncSetAttribute(noi_round_smem_k<WT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)noi_round_smem(kNoiSmemRoundMaxN)));
-        ready[dev] = true;
-      }
-    }
-    noi_round_smem_k<WT><<<1, 32, noi_round_smem((int)g.n), s>>>(g.n, g.off, g.adj, (const WT*)g.w, st, labels,
-                                                                 changed);
-  } else {
-    noi_round_k<WT><<<1, 32, 0, s>>>(g.n, g.off, g.adj, (const WT*)g.w, st, r, seen, queue, labels, changed);
-  }
-  count_launch();
-  VC_CHECK_LAUNCH();
-}
-
-void noi_round_sparse(const GraphView& g, const DevState* st, long long* r, int* seen,
-                      int32_t* parent, int32_t* labels, int* changed, cudaStream_t s) {
-  // parent (n entries) holds the queue of taken vertices
-  if (g.wbytes == 4)
-    noi_round_launch<int32_t>(g, st, r, seen, parent, labels, changed, s);
-  else
-    noi_round_launch<long long>(g, st, r, seen, parent, labels, changed, s);
-}
-
-// Batches: the round of each listed graph by a warp (persistent grid of 8-warp blocks
-// pulling graphs from the list).  With ncap > 0 (every listed graph of at most ncap
-// vertices) each warp keeps its graph's taken bits in shared memory; the attachments
-// and queues stay in global memory (every graph of the list in flight at once).
-__host__ __device__ constexpr size_t noi_batch_warp_smem(int ncap) { return (size_t)(ncap / 32 + 1) * 12; }
-constexpr size_t kNoiBatchSmemMax = 160 * 1024;
-
-template <typename WT>
-__global__ void __launch_bounds__(256) noi_round_batch_k(const int32_t* __restrict__ list, int count,
-                                                         const int64_t* __restrict__ off,
-                                                         const int32_t* __restrict__ adj, const WT* __restrict__ w,
-                                                         const long long* vbase, const long long* nv,
-                                                         const long long* glam, long long* r, int* seen,
-                                                         long long* cmax, int32_t* queue, int32_t* labels,
-                                                         int* gchanged, int ncap) {
-  extern __shared__ __align__(16) unsigned char noi_bs[];
-  const int warps = gridDim.x * (blockDim.x >> 5);
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int words = ncap / 32 + 1;
-  long long* wc = (long long*)noi_bs + (size_t)wid * words;
-  unsigned* wb = (unsigned*)((long long*)noi_bs + (size_t)(blockDim.x >> 5) * words) + (size_t)wid * words;
-  for (int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; idx < count; idx += warps) {
-    const int g = list[idx];
-    const long long lo = vbase[g], n = nv[g];
+  __shared__ NoiShared sh;
+  for (int idx = blockIdx.x; idx < count; idx += gridDim.x) {
+    const int g = list ? list[idx] : 0;
+    const int64_t lo = list ? vbase[g] : 0;
+    const int n = (int)(list ? nv[g] : n1);
+    const long long lam = list ? glam[g] : st->lambda_hat;
+    const int64_t* goff = off + lo;
+    const int64_t e0 = goff[0];
+    auto put = [&](int x, int m) { labels[lo + x] = (int32_t)(lo + m); };
     bool any;
-    if (ncap > 0 && n <= ncap)
-      any = noi_closure_warp<WT>(lo, n, off, adj, w, glam[g], r, 0, BitSeen{wb, lo}, wc, queue, 0, labels);
-    else
-      any = noi_closure_warp<WT>(lo, n, off, adj, w, glam[g], r, 0, WordSeen{seen, 0}, cmax + lo, queue, 0, labels);
-    if (any && lane == 0) atomicOr(gchanged + g, 1);
-    __syncwarp();
+    if (n > ncap) {
+      const ClosureGlobal S{r + lo, cmax + lo, queue + lo, goff, e0};
+      any = noi_closure_block<NW>((int32_t)lo, n, adj, w, lam, S, sh, put);
+    } else if (noi_fits32(lam, goff[n] - e0)) {
+      ClosureSmem<int, int32_t, true> S;
+      S.r = (int*)noi_rs;
+      S.soff = (int32_t*)(S.r + ((n + 3) & ~3));
+      S.queue = (uint16_t*)(S.soff + n + 1);
+      S.goff = goff;
+      S.e0 = e0;
+      any = noi_closure_block<NW>((int32_t)lo, n, adj, w, lam, S, sh, put);
+    } else {
+      ClosureSmem<long long, int64_t, false> S;
+      S.r = (long long*)noi_rs;
+      S.soff = nullptr;
+      S.queue = (uint16_t*)(S.r + ((n + 3) & ~3));
+      S.goff = goff;
+      S.e0 = e0;
+      any = noi_closure_block<NW>((int32_t)lo, n, adj, w, lam, S, sh, put);
+    }
+    if (any && threadIdx.x == 0) atomicOr(list ? changed + g : changed, 1);
   }
 }
 
-template <typename WT>
-static void noi_round_batch_launch(const GraphView& u, const int32_t* list, int count, const long long* vbase,
-                                   const long long* nv, const long long* glam, long long* r, int* seen,
-                                   long long* cmax, int32_t* queue, int32_t* labels, int* gchanged, int max_n,
-                                   cudaStream_t s) {
-  static std::mutex mu;
-  static std::unordered_map<int, bool> ready;  // per device: the shared-memory limit was raised
-  {
-    int dev = 0;
-    VC_CUDA(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lk(mu);
-    if (!ready[dev]) {
-      VC_CUDA(cudaFuncSetAttribute(noi_round_batch_k<WT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)kNoiBatchSmemMax));
-      ready[dev] = true;
-    }
-  }
-  const size_t smem = 8 * noi_batch_warp_smem(max_n);
-  const bool in_smem = max_n > 0 && smem <= kNoiBatchSmemMax;
-  const int blocks = grid_for(count, 8, kSMs * 4);
-  noi_round_batch_k<WT><<<blocks, 256, in_smem ? smem : 0, s>>>(list, count, u.off, u.adj, (const WT*)u.w, vbase, nv,
-                                                               glam, r, seen, cmax, queue, labels, gchanged,
-                                                               in_smem ? max_n : 0);
+template <int NW, typename WT>
+static void noi_round_launch(const GraphView& u, const int32_t* list, int count, const DevState* st,
+                             const long long* vbase, const long long* nv, const long long* glam, long long* r,
+                             int32_t* queue, int32_t* labels, int* changed, int ncap, cudaStream_t s) {
+  noi_set_smem(noi_round_k<WT, NW>, noi_round_smem(kNoiSmemRoundMaxN));
+  noi_round_k<WT, NW><<<std::min(count, kSMs * 8), NW * 32, noi_round_smem(ncap), s>>>(
+      list, count, u.n, st, vbase, nv, glam, u.off, u.adj, (const WT*)u.w, r, (unsigned long long*)r + u.n, queue,
+      labels, changed, ncap);
   count_launch();
   VC_CHECK_LAUNCH();
+}
+
+template <int NW>
+static void noi_round_by_weight(const GraphView& u, const int32_t* list, int count, const DevState* st,
+                                const long long* vbase, const long long* nv, const long long* glam, long long* r,
+                                int32_t* queue, int32_t* labels, int* changed, int ncap, cudaStream_t s) {
+  if (u.unit)
+    noi_round_launch<NW, UnitW>(u, list, count, st, vbase, nv, glam, r, queue, labels, changed, ncap, s);
+  else if (u.wbytes == 4)
+    noi_round_launch<NW, int32_t>(u, list, count, st, vbase, nv, glam, r, queue, labels, changed, ncap, s);
+  else
+    noi_round_launch<NW, long long>(u, list, count, st, vbase, nv, glam, r, queue, labels, changed, ncap, s);
+}
+
+void noi_round_sparse(const GraphView& g, const DevState* st, long long* r, int32_t* parent, int32_t* labels,
+                      int* changed, cudaStream_t s) {
+  // parent (n entries) holds the queue of taken vertices
+  const int ncap = (int)std::min<int64_t>(g.n, kNoiSmemRoundMaxN);
+  noi_round_by_weight<16>(g, nullptr, 1, st, nullptr, nullptr, nullptr, r, parent, labels, changed, ncap, s);
 }
 
 void noi_round_batch(const GraphView& u, const int32_t* list, int count, const long long* vbase, const long long* nv,
-                     const long long* glam, long long* r, int* seen, int32_t* parent, int32_t* labels,
-                     int* gchanged, int max_n, cudaStream_t s) {
+                     const long long* glam, long long* r, int32_t* parent, int32_t* labels, int* gchanged, int cls,
+                     cudaStream_t s) {
   if (count <= 0) return;
-  // r holds noi_round_scratch(union size) entries: the attachments, then each graph's
-  // chunk bounds at its own range; seen: the taken flags (union size); parent (union
-  // size) holds the queues
-  long long* cmax = r + u.n;
-  if (u.wbytes == 4)
-    noi_round_batch_launch<int32_t>(u, list, count, vbase, nv, glam, r, seen, cmax, parent, labels, gchanged, max_n,
-                                    s);
+  // r holds noi_round_scratch(union size) entries: the values, then each graph's chunk
+  // bounds at its own range; parent (union size) holds the queues
+  const int ncap = std::min(noi_class_max(cls), kNoiSmemRoundMaxN);
+  if (cls == kNoiClasses - 1)
+    noi_round_by_weight<16>(u, list, count, nullptr, vbase, nv, glam, r, parent, labels, gchanged, ncap, s);
   else
-    noi_round_batch_launch<long long>(u, list, count, vbase, nv, glam, r, seen, cmax, parent, labels, gchanged, max_n,
-                                      s);
+    noi_round_by_weight<8>(u, list, count, nullptr, vbase, nv, glam, r, parent, labels, gchanged, ncap, s);
 }
 
 // ------------------------------------------------------- allocation-free round
