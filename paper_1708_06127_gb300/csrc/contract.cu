@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long lon
     const long long b = cbase[x];
     const int T = (int)(cbase[x + 1] - b);
     if (T > kMergeMax) continue;  // the block kernel takes it
-    RegList<S> L;
+    RegList<long long, S> L;
     L.slots = (T + 31) >> 5;
     L.todo = 0;
 #pragma unroll

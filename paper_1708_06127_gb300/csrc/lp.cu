@@ -414,9 +414,8 @@ __global__ void __launch_bounds__(kAggThreads) lp_warp_k(
 }
 
 // ------------------------------------------------------------ register class
-// Lists of at most kWarpMaxDeg = 128 entries.  A group of G lanes (G = 16 for lists
-// of at most 64 entries, two vertices per warp; G = 32 for 65..128) holds the whole
-// list in registers (slot r of group lane i holds entry G r + i) and visits its
+// Lists of at most kWarpMaxDeg = 128 entries (and, in other launches, of at most
+// kMidMaxDeg).  A group of G lanes (see RegShape) holds the whole list in registers (slot r of group lane i holds entry G r + i) and visits its
 // distinct keys one at a time, slot by slot: the first lane whose slot r is still
 // unvisited broadcasts its key, every lane marks its entries holding it (only slots
 // >= r can), and a group reduction gives the key's count (unit weights) or weight
@@ -433,52 +432,68 @@ constexpr int kEmitWalkKeys = 6;
 constexpr int kEmitBlockPerVertexMax = kSMs * 8;  // block-class lists pre-merged a block each
 constexpr int kLpBailKeys = 16;
 constexpr int kLpWalkKeys = 8;      // short classes: labels walked before the table
-constexpr int kLpTableMaxS = 4;     // classes of at most this many slots per lane
-constexpr int kLpTableSlots = 256;  // table slots per warp (split between its groups)
+constexpr int kLpTableMaxS = 8;     // classes of at most this many slots per lane
+constexpr int kLpTableSlots = 512;  // table slots per warp (split between its groups)
 // The table serves weighted graphs only: on unit weights its registers and shared
 // memory cost an SM block of the kernel, and lists with many labels are rare there.
 template <typename WT, int S>
 constexpr bool lp_has_table() { return S <= kLpTableMaxS && !std::is_same<WT, UnitW>::value; }
 
-// Neighbour ids (and weights) of one list in registers.
-template <int S>
+// Lanes per vertex for lists of at most 64 and 128 entries.  Weights of at most 32 bits:
+// eight slots per lane, so four (two) vertices per warp; a step costs a few instructions per
+// slot but serves every group of the warp, and the warp steps as often as its group with the
+// most keys, which grows slowly with the number of groups.  Unit weights, RHG n = 2^22,
+// average degree 64, by vertices per warp of the shorter class: two (four slots): label
+// propagation's later round 416 + 332 us, pre-merge 475 + 452; four: 304 + 263 and
+// 355 + 366; eight (sixteen slots): 353 + 266 and 350 + 354.  32-bit weights, RHG
+// n = 250,000, average degree 32: 243 and 183 us with four slots, 170 and 157 with eight.
+// 64-bit weights keep four slots (eight of them per lane would cost blocks per SM).
+template <typename WT>
+struct RegShape {
+  static constexpr int S = std::is_same<WT, long long>::value ? 4 : 8, G64 = 64 / S, G128 = 128 / S;
+};
+
+// Neighbour ids (and weights, as they are stored) of one list in registers.  The loads have
+// no branches: a slot past the list's end reads its last entry again (left out by `todo`),
+// and an empty list reads `safe`, an array of vertex ids.
+template <typename WT, int S>
 struct RegIds {
   int32_t u[S];
-  long long wt[S];
+  typename RegWeight<WT>::type wt[S];
 };
 
 template <typename WT, int G, int S>
-__device__ __forceinline__ void reg_ids(RegIds<S>& R, int64_t beg, int64_t end, int glane,
-                                        const int32_t* __restrict__ adj, const WT* __restrict__ w) {
+__device__ __forceinline__ void reg_ids(RegIds<WT, S>& R, int64_t beg, int64_t end, int glane,
+                                        const int32_t* __restrict__ adj, const WT* __restrict__ w,
+                                        const int32_t* __restrict__ safe) {
   const int64_t dd = end - beg;
-  const int d = dd > S * G ? 0 : (int)dd;
-  const int32_t* a = adj + beg;
+  const int last = (dd > S * G ? 0 : (int)dd) - 1;
+  const int32_t* a = last >= 0 ? adj + beg : safe;
 #pragma unroll
   for (int r = 0; r < S; ++r) {
-    const int i = glane + G * r;
-    R.u[r] = -1;
-    R.wt[r] = 0;
-    if (i < d) {
-      R.u[r] = __ldcs(a + i);  // read once: evict first, keeping the gathered labels in L2
-      R.wt[r] = ldw(w, beg + i);
-    }
+    const int i = max(min(glane + G * r, last), 0);
+    R.u[r] = __ldcs(a + i);  // read once: evict first, keeping the gathered labels in L2
+    if constexpr (!std::is_same<WT, UnitW>::value) R.wt[r] = last >= 0 ? __ldg(w + beg + i) : 0;
   }
 }
 
-template <int MODE, bool FIRST, int G, int S>
-__device__ __forceinline__ void reg_keys(RegList<S>& L, const RegIds<S>& R, int deg, const int32_t* __restrict__ lab,
-                                         int32_t own) {
+// Keys of the entries and, in L.todo, the slots that hold one to visit.
+template <int MODE, bool FIRST, int G, int S, typename WT>
+__device__ __forceinline__ void reg_keys(RegList<WT, S>& L, const RegIds<WT, S>& R, int deg, int glane,
+                                         const int32_t* __restrict__ lab, int32_t own) {
   L.slots = (deg + G - 1) / G;
-  L.todo = 0;
+  L.todo = (1u << ((deg - glane + G - 1) / G)) - 1u;  // this lane's entries: deg <= S G < 32 G
 #pragma unroll
   for (int r = 0; r < S; ++r) {
-    L.k[r] = -1;
-    L.wt[r] = R.wt[r];
-    if (R.u[r] >= 0) {
-      int32_t kk;
-      if (entry_key<MODE, FIRST>(lab, R.u[r], own, &kk)) L.todo |= 1u << r;
-      L.k[r] = kk;
-    }
+    if constexpr (!std::is_same<WT, UnitW>::value) L.wt[r] = R.wt[r];
+    L.k[r] = FIRST ? R.u[r] : __ldg(lab + R.u[r]);
+  }
+  if (MODE == kModeEmit) {
+    unsigned intra = 0;
+#pragma unroll
+    for (int r = 0; r < S; ++r)
+      if (L.k[r] == own) intra |= 1u << r;
+    L.todo &= ~intra;
   }
 }
 
@@ -508,17 +523,17 @@ __device__ __forceinline__ void reg_pipeline(const int32_t* __restrict__ list, i
   int64_t v, beg, end, vn, nbeg, nend;
   int32_t x, xn;
   fetch(base, v, beg, end, x);
-  RegIds<S> cur;
-  reg_ids<WT, G, S>(cur, beg, end, glane, adj, w);
+  RegIds<WT, S> cur;
+  reg_ids<WT, G, S>(cur, beg, end, glane, adj, w, list);
   int64_t bn = base + stride;
   fetch(bn, vn, nbeg, nend, xn);
   for (;;) {
-    RegIds<S> nxt;
+    RegIds<WT, S> nxt;
     int64_t vnn = -1, nnbeg = 0, nnend = 0;
     int32_t xnn = 0;
     const int64_t bnn = bn + stride;
     if (bn < total) {
-      reg_ids<WT, G, S>(nxt, nbeg, nend, glane, adj, w);
+      reg_ids<WT, G, S>(nxt, nbeg, nend, glane, adj, w, list);
       fetch(bnn, vnn, nnbeg, nnend, xnn);
     }
     body(v, v >= 0, beg, end, x, cur);
@@ -562,15 +577,14 @@ __global__ void __launch_bounds__(kAggThreads) lp_reg_k(const int32_t* __restric
                         if (vact && !vact[v]) return INT_MIN;
                         return FIRST ? 0 : __ldg(lab + v);
                       },
-                      [&](int64_t v, bool valid, int64_t beg, int64_t end, int32_t own, const RegIds<S>& ids) {
+                      [&](int64_t v, bool valid, int64_t beg, int64_t end, int32_t own, const RegIds<WT, S>& ids) {
     const int64_t d = end - beg;
     const bool mine = valid && own != INT_MIN;
     if (mine && d == 0) {
       if (glane == 0) lab_out[v] = FIRST ? (int32_t)v : __ldg(lab + v);
     }
-    RegList<S> L;
-    reg_keys<kModeLP, FIRST, G, S>(L, ids, mine ? (int)d : 0, lab, 0);
-    if (!mine) L.todo = 0;
+    RegList<WT, S> L;
+    reg_keys<kModeLP, FIRST, G, S>(L, ids, mine ? (int)d : 0, glane, lab, 0);
     // running best (sum, hash, -label), the same in the group's lanes; the hash of
     // the best is read only once a tie needs it.  `left` is the weight of the keys not
     // visited yet: once the best exceeds it, no other key can reach the best, and the
@@ -582,7 +596,7 @@ __global__ void __launch_bounds__(kAggThreads) lp_reg_k(const int32_t* __restric
       long long sum = 0;
 #pragma unroll
       for (int r = 0; r < S; ++r)
-        if (L.todo >> r & 1u) sum += L.wt[r];
+        if (L.todo >> r & 1u) sum += (long long)L.wt[r];
 #pragma unroll
       for (int o = G / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       left = (ACC)sum;
@@ -598,7 +612,8 @@ __global__ void __launch_bounds__(kAggThreads) lp_reg_k(const int32_t* __restric
       unsigned hit = 0;
 #pragma unroll
       for (int r = 0; r < S; ++r)
-        if (((L.todo >> r) & 1u) && L.k[r] == own) hit |= 1u << r;
+        if (L.k[r] == own) hit |= 1u << r;
+      hit &= L.todo;
       ACC t;
       if (std::is_same<WT, UnitW>::value) {
         t = (ACC)__reduce_add_sync(gmask, (unsigned)__popc(hit));
@@ -606,7 +621,7 @@ __global__ void __launch_bounds__(kAggThreads) lp_reg_k(const int32_t* __restric
         long long sum = 0;
 #pragma unroll
         for (int r = 0; r < S; ++r)
-          if ((hit >> r) & 1u) sum += L.wt[r];
+          if ((hit >> r) & 1u) sum += (long long)L.wt[r];
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         t = (ACC)sum;
@@ -656,7 +671,7 @@ __global__ void __launch_bounds__(kAggThreads) lp_reg_k(const int32_t* __restric
       // adds its weight to its label's slot, then the group takes the best slot and
       // compares it with the walk's best; the slots are emptied for the next vertex
       constexpr int CAPG = kLpTableSlots / (32 / G);
-      constexpr int LG = CAPG >= 256 ? 8 : 7;
+      constexpr int LG = CAPG >= 512 ? 9 : CAPG >= 256 ? 8 : 7;
       static_assert((1 << LG) == CAPG && CAPG >= 2 * S * G, "table of twice the list capacity");
       int32_t* tk = tab_k + gi * CAPG;
       ACC* tv = tab_v + gi * CAPG;
@@ -720,12 +735,11 @@ __global__ void __launch_bounds__(kAggThreads) emit_reg_k(const int32_t* __restr
   const bool rows = out.by_rows();
   reg_pipeline<WT, G, S>(list, *count_ptr, first, stride, glane, gi, off, adj, w,
                       [&](int64_t v) { return __ldg(cid + v); },
-                      [&](int64_t v, bool valid, int64_t beg, int64_t end, int32_t own, const RegIds<S>& ids) {
+                      [&](int64_t v, bool valid, int64_t beg, int64_t end, int32_t own, const RegIds<WT, S>& ids) {
     const int64_t d = end - beg;
     const bool mine = valid;
-    RegList<S> L;
-    reg_keys<kModeEmit, false, G, S>(L, ids, (mine && own >= 0) ? (int)d : 0, cid, own);
-    if (!(mine && own >= 0)) L.todo = 0;
+    RegList<WT, S> L;
+    reg_keys<kModeEmit, false, G, S>(L, ids, (mine && own >= 0) ? (int)d : 0, glane, cid, own);
     int made = 0;  // the same in the group's lanes
     // one pass per row r (entries r G .. r G + G - 1) over the entries still to do:
     // lanes holding the same key (tagged with the group) match, the lowest of them sums
@@ -832,14 +846,17 @@ void launch_lp_reg(const GraphView& g, const Bins& b, const WT* w, const int32_t
                    const unsigned long long* hv, cudaStream_t s, bool mid_bail) {
   int32_t* bl = (FIRST || !mid_bail) ? nullptr : b.bail_list;
   int* bc = (FIRST || !mid_bail) ? nullptr : b.counts + 7;
+  using R = RegShape<WT>;
   if (b.h_small > 0) {
-    lp_reg_k<WT, ACC, FIRST, 16, 4><<<grid_for(b.h_small, kWarpsPerBlock * 2, kSMs * 16), kAggThreads, 0, s>>>(
+    lp_reg_k<WT, ACC, FIRST, R::G64, R::S>
+        <<<grid_for(b.h_small, kWarpsPerBlock * (32 / R::G64), kSMs * 16), kAggThreads, 0, s>>>(
         b.small_list, b.counts + 4, g.off, g.adj, w, lab, lab_out, hv, g.vact, nullptr, nullptr);
     count_launch();
     VC_CHECK_LAUNCH();
   }
   if (b.h_reg > 0) {
-    lp_reg_k<WT, ACC, FIRST, 32, 4><<<grid_for(b.h_reg, kWarpsPerBlock, kSMs * 16), kAggThreads, 0, s>>>(
+    lp_reg_k<WT, ACC, FIRST, R::G128, R::S>
+        <<<grid_for(b.h_reg, kWarpsPerBlock * (32 / R::G128), kSMs * 16), kAggThreads, 0, s>>>(
         b.reg_list, b.counts + 5, g.off, g.adj, w, lab, lab_out, hv, g.vact, nullptr, nullptr);
     count_launch();
     VC_CHECK_LAUNCH();
@@ -1252,14 +1269,17 @@ void launch_lp(const GraphView& g, const Bins& b, const GlobalTables& gt, const 
 template <typename WT>
 void launch_emit_reg(const GraphView& g, const Bins& b, const WT* w, const int32_t* cid, const PairOut& out,
                      int32_t* cnt, cudaStream_t s) {
+  using R = RegShape<WT>;
   if (b.h_small > 0) {
-    emit_reg_k<WT, 16, 4><<<grid_for(b.h_small, kWarpsPerBlock * 2, kSMs * 16), kAggThreads, 0, s>>>(
+    emit_reg_k<WT, R::G64, R::S>
+        <<<grid_for(b.h_small, kWarpsPerBlock * (32 / R::G64), kSMs * 16), kAggThreads, 0, s>>>(
         b.small_list, b.counts + 4, g.off, g.adj, w, cid, out, cnt, nullptr, nullptr);
     count_launch();
     VC_CHECK_LAUNCH();
   }
   if (b.h_reg > 0) {
-    emit_reg_k<WT, 32, 4><<<grid_for(b.h_reg, kWarpsPerBlock, kSMs * 16), kAggThreads, 0, s>>>(
+    emit_reg_k<WT, R::G128, R::S>
+        <<<grid_for(b.h_reg, kWarpsPerBlock * (32 / R::G128), kSMs * 16), kAggThreads, 0, s>>>(
         b.reg_list, b.counts + 5, g.off, g.adj, w, cid, out, cnt, nullptr, nullptr);
     count_launch();
     VC_CHECK_LAUNCH();

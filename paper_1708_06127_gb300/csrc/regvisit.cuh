@@ -17,10 +17,20 @@ __device__ __forceinline__ unsigned group_mask(int lane) {
   return G == 32 ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
 }
 
-template <int S>
+// A slot's weight as it is stored (unit weights: none).
+template <typename WT>
+struct RegWeight {
+  using type = WT;
+};
+template <>
+struct RegWeight<UnitW> {
+  using type = unsigned char;  // never read
+};
+
+template <typename WT, int S>
 struct RegList {
   int32_t k[S];
-  long long wt[S];
+  typename RegWeight<WT>::type wt[S];
   unsigned todo;  // bit r: slot r holds a used entry not yet visited
   int slots;      // slots in use: ceil(deg / G), the same in every lane of the group
 };
@@ -29,7 +39,7 @@ struct RegList {
 // vote per step, no empty pass per slot; a lane finds its lowest unvisited slot with
 // S - 1 selects); longer lists go slot by slot, where the selects would cost more
 // than the empty passes they save.
-constexpr int kVoteAllMaxS = 4;
+constexpr int kVoteAllMaxS = 8;
 
 // Calls visit(key, total) once per distinct used key of the group's list; total is
 // the same in the group's lanes.  The order of the visits is not a contract: callers
@@ -37,7 +47,7 @@ constexpr int kVoteAllMaxS = 4;
 // group's walk (its remaining keys are not visited).  Every lane of the warp must
 // call it (groups without a list pass slots = todo = 0).
 template <typename WT, typename ACC, int G, int S, typename F>
-__device__ __forceinline__ void reg_visit(RegList<S>& L, unsigned gmask, F visit) {
+__device__ __forceinline__ void reg_visit(RegList<WT, S>& L, unsigned gmask, F visit) {
   // one step: key kk (held by the group's first lane of the vote when gb != 0) is
   // marked visited in every slot >= r0 holding it, and visited with its total
   auto step = [&](unsigned gb, int32_t kk, int r0) {
@@ -54,7 +64,7 @@ __device__ __forceinline__ void reg_visit(RegList<S>& L, unsigned gmask, F visit
       long long sum = 0;
 #pragma unroll
       for (int q = 0; q < S; ++q)
-        if (hit >> q & 1u) sum += L.wt[q];
+        if (hit >> q & 1u) sum += (long long)L.wt[q];
 #pragma unroll
       for (int o = G / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       total = (ACC)sum;
