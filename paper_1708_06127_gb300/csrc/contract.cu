@@ -331,13 +331,17 @@ __global__ void __launch_bounds__(256) cluster_scatter_k(int64_t n, const int64_
 // sums its run (a step per target costs slots x compares, which only pays while
 // targets are few).  With sort_first (a contraction whose clusters are mostly one or
 // two vertices: nearly every pair its own target) a cluster of at least kMergeSortMin
-// pairs is sorted without walking first.
+// pairs is sorted without walking first.  With a list (list_n not null) only the listed
+// clusters are visited (a sparse contraction leaves nearly all of them without pairs:
+// 0.75 ms for 3.5 million empty clusters, 0.04 ms to list the others).
 constexpr int kMergeWarpKeys = 32;
 constexpr int kMergeSortMin = 12;
 
 __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long long* __restrict__ cbase,
                                                        int32_t* __restrict__ seg_key, long long* __restrict__ seg_val,
-                                                       int32_t* __restrict__ dcount, bool sort_first) {
+                                                       int32_t* __restrict__ dcount, bool sort_first,
+                                                       const int32_t* __restrict__ list,
+                                                       const int* __restrict__ list_n) {
   constexpr int S = kMergeMax / 32;
   __shared__ int32_t sk_all[8][kMergeMax];
   __shared__ long long sv_all[8][kMergeMax];
@@ -345,7 +349,9 @@ __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long lon
   int32_t* sk = sk_all[wid];
   long long* sv = sv_all[wid];
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < c; x += warps) {
+  if (list_n) c = *list_n;
+  for (int64_t xi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; xi < c; xi += warps) {
+    const int64_t x = list_n ? (int64_t)list[xi] : xi;
     const long long b = cbase[x];
     const int T = (int)(cbase[x + 1] - b);
     if (T > kMergeMax) continue;  // the block kernel takes it
@@ -1096,6 +1102,23 @@ __global__ void block_class_list_k(int64_t c, const long long* __restrict__ cbas
   }
 }
 
+// The clusters of 1 to kMergeMax pairs.
+__global__ void warp_class_list_k(int64_t c, const long long* __restrict__ cbase, int32_t* __restrict__ list,
+                                  int* __restrict__ count) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; b < c;
+       b += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t x = b + lane;
+    const long long T = x < c ? cbase[x + 1] - cbase[x] : 0;
+    const bool in = T > 0 && T <= kMergeMax;
+    const unsigned bal = __ballot_sync(0xffffffffu, in);
+    int at = 0;
+    if (lane == 0 && bal) at = atomicAdd(count, __popc(bal));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (in) list[at + __popc(bal & ((1u << lane) - 1u))] = (int32_t)x;
+  }
+}
+
 void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int32_t* ccount, int64_t c,
                    long long* cbase, long long* cursor, int32_t* seg_key, long long* seg_val, int64_t* coff,
                    int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, bool big, bool sort_first,
@@ -1105,7 +1128,13 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
   const int gv = grid_for(g.n, 256, kSMs * 8), gc = grid_for(c, 8, kSMs * 16);
   const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
   cluster_scatter_k<<<gv, 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, cursor, seg_key, seg_val);
-  cluster_merge_k<<<gc, 256, 0, s>>>(c, cbase, seg_key, seg_val, ccount, sort_first);
+  if (sp) {
+    VC_CUDA(cudaMemsetAsync(sp->list_n, 0, sizeof(int), s));
+    warp_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, sp->list, sp->list_n);
+    count_launch();
+  }
+  cluster_merge_k<<<gc, 256, 0, s>>>(c, cbase, seg_key, seg_val, ccount, sort_first, sp ? sp->list : nullptr,
+                                     sp ? sp->list_n : nullptr);
   count_launch(2);
   VC_CHECK_LAUNCH();
   if (big) {

@@ -34,6 +34,10 @@ struct Buf {
     p = nullptr;
     cap = 0;
   }
+  void swap(Buf& o) {
+    std::swap(p, o.p);
+    std::swap(cap, o.cap);
+  }
   void* ensure(size_t bytes) {
     if (bytes == 0) bytes = 16;
     if (bytes > cap) {
@@ -64,6 +68,8 @@ struct Counters {
   int ngiant;         // clusters of more than kMergeBlockMax pairs
   long long gpairs;   // their pairs
   int blist_n;        // clusters listed for the block-level merge
+  int nlist;          // vertices or clusters listed (flag_list, the sparse contraction's merge)
+  int nab[2];         // vertices whose list is new for pass A, for pass B
 };
 
 enum Phase { kPhLP = 0, kPhContract, kPhPR, kPhNOI, kPhOther, kPhCount };
@@ -73,7 +79,7 @@ struct Workspace {
   cudaStream_t s = nullptr;
   // vertex-sized
   Buf deg, labA, labB, map0, cidT, cur1, side1, flags, rank, cnt, pos, scan64, scan32, hv;
-  Buf partner, pw, parent, slist, rlist, mlist, blist, glist, bl1, bcounts, noi_r;
+  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, slist, rlist, mlist, blist, glist, bl1, bcounts, noi_r;
   // entry-sized
   Buf tmpK, tmpV, cmpK, cmpV;
   // pair-sized
@@ -295,10 +301,52 @@ struct Workspace {
     bins_valid = true;
   }
 
+  // Partners and degrees of graph h, contracted from an nf-vertex graph by cid.  After a
+  // sparse contraction of a graph whose own arrays are valid (had), only changed lists are
+  // read; pr_new (after the next read_state, pr_new_read) says how many lists are new for a
+  // pass.  Graphs below kFlagMinN keep no flags: their passes cost launches, not lists.
+  static constexpr int64_t kFlagMinN = int64_t(1) << 15;
+  bool flags_ok = false;  // prflag describes the current graph
+  bool carried = false;
+  int64_t pr_new[2] = {0, 0};
+  void contracted_partners(const GraphView& h, int64_t nf, const int32_t* cid, bool had) {
+    carried = had && flags_ok && last_sparse && h.n >= kFlagMinN;
+    if (carried) {
+      const PrLists from{partner.as<int32_t>(), pw.as<long long>(), deg.as<long long>(), prflag.as<unsigned char>()};
+      // as large as the arrays they change places with, which serve larger graphs too
+      partner2.ensure(partner.cap);
+      pw2.ensure(pw.cap);
+      deg2.ensure(deg.cap);
+      prflag2.ensure(prflag.cap);
+      const PrLists to{partner2.as<int32_t>(), pw2.as<long long>(), deg2.as<long long>(),
+                       prflag2.as<unsigned char>()};
+      int32_t* list = prlist.ensure_n<int32_t>(nf);
+      pr_carry(nf, cid, sdeg.as<int32_t>(), sdirty.as<unsigned char>(), from, to, h.n, s);
+      flag_list(h.n, to.flag, kListNew, list, &ctr()->nlist, ctr()->nab, s);
+      pr_partners(h, to.partner, to.pw, to.deg, s, list, &ctr()->nlist, to.flag);
+      partner.swap(partner2);
+      pw.swap(pw2);
+      deg.swap(deg2);
+      prflag.swap(prflag2);
+    } else {
+      pr_partners(h, partner.as<int32_t>(), pw.as<long long>(), deg.as<long long>(), s);
+      flags_ok = h.n >= kFlagMinN;
+      if (flags_ok)
+        VC_CUDA(cudaMemsetAsync(prflag.ensure_n<unsigned char>(h.n), kListA | kListB, (size_t)h.n, s));
+    }
+    pr_new[0] = pr_new[1] = h.n;
+  }
+  void pr_new_read() {
+    if (carried)
+      for (int k = 0; k < 2; ++k) pr_new[k] = h_counters->nab[k];
+    carried = false;
+  }
+
   // Sparse contraction by union-find roots: counts the coarse lists of the lone vertices
   // it handles and bins the others (members of merged groups, lone vertices with too
   // many entries into them).  True when those are at most half of g's vertices; then
   // dbins holds their bins.
+  bool last_sparse = false;  // the last contraction was a sparse one
   Bins dbins;
   Buf smflag, scidm, sdirty, sdeg, sclean, sdlist, dsl, drl, dml, dbl, dgl, dbail, dcounts;
   // dbins' lists, for at most n listed vertices
@@ -470,6 +518,7 @@ struct Workspace {
     }
     const bool sparse = sparse_ok && !correct && g.simple && g.n > 0 && mark_sparse(g, labels, cid_out);
     if (!sparse && !bins_valid) build_bins(g);
+    last_sparse = sparse;
     const Bins& B = sparse ? dbins : bins;
     PairOut po{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
     po.nclust = &ctr()->c;
@@ -536,7 +585,7 @@ struct Workspace {
         gs.hist = hist.ensure_n<long long>(radix_hist_elems(GP));
       }
       const SparseCtx sp{scidm.as<int32_t>(), sdeg.as<int32_t>(), sclean.as<unsigned char>(),
-                         sdirty.as<unsigned char>()};
+                         sdirty.as<unsigned char>(), sdlist.as<int32_t>(), &ctr()->nlist};
       cluster_merge(g, cid_out, cs, ccount, c, cbase, cur, sk, sv, co, ca, cwp, csp, &st()->nnz,
                     h_counters->maxt > kMergeMax, 2 * c >= g.n, ng ? &gs : nullptr, cs.cnt, &ctr()->blist_n, s,
                     sparse ? &sp : nullptr);

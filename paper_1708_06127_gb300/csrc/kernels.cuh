@@ -227,6 +227,8 @@ struct SparseCtx {
   const int32_t* sdeg;
   unsigned char* clean;
   const unsigned char* dirty;  // 1: left to the pre-merge; 2: a lone list with no entry into a merged group
+  int32_t* list;               // scratch: c ids
+  int* list_n;
 };
 void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, unsigned char* mflag, int32_t* cidm,
                  unsigned char* dirty, int32_t* sdeg, int32_t* list, int* count, cudaStream_t s);
@@ -263,16 +265,40 @@ void side_bits2(const int32_t* orig_map, int64_t n, const unsigned char* side1, 
 void trace_push(DevState* st, TraceStep* trace, int cap, int kind, int level, cudaStream_t s);
 
 // ------------------------------------------------------------------ Padberg-Rinaldi
-void pr_partners(const GraphView& g, int32_t* partner, long long* pw, long long* deg, cudaStream_t s);
+// Degree, partner and partner weight of every vertex, or of the listed ones only (list,
+// list_n: on the device; flag then says which lists are long and listed).
+void pr_partners(const GraphView& g, int32_t* partner, long long* pw, long long* deg, cudaStream_t s,
+                 const int32_t* list = nullptr, const int* list_n = nullptr, const unsigned char* flag = nullptr);
+// What a vertex's list is new for (see pr.cu, "unchanged lists").
+constexpr int kListA = 1, kListB = 2, kListNew = 4;
+struct PrLists {
+  int32_t* partner;
+  long long *pw, *deg;
+  unsigned char* flag;
+};
+// After a sparse contraction of an n-vertex graph into c vertices: what unchanged lists
+// keep, from the old arrays into the new ones (the other vertices flagged with every bit).
+void pr_carry(int64_t n, const int32_t* cid, const int32_t* sdeg, const unsigned char* dirty, const PrLists& from,
+              const PrLists& to, int64_t c, cudaStream_t s);
+// list[0, *count): the vertices flagged with bit; nab (may be null): the numbers flagged
+// kListA and kListB.
+void flag_list(int64_t n, const unsigned char* flag, int bit, int32_t* list, int* count, int* nab, cudaStream_t s);
+void flag_clear(int64_t n, unsigned char* flag, int bit, cudaStream_t s);
 // Pass A: PR1 edges and PR2 designated-partner edges, union-find, roots -> labels.
 // With a batch context only active graphs are touched and `labels` must already
 // hold the identity for every other vertex.
 void pr_pass_a(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
                const DevState* st, int32_t* parent, int32_t* labels, int* changed, cudaStream_t s,
                const BatchCtx* bc = nullptr);
-// Pass B: PR3 / PR4 on mutual partner pairs.
+// Pass A where only the listed vertices' lists changed since a pass A with the same bound.
+void pr_pass_a_lists(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
+                     const DevState* st, const int32_t* list, const int* list_n, int32_t* parent, int32_t* labels,
+                     int* changed, cudaStream_t s);
+// Pass B: PR3 / PR4 on mutual partner pairs (flag not null: those with an end flagged
+// kListB, the others being unchanged since a pass B with the same bound).
 void pr_pass_b(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
-               const DevState* st, int32_t* labels, int* changed, cudaStream_t s, const BatchCtx* bc = nullptr);
+               const DevState* st, int32_t* labels, int* changed, cudaStream_t s, const BatchCtx* bc = nullptr,
+               const unsigned char* flag = nullptr);
 
 // ------------------------------------------------------------------ NOI
 constexpr int kDenseMax = 512;

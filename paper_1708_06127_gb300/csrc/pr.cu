@@ -45,15 +45,19 @@ __device__ __forceinline__ void partner_fold(long long& s, long long& bw, int& b
   if (x > bw || (x == bw && u < bu)) { bw = x; bu = u; }
 }
 
+// With a list (list_n not null) only the listed vertices list[0, *list_n).
 template <typename WT>
 __global__ void partners_k(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                            const WT* __restrict__ w, int32_t* __restrict__ partner, long long* __restrict__ pw,
-                           long long* __restrict__ deg) {
+                           long long* __restrict__ deg, const int32_t* __restrict__ list,
+                           const int* __restrict__ list_n) {
   constexpr int G = kPartnerG;
   const int lane = threadIdx.x & 31, glane = lane & (G - 1);
   const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (lane & ~(G - 1));
   const int64_t groups = (int64_t)gridDim.x * (blockDim.x / G);
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; v < n; v += groups) {
+  if (list_n) n = *list_n;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G; i < n; i += groups) {
+    const int64_t v = list_n ? (int64_t)list[i] : i;
     const int64_t beg = off[v], end = off[v + 1];
     if (end - beg > kPartnerBlockMin) continue;  // partners_long_k
     long long s = 0, bw = -1;
@@ -76,12 +80,14 @@ __global__ void partners_k(int64_t n, const int64_t* __restrict__ off, const int
 }
 
 // The lists of more than kPartnerBlockMin entries: each block lists the long ones among
-// 256 consecutive vertices, then folds each of them with all its threads.
+// 256 consecutive vertices (those flagged kListNew, where flags are given), then folds
+// each of them with all its threads.
 template <typename WT>
 __global__ void __launch_bounds__(256) partners_long_k(int64_t n, const int64_t* __restrict__ off,
                                                        const int32_t* __restrict__ adj, const WT* __restrict__ w,
                                                        int32_t* __restrict__ partner, long long* __restrict__ pw,
-                                                       long long* __restrict__ deg) {
+                                                       long long* __restrict__ deg,
+                                                       const unsigned char* __restrict__ flag) {
   __shared__ int32_t s_list[256];
   __shared__ int s_n;
   __shared__ long long s_s[8], s_bw[8];
@@ -91,7 +97,7 @@ __global__ void __launch_bounds__(256) partners_long_k(int64_t n, const int64_t*
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     const int64_t v0 = base + threadIdx.x;
-    if (v0 < n && off[v0 + 1] - off[v0] > kPartnerBlockMin) s_list[atomicAdd(&s_n, 1)] = (int32_t)v0;
+    if (v0 < n && (!flag || (flag[v0] & kListNew)) && off[v0 + 1] - off[v0] > kPartnerBlockMin) s_list[atomicAdd(&s_n, 1)] = (int32_t)v0;
     __syncthreads();
     const int cnt = s_n;
     for (int i = 0; i < cnt; ++i) {
@@ -123,16 +129,98 @@ __global__ void __launch_bounds__(256) partners_long_k(int64_t n, const int64_t*
   }
 }
 
-void pr_partners(const GraphView& g, int32_t* partner, long long* pw, long long* deg, cudaStream_t s) {
+void pr_partners(const GraphView& g, int32_t* partner, long long* pw, long long* deg, cudaStream_t s,
+                 const int32_t* list, const int* list_n, const unsigned char* flag) {
   const int grid = grid_for(g.n, 256 / kPartnerG, kSMs * 16), gl = grid_for(g.n, 256, kSMs * 4);
   if (g.wbytes == 4) {
-    partners_k<int32_t><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const int32_t*)g.w, partner, pw, deg);
-    partners_long_k<int32_t><<<gl, 256, 0, s>>>(g.n, g.off, g.adj, (const int32_t*)g.w, partner, pw, deg);
+    partners_k<int32_t><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const int32_t*)g.w, partner, pw, deg, list, list_n);
+    partners_long_k<int32_t><<<gl, 256, 0, s>>>(g.n, g.off, g.adj, (const int32_t*)g.w, partner, pw, deg, flag);
   } else {
-    partners_k<long long><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const long long*)g.w, partner, pw, deg);
-    partners_long_k<long long><<<gl, 256, 0, s>>>(g.n, g.off, g.adj, (const long long*)g.w, partner, pw, deg);
+    partners_k<long long><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const long long*)g.w, partner, pw, deg, list,
+                                               list_n);
+    partners_long_k<long long><<<gl, 256, 0, s>>>(g.n, g.off, g.adj, (const long long*)g.w, partner, pw, deg, flag);
   }
   count_launch(2);
+  VC_CHECK_LAUNCH();
+}
+
+// ------------------------------------------------------------ unchanged lists
+// A contraction that merges few vertices leaves most lists as they were but for the
+// renumbering.  What such a list gave keeps: its vertex's degree, partner and partner weight;
+// and an edge (a pair) both of whose lists are unchanged since a pass tested it with the same
+// bound still fails that test, as the pass merged whatever passed.  flag[v] says what v's
+// list is new for: kListNew (degree and partner, just now), kListA, kListB (a test of pass A,
+// of pass B).
+
+// From the old graph's vertices whose lists the sparse contraction copied unchanged (dirty
+// 2): degree, partner and flags under the new ids (flag1 starts with every bit set).
+__global__ void carry_k(int64_t n, const int32_t* __restrict__ cid, const int32_t* __restrict__ sdeg,
+                        const unsigned char* __restrict__ dirty, const long long* __restrict__ deg0,
+                        const int32_t* __restrict__ partner0, const long long* __restrict__ pw0,
+                        const unsigned char* __restrict__ flag0, long long* __restrict__ deg1,
+                        int32_t* __restrict__ partner1, long long* __restrict__ pw1,
+                        unsigned char* __restrict__ flag1) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+    if (sdeg[v] < 0 || dirty[v] != 2) continue;
+    const int32_t x = cid[v], p = partner0[v];
+    deg1[x] = deg0[v];
+    partner1[x] = p < 0 ? -1 : cid[p];  // a neighbour, so alone in its cluster too
+    pw1[x] = pw0[v];
+    flag1[x] = flag0[v] & (kListA | kListB);
+  }
+}
+
+// The vertices flagged with bit, listed (in no particular order), and the numbers of
+// vertices flagged kListA and kListB.
+__global__ void flag_list_k(int64_t n, const unsigned char* __restrict__ flag, int bit, int32_t* __restrict__ list,
+                            int* __restrict__ count, int* __restrict__ nab) {
+  const int lane = threadIdx.x & 31;
+  int na = 0, nb = 0;
+  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; b < n;
+       b += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = b + lane;
+    const int f = v < n ? flag[v] : 0;
+    na += (f & kListA) != 0;
+    nb += (f & kListB) != 0;
+    const unsigned bal = __ballot_sync(0xffffffffu, (f & bit) != 0);
+    int at = 0;
+    if (lane == 0 && bal) at = atomicAdd(count, __popc(bal));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (f & bit) list[at + __popc(bal & ((1u << lane) - 1u))] = (int32_t)v;
+  }
+  if (nab) {
+    na = (int)__reduce_add_sync(0xffffffffu, (unsigned)na);
+    nb = (int)__reduce_add_sync(0xffffffffu, (unsigned)nb);
+    if (lane == 0 && na) atomicAdd(nab, na);
+    if (lane == 0 && nb) atomicAdd(nab + 1, nb);
+  }
+}
+
+__global__ void flag_clear_k(int64_t n, unsigned char* __restrict__ flag, int bit) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+    flag[v] = (unsigned char)(flag[v] & ~bit);
+}
+
+void flag_clear(int64_t n, unsigned char* flag, int bit, cudaStream_t s) {
+  flag_clear_k<<<grid_for(n, 256, kSMs * 8), 256, 0, s>>>(n, flag, bit);
+  count_launch();
+  VC_CHECK_LAUNCH();
+}
+
+void flag_list(int64_t n, const unsigned char* flag, int bit, int32_t* list, int* count, int* nab, cudaStream_t s) {
+  VC_CUDA(cudaMemsetAsync(count, 0, sizeof(int), s));
+  if (nab) VC_CUDA(cudaMemsetAsync(nab, 0, 2 * sizeof(int), s));
+  flag_list_k<<<grid_for(n, 256, kSMs * 8), 256, 0, s>>>(n, flag, bit, list, count, nab);
+  count_launch();
+  VC_CHECK_LAUNCH();
+}
+
+void pr_carry(int64_t n, const int32_t* cid, const int32_t* sdeg, const unsigned char* dirty, const PrLists& from,
+              const PrLists& to, int64_t c, cudaStream_t s) {
+  VC_CUDA(cudaMemsetAsync(to.flag, kListNew | kListA | kListB, (size_t)c, s));
+  carry_k<<<grid_for(n, 256, kSMs * 8), 256, 0, s>>>(n, cid, sdeg, dirty, from.deg, from.partner, from.pw, from.flag,
+                                                     to.deg, to.partner, to.pw, to.flag);
+  count_launch();
   VC_CHECK_LAUNCH();
 }
 
@@ -265,6 +353,27 @@ __global__ void pr_a_partner_k(int64_t n, const int64_t* __restrict__ off, const
   }
 }
 
+// Condition 1 on the entries of the listed vertices (a warp each), in both directions: an
+// edge with a listed end is seen from there.
+template <typename WT>
+__global__ void pr_a_list_k(const int32_t* __restrict__ list, const int* __restrict__ list_n,
+                            const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+                            const WT* __restrict__ w, const DevState* st, int32_t* parent) {
+  const int lane = threadIdx.x & 31, n = *list_n;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  const long long lam = st->lambda_hat;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
+    const int32_t v = list[i];
+    const int64_t beg = off[v], end = off[v + 1];
+    if (end - beg < 2) continue;
+    for (int64_t e = beg + lane; e < end; e += 32) {
+      if ((long long)w[e] < lam) continue;
+      const int32_t u = adj[e];
+      if (off[u + 1] - off[u] >= 2) uf_unite(parent, v, u);
+    }
+  }
+}
+
 template <typename WT>
 __global__ void pr_a_mark_k(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                             const WT* __restrict__ w, const int32_t* __restrict__ partner,
@@ -336,19 +445,36 @@ void pr_pass_a(const GraphView& g, const int32_t* partner, const long long* pw, 
   VC_CHECK_LAUNCH();
 }
 
+void pr_pass_a_lists(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
+                     const DevState* st, const int32_t* list, const int* list_n, int32_t* parent, int32_t* labels,
+                     int* changed, cudaStream_t s) {
+  const BatchCtx bc{};
+  const int grid1 = grid_for(g.n, 256, kSMs * 8), grid = grid_for(g.n, 8, kSMs * 16);
+  uf_init_k<<<grid1, 256, 0, s>>>(parent, g.n);
+  if (g.wbytes == 4)
+    pr_a_list_k<int32_t><<<grid, 256, 0, s>>>(list, list_n, g.off, g.adj, (const int32_t*)g.w, st, parent);
+  else
+    pr_a_list_k<long long><<<grid, 256, 0, s>>>(list, list_n, g.off, g.adj, (const long long*)g.w, st, parent);
+  pr_a_partner_k<<<grid1, 256, 0, s>>>(g.n, g.off, partner, pw, deg, st, parent, bc);
+  uf_flatten_k<<<grid1, 256, 0, s>>>(parent, g.n, labels, changed, bc);
+  count_launch(4);
+  VC_CHECK_LAUNCH();
+}
+
 // Conditions 3 and 4 on mutual partner pairs v < w = p(v), p(w) = v, through the
 // common neighbourhood: the warp walks the shorter of the two lists and finds each entry
 // in the longer one by binary search (a longer list of at most kPrBStage ids is first
 // copied into the warp's shared memory, so the searches there wait on no global loads).
 // Walking the shorter list keeps a pair of a hub and a small vertex as cheap as the
-// small vertex's list.
+// small vertex's list.  With flags, only pairs with an end flagged kListB are tested.
 constexpr int kPrBStage = 1024;
 template <typename WT>
 __global__ void __launch_bounds__(256) pr_b_k(int64_t n, const int64_t* __restrict__ off,
                                               const int32_t* __restrict__ adj, const WT* __restrict__ w,
                                               const int32_t* __restrict__ partner, const long long* __restrict__ pw,
                                               const long long* __restrict__ deg, const DevState* st,
-                                              int32_t* __restrict__ labels, int* changed, BatchCtx bc) {
+                                              int32_t* __restrict__ labels, int* changed, BatchCtx bc,
+                                              const unsigned char* __restrict__ flag) {
   __shared__ int32_t s_list[8][kPrBStage];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int32_t* sl = s_list[wid];
@@ -358,6 +484,7 @@ __global__ void __launch_bounds__(256) pr_b_k(int64_t n, const int64_t* __restri
     if (!pr_graph(bc, st, v, &lam)) continue;
     const int p = partner[v];
     if (p <= v || partner[p] != v) continue;
+    if (flag && !((flag[v] | flag[p]) & kListB)) continue;
     const int64_t vb = off[v], ve = off[v + 1], pb = off[p], pe = off[p + 1];
     if (ve - vb < 2 || pe - pb < 2) continue;
     const long long cvw = pw[v], dv = deg[v], dp = deg[p];
@@ -407,16 +534,17 @@ __global__ void __launch_bounds__(256) pr_b_k(int64_t n, const int64_t* __restri
 }
 
 void pr_pass_b(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
-               const DevState* st, int32_t* labels, int* changed, cudaStream_t s, const BatchCtx* bcp) {
+               const DevState* st, int32_t* labels, int* changed, cudaStream_t s, const BatchCtx* bcp,
+               const unsigned char* flag) {
   BatchCtx bc = bcp ? *bcp : BatchCtx{};
   if (!bc.gid) iota(labels, g.n, s);
   int grid = grid_for(g.n, 8, kSMs * 16);
   if (g.wbytes == 4)
     pr_b_k<int32_t><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const int32_t*)g.w, partner, pw, deg, st, labels,
-                                         changed, bc);
+                                         changed, bc, flag);
   else
     pr_b_k<long long><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const long long*)g.w, partner, pw, deg, st, labels,
-                                           changed, bc);
+                                           changed, bc, flag);
   count_launch();
   VC_CHECK_LAUNCH();
 }

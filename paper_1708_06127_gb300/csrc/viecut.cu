@@ -200,6 +200,7 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
   G.unit = H.unit;
   G.simple = H.simple;
   W.bins_valid = false;
+  W.flags_ok = W.carried = false;
 
   cudaEvent_t a = W.mark();
   degrees(G, W.deg.as<long long>(), s);
@@ -217,6 +218,9 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
   // W.partner / W.pw / W.deg hold the partners of the current G (a pass that merged
   // nothing leaves G, and so them, as they were)
   bool partners_ok = false;
+  // the bound of the last pass A and pass B (-1: none): W.prflag says which lists changed
+  // since, and a pass with the same bound tests only what those hold
+  long long lam_a = -1, lam_b = -1;
 
   // contraction + bound update; returns false when the run ends
   auto step = [&](const int32_t* labels, int kind) -> bool {
@@ -240,11 +244,12 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
     slot = dst;
     W.span(kPhContract, a0);
     cudaEvent_t a1 = W.mark();
+    const bool had_partners = partners_ok;
     partners_ok = false;
     if (G.n > 1) {
       // the weighted degrees for the bound, with the partners the next Padberg-Rinaldi
-      // pass reads (the same scan of every list)
-      pr_partners(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), s);
+      // pass reads (the same scan of the changed lists)
+      W.contracted_partners(G, fine.n, cid, had_partners);
       partners_ok = true;
       bound_update(W.deg.as<long long>(), G.n, st, W.partial.as<long long>(), s);
       snapshot_side(W.cur1.as<int32_t>(), n1, W.side1.as<unsigned char>(), st, s);
@@ -252,6 +257,7 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
     trace_push(st, tr, tcap, kind, level, s);
     W.span(kPhOther, a1);
     W.read_state();
+    W.pr_new_read();
     G.nnz = W.h_state->nnz;
     W.count_contract(fine, G.n, G.nnz);
     return G.n > 1 && W.h_state->lambda_hat > 0;
@@ -287,15 +293,27 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
       for (int pass = 0; pass < 2; ++pass) {
         cudaEvent_t ap = W.mark();
         VC_CUDA(cudaMemsetAsync(&W.ctr()->changed, 0, sizeof(int), s));
-        if (!partners_ok) pr_partners(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), s);
-        partners_ok = true;
         int32_t* lab = W.labA.as<int32_t>();
-        if (pass == 0)
+        const long long lam = W.h_state->lambda_hat;
+        const int bit = pass == 0 ? kListA : kListB;
+        // few lists changed since this pass last ran, with the same bound: only those
+        const bool few = W.flags_ok && (pass == 0 ? lam_a : lam_b) == lam && 4 * W.pr_new[pass] <= G.n;
+        unsigned char* flag = W.prflag.as<unsigned char>();
+        if (pass == 0 && few) {
+          int32_t* list = W.prlist.ensure_n<int32_t>(G.n);
+          flag_list(G.n, flag, kListA, list, &W.ctr()->nlist, nullptr, s);
+          pr_pass_a_lists(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), st, list,
+                          &W.ctr()->nlist, W.parent.as<int32_t>(), lab, &W.ctr()->changed, s);
+        } else if (pass == 0) {
           pr_pass_a(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), st,
                     W.parent.as<int32_t>(), lab, &W.ctr()->changed, s);
-        else
+        } else {
           pr_pass_b(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), st, lab,
-                    &W.ctr()->changed, s);
+                    &W.ctr()->changed, s, nullptr, few ? flag : nullptr);
+        }
+        if (W.flags_ok) flag_clear(G.n, flag, bit, s);
+        W.pr_new[pass] = 0;
+        (pass == 0 ? lam_a : lam_b) = lam;
         W.span(kPhPR, ap);
         if (read_changed()) {
           any = true;
