@@ -52,7 +52,8 @@ void relabel(const int32_t* lab, int64_t n, int32_t* cid, ContractScratch& cs, i
 template <int W>
 __global__ void build_pairs_k(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ cid,
                               const int32_t* __restrict__ cnt, const long long* __restrict__ pos, PairOut in,
-                              int bits, unsigned long long* __restrict__ keys, long long* __restrict__ vals) {
+                              int bits, unsigned long long* __restrict__ keys, long long* __restrict__ vals,
+                              LongLists longs) {
   const int lane = threadIdx.x & (W - 1);
   const int64_t groups = (int64_t)gridDim.x * (blockDim.x / W);
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W; v < n; v += groups) {
@@ -60,6 +61,10 @@ __global__ void build_pairs_k(int64_t n, const int64_t* __restrict__ off, const 
     if (k == 0) continue;
     const int64_t src = off[v];
     const long long dst = pos[v];
+    if (longs.item && k > kLongList) {
+      if (lane == 0) longs.push((int32_t)v, dst);
+      continue;
+    }
     const unsigned long long hi = (unsigned long long)cid[v] << bits;
     for (int j = lane; j < k; j += W) {
       int32_t kk;
@@ -71,16 +76,44 @@ __global__ void build_pairs_k(int64_t n, const int64_t* __restrict__ off, const 
   }
 }
 
+// The lists build_pairs_k left out.
+__global__ void build_pairs_long_k(const int64_t* __restrict__ off, const int32_t* __restrict__ cid,
+                                   const int32_t* __restrict__ cnt, PairOut in, int bits,
+                                   unsigned long long* __restrict__ keys, long long* __restrict__ vals,
+                                   LongLists longs) {
+  const int n = *longs.n;
+  const GridShare G(n);
+  for (int i = G.first; i < n; i += G.step) {
+    const int32_t v = longs.item[i];
+    const long long dst = longs.at[i];
+    const int64_t src = off[v];
+    const int k = cnt[v];
+    const unsigned long long hi = (unsigned long long)cid[v] << bits;
+    for (int64_t j = (int64_t)G.part * blockDim.x + threadIdx.x; j < k; j += (int64_t)G.parts * blockDim.x) {
+      int32_t kk;
+      long long x;
+      in.get(v, src, (int)j, &kk, &x);
+      keys[dst + j] = hi | (unsigned long long)(uint32_t)kk;
+      vals[dst + j] = x;
+    }
+  }
+}
+
 void build_pairs(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int bits, int64_t pairs,
-                 unsigned long long* keys, long long* vals, cudaStream_t s) {
+                 const LongLists& longs, unsigned long long* keys, long long* vals, cudaStream_t s) {
+  if (longs.item) VC_CUDA(cudaMemsetAsync(longs.n, 0, sizeof(int), s));
   const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
   if (pairs <= 2 * g.n)
-    build_pairs_k<1><<<grid_for(g.n, 256, kSMs * 8), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals);
+    build_pairs_k<1><<<grid_for(g.n, 256, kSMs * 8), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals, longs);
   else if (pairs <= 16 * g.n)
-    build_pairs_k<8><<<grid_for(g.n, 32, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals);
+    build_pairs_k<8><<<grid_for(g.n, 32, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals, longs);
   else
-    build_pairs_k<32><<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals);
+    build_pairs_k<32><<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals, longs);
   count_launch();
+  if (longs.item) {
+    build_pairs_long_k<<<kSMs * 4, 256, 0, s>>>(g.off, cid, cs.cnt, in, bits, keys, vals, longs);
+    count_launch();
+  }
   VC_CHECK_LAUNCH();
 }
 
@@ -275,7 +308,7 @@ __global__ void __launch_bounds__(256) cluster_scatter_k(int64_t n, const int64_
                                                          const int32_t* __restrict__ cid,
                                                          const int32_t* __restrict__ cnt, PairOut in,
                                                          long long* __restrict__ cursor, int32_t* __restrict__ seg_key,
-                                                         long long* __restrict__ seg_val) {
+                                                         long long* __restrict__ seg_val, LongLists longs) {
   __shared__ int s_k[8][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -309,8 +342,11 @@ __global__ void __launch_bounds__(256) cluster_scatter_k(int64_t n, const int64_
         }
       }
     }
-    // the rest of the long lists, laid end to end over the lanes (coalesced)
-    const bool longl = c >= 0 && k > kScatterWarpMin;
+    // the rest of the long lists, laid end to end over the lanes (coalesced); the longest by
+    // cluster_scatter_long_k
+    const bool whole = longs.item && k > kLongList;
+    if (c >= 0 && whole) longs.push((int32_t)v, dst);
+    const bool longl = c >= 0 && k > kScatterWarpMin && !whole;
     if (__any_sync(0xffffffffu, longl)) {
       warp_pieces<KeyVal>(
           longl ? (int64_t)(k - kPairSlots) : 0, longl ? off[v] + kPairSlots : 0, dst + kPairSlots,
@@ -319,6 +355,25 @@ __global__ void __launch_bounds__(256) cluster_scatter_k(int64_t n, const int64_
             seg_key[at] = kv.k;
             seg_val[at] = kv.v;
           });
+    }
+  }
+}
+
+// The rests of the lists cluster_scatter_k left out.
+__global__ void cluster_scatter_long_k(const int64_t* __restrict__ off, const int32_t* __restrict__ cnt, PairOut in,
+                                       int32_t* __restrict__ seg_key, long long* __restrict__ seg_val,
+                                       LongLists longs) {
+  const int n = *longs.n;
+  const GridShare G(n);
+  for (int i = G.first; i < n; i += G.step) {
+    const int32_t v = longs.item[i];
+    const long long dst = longs.at[i];
+    const int64_t src = off[v];
+    const int k = cnt[v];
+    for (int64_t j = kPairSlots + (int64_t)G.part * blockDim.x + threadIdx.x; j < k;
+         j += (int64_t)G.parts * blockDim.x) {
+      seg_key[dst + j] = in.tkey[src + j];
+      seg_val[dst + j] = in.tval[src + j];
     }
   }
 }
@@ -566,7 +621,7 @@ __global__ void __launch_bounds__(256) cluster_place_k(int64_t c, const long lon
                                                        const long long* __restrict__ seg_val,
                                                        int32_t* __restrict__ cadj, long long* __restrict__ cw,
                                                        int32_t* __restrict__ csrc,
-                                                       const unsigned char* __restrict__ skip) {
+                                                       const unsigned char* __restrict__ skip, LongLists longs) {
   // 32 clusters per warp step, their lists laid end to end over the lanes
   const int lane = threadIdx.x & 31;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -575,7 +630,11 @@ __global__ void __launch_bounds__(256) cluster_place_k(int64_t c, const long lon
     const bool take = x < c && !(skip && skip[x]);
     const long long b = take ? cbase[x] : 0;
     const int64_t o = take ? coff[x] : 0;
-    const int64_t D = take ? coff[x + 1] - o : 0;
+    int64_t D = take ? coff[x + 1] - o : 0;
+    if (longs.item && D > kLongList) {
+      longs.push((int32_t)x, o);
+      D = 0;
+    }
     warp_pieces<KeyVal>(
         D, b, o, [&](int64_t at) { return KeyVal{seg_key[at], seg_val[at]}; },
         [&](int64_t at, int j, const KeyVal& kv) {
@@ -586,6 +645,25 @@ __global__ void __launch_bounds__(256) cluster_place_k(int64_t c, const long lon
   }
 }
 
+
+// The lists cluster_place_k left out.
+__global__ void cluster_place_long_k(const long long* __restrict__ cbase, const int64_t* __restrict__ coff,
+                                     const int32_t* __restrict__ seg_key, const long long* __restrict__ seg_val,
+                                     int32_t* __restrict__ cadj, long long* __restrict__ cw,
+                                     int32_t* __restrict__ csrc, LongLists longs) {
+  const int n = *longs.n;
+  const GridShare G(n);
+  for (int i = G.first; i < n; i += G.step) {
+    const int32_t x = longs.item[i];
+    const long long b = cbase[x];
+    const int64_t o = longs.at[i], D = coff[x + 1] - o;
+    for (int64_t j = (int64_t)G.part * blockDim.x + threadIdx.x; j < D; j += (int64_t)G.parts * blockDim.x) {
+      cadj[o + j] = seg_key[b + j];
+      cw[o + j] = seg_val[b + j];
+      csrc[o + j] = x;
+    }
+  }
+}
 
 // ---------------------------------------------------------------- sparse contraction
 // Contractions in which most vertices keep their own id as label, alone in their cluster
@@ -1122,12 +1200,18 @@ __global__ void warp_class_list_k(int64_t c, const long long* __restrict__ cbase
 void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int32_t* ccount, int64_t c,
                    long long* cbase, long long* cursor, int32_t* seg_key, long long* seg_val, int64_t* coff,
                    int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, bool big, bool sort_first,
-                   const GiantScratch* giant, int32_t* blist, int* blist_n, cudaStream_t s, const SparseCtx* sp) {
+                   const GiantScratch* giant, int32_t* blist, int* blist_n, cudaStream_t s, const SparseCtx* sp,
+                   const LongLists& longs) {
   exclusive_scan<int, long long>(ccount, cbase, c, cbase + c, cs.scan_scr, s);
   VC_CUDA(cudaMemcpyAsync(cursor, cbase, sizeof(long long) * c, cudaMemcpyDeviceToDevice, s));
   const int gv = grid_for(g.n, 256, kSMs * 8), gc = grid_for(c, 8, kSMs * 16);
   const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
-  cluster_scatter_k<<<gv, 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, cursor, seg_key, seg_val);
+  if (longs.item) VC_CUDA(cudaMemsetAsync(longs.n, 0, sizeof(int), s));
+  cluster_scatter_k<<<gv, 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, cursor, seg_key, seg_val, longs);
+  if (longs.item) {
+    cluster_scatter_long_k<<<kSMs * 4, 256, 0, s>>>(g.off, cs.cnt, in, seg_key, seg_val, longs);
+    count_launch();
+  }
   if (sp) {
     VC_CUDA(cudaMemsetAsync(sp->list_n, 0, sizeof(int), s));
     warp_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, sp->list, sp->list_n);
@@ -1150,8 +1234,13 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
   if (giant && giant->ngiant > 0) giant_merge(*giant, c, cbase, seg_key, seg_val, ccount, cs.scan_scr, s);
   if (sp) sparse_finish_degrees(g, cid, sp->sdeg, ccount, sp->clean, c, s);
   exclusive_scan<int, long long>(ccount, (long long*)coff, c, (long long*)coff + c, cs.scan_scr, s);
+  if (longs.item) VC_CUDA(cudaMemsetAsync(longs.n, 0, sizeof(int), s));
   cluster_place_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, coff, seg_key, seg_val, cadj, cw, csrc,
-                                                               sp ? sp->clean : nullptr);
+                                                               sp ? sp->clean : nullptr, longs);
+  if (longs.item) {
+    cluster_place_long_k<<<kSMs * 4, 256, 0, s>>>(cbase, coff, seg_key, seg_val, cadj, cw, csrc, longs);
+    count_launch();
+  }
   count_launch();
   VC_CHECK_LAUNCH();
   if (sp) sparse_copy(g, sp->cidm, sp->sdeg, sp->dirty, coff, cadj, cw, csrc, s);

@@ -69,6 +69,7 @@ struct Counters {
   long long gpairs;   // their pairs
   int blist_n;        // clusters listed for the block-level merge
   int nlist;          // vertices or clusters listed (flag_list, the sparse contraction's merge)
+  int nlong;          // lists left to a grid's blocks to share (LongLists, PrLong)
   int nab[2];         // vertices whose list is new for pass A, for pass B
 };
 
@@ -79,7 +80,7 @@ struct Workspace {
   cudaStream_t s = nullptr;
   // vertex-sized
   Buf deg, labA, labB, map0, cidT, cur1, side1, flags, rank, cnt, pos, scan64, scan32, hv;
-  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, slist, rlist, mlist, blist, glist, bl1, bcounts, noi_r;
+  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, longV, longAt, longHit, slist, rlist, mlist, blist, glist, bl1, bcounts, noi_r;
   // entry-sized
   Buf tmpK, tmpV, cmpK, cmpV;
   // pair-sized
@@ -336,6 +337,18 @@ struct Workspace {
     }
     pr_new[0] = pr_new[1] = h.n;
   }
+  // Room for the long pairs that pass B leaves to a second kernel (none on graphs too small
+  // to hold long lists in number: two launches and the clearing for every pass).
+  PrLong pr_long(int64_t nnz) {
+    PrLong L;
+    if (nnz < (int64_t(1) << 20)) return L;
+    const int64_t cap = pr_long_cap(nnz);
+    L.v = longV.ensure_n<int32_t>(cap);
+    L.sum = longAt.ensure_n<unsigned long long>(cap);
+    L.pr3 = longHit.ensure_n<int>(cap);
+    L.n = &ctr()->nlong;
+    return L;
+  }
   void pr_new_read() {
     if (carried)
       for (int k = 0; k < 2; ++k) pr_new[k] = h_counters->nab[k];
@@ -560,6 +573,12 @@ struct Workspace {
     // those hold most of the pairs (then one radix sort of all pairs)
     const int ng = h_counters->maxt > kMergeBlockMax ? h_counters->ngiant : 0;
     const int64_t GP = ng ? h_counters->gpairs : 0;
+    LongLists longs;  // a list that long makes its cluster a giant one
+    if (ng) {
+      longs.item = longV.ensure_n<int32_t>(long_list_cap(P));
+      longs.at = longAt.ensure_n<long long>(long_list_cap(P));
+      longs.n = &ctr()->nlong;
+    }
     if (2 * GP <= P || sparse) {
       long long* cbase = pos.as<long long>();  // n + 1 >= c + 1 entries
       long long* cur = ccur.ensure_n<long long>(std::max<int64_t>(c, 1));
@@ -588,7 +607,7 @@ struct Workspace {
                          sdirty.as<unsigned char>(), sdlist.as<int32_t>(), &ctr()->nlist};
       cluster_merge(g, cid_out, cs, ccount, c, cbase, cur, sk, sv, co, ca, cwp, csp, &st()->nnz,
                     h_counters->maxt > kMergeMax, 2 * c >= g.n, ng ? &gs : nullptr, cs.cnt, &ctr()->blist_n, s,
-                    sparse ? &sp : nullptr);
+                    sparse ? &sp : nullptr, longs);
     } else {
       exclusive_scan<int, long long>(cs.cnt, cs.pos, g.n, &ctr()->pairs, cs.scan_scr, s);
       int bits = ceil_log2(c);
@@ -601,7 +620,7 @@ struct Workspace {
       auto* hd = heads.ensure_n<int32_t>(P);
       auto* hp = hpos.ensure_n<long long>(P + 1);
       scan64.ensure_n<long long>(scan_scratch_elems(std::max<int64_t>(P, 1)) + 1);
-      build_pairs(g, cid_out, cs, bits, P, kA, vA, s);
+      build_pairs(g, cid_out, cs, bits, P, longs, kA, vA, s);
       radix_sort_pairs(kA, vA, kB, vB, P, 2 * bits, hs, s);
       reduce_pairs(kA, vA, P, bits, c, hd, hp, scan64.as<long long>(), co, ca, cwp, csp, &st()->nnz, s);
     }

@@ -191,6 +191,36 @@ struct CorrectScratch {
 };
 void correct_clusters(const GraphView& g, int32_t* cid, int* c_dev, const CorrectScratch& cs, cudaStream_t s);
 
+// How the blocks of a grid share n lists of any length: fewer lists than blocks get `parts`
+// blocks each (this block is number `part` of list `first`), more go round the blocks.
+struct GridShare {
+  int first, step, parts, part;
+  __device__ __forceinline__ explicit GridShare(int n) {
+    const int g = (int)gridDim.x, b = (int)blockIdx.x;
+    parts = n > 0 && n < g ? g / n : 1;
+    step = g / parts;
+    part = b / step;
+    first = part < parts ? b - part * step : n;
+  }
+};
+
+// Lists of more than kLongList pieces are left by the kernels that copy a list with a warp
+// to a second one in which the grid's blocks share them (a hub that absorbed many vertices
+// holds a tenth of a graph's entries: 3 ms by one warp).  item[*n] receives the vertex or
+// cluster, at[*n] where its list goes; both hold long_list_cap(pairs) entries.
+constexpr int kLongList = 4096;
+inline int64_t long_list_cap(int64_t pairs) { return pairs / kLongList + 1; }
+struct LongLists {
+  int32_t* item = nullptr;  // null: no list is that long
+  long long* at = nullptr;
+  int* n = nullptr;
+  __device__ __forceinline__ void push(int32_t x, long long to) const {
+    const int i = atomicAdd(n, 1);
+    item[i] = x;
+    at[i] = to;
+  }
+};
+
 // Cluster merge: a warp merges clusters of at most kMergeMax pre-merged pairs in
 // registers, a block those of at most kMergeBlockMax; the few "giant" clusters beyond
 // that (GiantScratch) are merged together by one radix sort of their pairs keyed by
@@ -236,11 +266,11 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
                    long long* cbase, long long* cursor, int32_t* seg_key, long long* seg_val, int64_t* coff,
                    int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, bool big, bool sort_first,
                    const GiantScratch* giant, int32_t* blist, int* blist_n, cudaStream_t s,
-                   const SparseCtx* sparse = nullptr);
+                   const SparseCtx* sparse = nullptr, const LongLists& longs = LongLists());
 
 // Builds (cid[v] << bits | cu, weight) pairs from the pre-merged lists.
 void build_pairs(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int bits, int64_t pairs,
-                 unsigned long long* keys, long long* vals, cudaStream_t s);
+                 const LongLists& longs, unsigned long long* keys, long long* vals, cudaStream_t s);
 
 // From sorted pairs: merge equal keys, write the coarse CSR (offsets for c
 // vertices).  Uses heads/hpos scratch of `pairs` elements; *nnz_dev gets the count.
@@ -290,6 +320,17 @@ void flag_clear(int64_t n, unsigned char* flag, int bit, cudaStream_t s);
 void pr_pass_a(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
                const DevState* st, int32_t* parent, int32_t* labels, int* changed, cudaStream_t s,
                const BatchCtx* bc = nullptr);
+// Pairs whose shorter list holds more than kPrLongMin entries, left to a kernel in which the
+// grid's blocks share them (hub and hub: 2.8 ms by one warp).  v[*n]: the pair's lower vertex;
+// sum and pr3: its results; all hold pr_long_cap(entries) entries.
+constexpr int kPrLongMin = 2048;
+inline int64_t pr_long_cap(int64_t nnz) { return nnz / kPrLongMin + 1; }
+struct PrLong {
+  int32_t* v = nullptr;  // null: a warp walks every pair
+  unsigned long long* sum = nullptr;
+  int* pr3 = nullptr;
+  int* n = nullptr;
+};
 // Pass A where only the listed vertices' lists changed since a pass A with the same bound.
 void pr_pass_a_lists(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
                      const DevState* st, const int32_t* list, const int* list_n, int32_t* parent, int32_t* labels,
@@ -298,7 +339,7 @@ void pr_pass_a_lists(const GraphView& g, const int32_t* partner, const long long
 // kListB, the others being unchanged since a pass B with the same bound).
 void pr_pass_b(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
                const DevState* st, int32_t* labels, int* changed, cudaStream_t s, const BatchCtx* bc = nullptr,
-               const unsigned char* flag = nullptr);
+               const unsigned char* flag = nullptr, const PrLong& longs = PrLong());
 
 // ------------------------------------------------------------------ NOI
 constexpr int kDenseMax = 512;

@@ -1143,6 +1143,49 @@ __global__ void __launch_bounds__(kAggThreads) emit_block_k(const int32_t* __res
   }
 }
 
+// Listed vertices of long lists (more than kBlockMaxDeg entries), shared by the grid's blocks:
+// a warp reserves its pairs' places with one addition to the vertex's count per 32 entries.
+// A hub of 400,000 entries took 0.44 ms by a block of its own.
+__global__ void emit_zero_k(const int32_t* __restrict__ list, const int* __restrict__ count_ptr,
+                            int32_t* __restrict__ cnt) {
+  const int count = *count_ptr;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) cnt[list[i]] = 0;
+}
+
+template <typename WT>
+__global__ void __launch_bounds__(kAggThreads) emit_split_k(const int32_t* __restrict__ list,
+                                                            const int* __restrict__ count_ptr,
+                                                            const int64_t* __restrict__ off,
+                                                            const int32_t* __restrict__ adj,
+                                                            const WT* __restrict__ w, const int32_t* __restrict__ cid,
+                                                            PairOut out, int32_t* __restrict__ cnt) {
+  __shared__ int s_made;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int count = *count_ptr;
+  const GridShare G(count);
+  for (int idx = G.first; idx < count; idx += G.step) {
+    const int32_t v = list[idx];
+    const int64_t beg = off[v], end = off[v + 1];
+    const int32_t own = cid[v];
+    if (own < 0) continue;  // the same in every thread
+    if (threadIdx.x == 0) s_made = 0;
+    __syncthreads();
+    for (int64_t base = beg + 32 * ((int64_t)G.part * kWarpsPerBlock + wib); base < end;
+         base += 32 * (int64_t)kWarpsPerBlock * G.parts)
+      emit_chunk_rows<WT, 32>(base + lane, end, adj, w, cid, own, lane, 0xffffffffu, out, v, beg, [&](int k) {
+        int at = 0;
+        if (lane == 0) {
+          at = atomicAdd(cnt + v, k);
+          atomicAdd(&s_made, k);
+        }
+        return __shfl_sync(0xffffffffu, at, 0);
+      });
+    __syncthreads();
+    if (threadIdx.x == 0 && out.ccount && s_made) atomicAdd(&out.ccount[own], s_made);
+    __syncthreads();
+  }
+}
+
 // --------------------------------------------------------- block / global classes
 // Label propagation, one block per listed vertex; the table lives in shared memory
 // (GLOBAL = false) or in this block's region of global scratch (GLOBAL = true).
@@ -1319,9 +1362,9 @@ void launch_emit(const GraphView& g, const Bins& b, const int32_t* cid, const Pa
     VC_CHECK_LAUNCH();
   }
   if (b.h_global > 0) {
-    emit_block_k<WT><<<grid_for(b.h_global, 1, kSMs * 4), kAggThreads, 0, s>>>(b.global_list, b.counts + 2, g.off,
-                                                                               g.adj, w, cid, out, cnt);
-    count_launch();
+    emit_zero_k<<<grid_for(b.h_global, 256, kSMs), 256, 0, s>>>(b.global_list, b.counts + 2, cnt);
+    emit_split_k<WT><<<kSMs * 4, kAggThreads, 0, s>>>(b.global_list, b.counts + 2, g.off, g.adj, w, cid, out, cnt);
+    count_launch(2);
     VC_CHECK_LAUNCH();
   }
 }

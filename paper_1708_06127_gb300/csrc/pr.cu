@@ -104,7 +104,20 @@ __global__ void __launch_bounds__(256) partners_long_k(int64_t n, const int64_t*
       const int32_t v = s_list[i];
       long long s = 0, bw = -1;
       int bu = INT_MAX;
-      for (int64_t e = off[v] + threadIdx.x; e < off[v + 1]; e += 256) partner_fold(s, bw, bu, (long long)w[e], adj[e]);
+      const int64_t end = off[v + 1];
+      for (int64_t e0 = off[v] + threadIdx.x; e0 < end; e0 += 8 * 256) {  // eight entries in flight per thread
+        long long x[8];
+        int u[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int64_t e = e0 + 256 * q;
+          x[q] = e < end ? (long long)w[e] : -1;
+          u[q] = e < end ? adj[e] : INT_MAX;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (x[q] >= 0) partner_fold(s, bw, bu, x[q], u[q]);
+      }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         const long long os = __shfl_xor_sync(0xffffffffu, s, o);
@@ -293,6 +306,7 @@ __global__ void pr_a_edge_k(int64_t n, const int32_t* __restrict__ src, const in
 // at the first row holding a marked entry below v or an entry at or above v.
 constexpr int kInitMinG = 8;
 constexpr int kInitMinRows = 4;
+constexpr int kInitMinReach = 1024;
 template <typename WT>
 __global__ void uf_init_min_k(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                               const WT* __restrict__ w, const DevState* st, int32_t* __restrict__ parent,
@@ -307,7 +321,10 @@ __global__ void uf_init_min_k(int64_t n, const int64_t* __restrict__ off, const 
     const int64_t beg = off[v], end = off[v + 1];
     if (end - beg >= 2 && pr_graph(bc, st, v, &lam)) {
       bool found = false;
-      for (int64_t b = beg; b < end && !found; b += kInitMinRows * G) {
+      // a start is only a start: a vertex without a marked neighbour among its first
+      // kInitMinReach stays its own (a hub's eight lanes would walk on alone)
+      const int64_t reach = end - beg > kInitMinReach ? beg + kInitMinReach : end;
+      for (int64_t b = beg; b < reach && !found; b += kInitMinRows * G) {
         // kInitMinRows rows in flight: ids, then the weights of the entries below v,
         // then the list lengths of the heavy ones
         int u[kInitMinRows];
@@ -474,7 +491,7 @@ __global__ void __launch_bounds__(256) pr_b_k(int64_t n, const int64_t* __restri
                                               const int32_t* __restrict__ partner, const long long* __restrict__ pw,
                                               const long long* __restrict__ deg, const DevState* st,
                                               int32_t* __restrict__ labels, int* changed, BatchCtx bc,
-                                              const unsigned char* __restrict__ flag) {
+                                              const unsigned char* __restrict__ flag, PrLong longs) {
   __shared__ int32_t s_list[8][kPrBStage];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int32_t* sl = s_list[wid];
@@ -490,6 +507,10 @@ __global__ void __launch_bounds__(256) pr_b_k(int64_t n, const int64_t* __restri
     const long long cvw = pw[v], dv = deg[v], dp = deg[p];
     // walk list s, search list l (s the shorter; ties: walk v's)
     const bool swap = pe - pb < ve - vb;
+    if (longs.v && (swap ? pe - pb : ve - vb) > kPrLongMin) {  // pr_b_long_k
+      if (lane == 0) longs.v[atomicAdd(longs.n, 1)] = (int32_t)v;
+      continue;
+    }
     const int64_t sb = swap ? pb : vb, se = swap ? pe : ve, lb = swap ? vb : pb, le = swap ? ve : pe;
     const bool staged = le - lb <= kPrBStage;
     if (staged)
@@ -533,19 +554,86 @@ __global__ void __launch_bounds__(256) pr_b_k(int64_t n, const int64_t* __restri
   }
 }
 
+// The pairs pr_b_k left out (the shorter list's entries over the threads of the blocks that
+// share the pair, a binary search of the longer one each); then the decision.
+template <typename WT>
+__global__ void __launch_bounds__(256) pr_b_long_k(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                   const WT* __restrict__ w, const int32_t* __restrict__ partner,
+                                                   const long long* __restrict__ pw,
+                                                   const long long* __restrict__ deg, PrLong longs) {
+  const int n = *longs.n, lane = threadIdx.x & 31;
+  const GridShare G(n);
+  for (int i = G.first; i < n; i += G.step) {
+    const int32_t v = longs.v[i], p = partner[v];
+    const int64_t vb = off[v], ve = off[v + 1], pb = off[p], pe = off[p + 1];
+    const long long cvw = pw[v], dv = deg[v], dp = deg[p];
+    const bool swap = pe - pb < ve - vb;
+    const int64_t sb = swap ? pb : vb, se = swap ? pe : ve, lb = swap ? vb : pb, le = swap ? ve : pe;
+    bool pr3 = false;
+    long long sum = 0;
+    for (int64_t e = sb + (int64_t)G.part * blockDim.x + threadIdx.x; e < se; e += (int64_t)G.parts * blockDim.x) {
+      const int u = adj[e];
+      int64_t lo = lb, hi = le;
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (adj[mid] < u) lo = mid + 1;
+        else hi = mid;
+      }
+      if (lo < le && adj[lo] == u) {
+        const long long cs = (long long)w[e], cl = (long long)w[lo];
+        const long long cvu = swap ? cl : cs, cwu = swap ? cs : cl;  // c(v, u), c(p, u)
+        if (dv <= 2 * (cvw + cvu) && dp <= 2 * (cvw + cwu)) pr3 = true;
+        sum += cvu < cwu ? cvu : cwu;
+      }
+    }
+    pr3 = __any_sync(0xffffffffu, pr3);
+    sum = warp_sum(sum);
+    if (lane == 0) {
+      if (pr3) atomicOr(longs.pr3 + i, 1);
+      if (sum) atomicAdd(longs.sum + i, (unsigned long long)sum);
+    }
+  }
+}
+
+__global__ void pr_b_long_done_k(const int32_t* __restrict__ partner, const long long* __restrict__ pw,
+                                 const DevState* st, int32_t* __restrict__ labels, int* changed, PrLong longs) {
+  const int n = *longs.n;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int32_t v = longs.v[i];
+    if (longs.pr3[i] || pw[v] + (long long)longs.sum[i] >= st->lambda_hat) {
+      labels[partner[v]] = v;
+      if (changed) atomicOr(changed, 1);
+    }
+  }
+}
+
 void pr_pass_b(const GraphView& g, const int32_t* partner, const long long* pw, const long long* deg,
                const DevState* st, int32_t* labels, int* changed, cudaStream_t s, const BatchCtx* bcp,
-               const unsigned char* flag) {
+               const unsigned char* flag, const PrLong& longs) {
   BatchCtx bc = bcp ? *bcp : BatchCtx{};
+  if (longs.v) {
+    const int64_t cap = pr_long_cap(g.nnz);
+    VC_CUDA(cudaMemsetAsync(longs.n, 0, sizeof(int), s));
+    VC_CUDA(cudaMemsetAsync(longs.sum, 0, sizeof(unsigned long long) * cap, s));
+    VC_CUDA(cudaMemsetAsync(longs.pr3, 0, sizeof(int) * cap, s));
+  }
   if (!bc.gid) iota(labels, g.n, s);
   int grid = grid_for(g.n, 8, kSMs * 16);
   if (g.wbytes == 4)
     pr_b_k<int32_t><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const int32_t*)g.w, partner, pw, deg, st, labels,
-                                         changed, bc, flag);
+                                         changed, bc, flag, longs);
   else
     pr_b_k<long long><<<grid, 256, 0, s>>>(g.n, g.off, g.adj, (const long long*)g.w, partner, pw, deg, st, labels,
-                                           changed, bc, flag);
+                                           changed, bc, flag, longs);
   count_launch();
+  if (longs.v) {
+    if (g.wbytes == 4)
+      pr_b_long_k<int32_t><<<kSMs * 4, 256, 0, s>>>(g.off, g.adj, (const int32_t*)g.w, partner, pw, deg, longs);
+    else
+      pr_b_long_k<long long><<<kSMs * 4, 256, 0, s>>>(g.off, g.adj, (const long long*)g.w, partner, pw, deg, longs);
+    pr_b_long_done_k<<<1, 256, 0, s>>>(partner, pw, st, labels, changed, longs);
+    count_launch(2);
+  }
   VC_CHECK_LAUNCH();
 }
 

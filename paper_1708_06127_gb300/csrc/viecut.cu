@@ -309,7 +309,7 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
                     W.parent.as<int32_t>(), lab, &W.ctr()->changed, s);
         } else {
           pr_pass_b(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), st, lab,
-                    &W.ctr()->changed, s, nullptr, few ? flag : nullptr);
+                    &W.ctr()->changed, s, nullptr, few ? flag : nullptr, W.pr_long(G.nnz));
         }
         if (W.flags_ok) flag_clear(G.n, flag, bit, s);
         W.pr_new[pass] = 0;
