@@ -64,9 +64,16 @@ struct Bins {
   int h_mid = 0, h_block = 0, h_global = 0, h_maxdeg = 0, h_small = 0, h_reg = 0;  // host copies
 };
 
+// Binning only the marked vertices: the others keep their label (out[v] = in[v]); the marks
+// are cleared.
+struct KeepLabels {
+  unsigned char* mark = nullptr;
+  const int32_t* in = nullptr;
+  int32_t* out = nullptr;
+};
 // list_n not null: bins the vertices list[0, *list_n) (at most g.n of them) instead of all.
 void bins_build(const GraphView& g, Bins& b, cudaStream_t s, const int32_t* list = nullptr,
-                const int* list_n = nullptr);
+                const int* list_n = nullptr, const KeepLabels& keep = KeepLabels());
 
 // Scratch for the global-class tables: blocks x cap slots.
 struct GlobalTables {
@@ -112,8 +119,10 @@ void async_wave_members(int64_t n, const unsigned char* wave_of, int k, int32_t*
 void async_apply(const int32_t* list, const int* count, int64_t cap, const int32_t* fresh, int32_t* lab,
                  unsigned char* joined, int32_t* took, cudaStream_t s);
 
-// *changed += the number of v with lab_out[v] != lab_in[v] (lab_in null: the identity).
-void count_changed(const int32_t* lab_in, const int32_t* lab_out, int64_t n, long long* changed, cudaStream_t s);
+// *changed += the number of v with lab_out[v] != lab_in[v] (lab_in null: the identity); with
+// mark (n bytes; may be null) the neighbours of those vertices are marked 1.
+void count_changed(const GraphView& g, const int32_t* lab_in, const int32_t* lab_out, long long* changed,
+                   unsigned char* mark, cudaStream_t s);
 
 // One synchronous label-propagation round; lab_in == nullptr means the identity
 // labelling (first round of a level).  hv: the level's tie-break table.
