@@ -68,24 +68,35 @@ __device__ __forceinline__ DegArg block_min(DegArg x) {
   return x;  // valid in thread 0
 }
 
-__global__ void min_partial_k(const long long* __restrict__ deg, int64_t n, long long* __restrict__ partial) {
+// Each block's minimum, and by the last block to finish the minimum of those with the bound
+// (a launch fewer than a kernel for each).
+constexpr int kMinBlocks = 512;
+__global__ void __launch_bounds__(256) min_deg_k(const long long* __restrict__ deg, int64_t n, long long* partial,
+                                                 unsigned* done, DevState* st, int initial) {
+  __shared__ bool s_last;
   DegArg best{LLONG_MAX, LLONG_MAX};
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     DegArg c{deg[v], v};
     if (deg_less(c, best)) best = c;
   }
   best = block_min<256>(best);
-  if (threadIdx.x == 0) { partial[2 * blockIdx.x] = best.d; partial[2 * blockIdx.x + 1] = best.v; }
-}
-
-__global__ void min_final_k(const long long* __restrict__ partial, int nb, DevState* st, int initial) {
-  DegArg best{LLONG_MAX, LLONG_MAX};
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    DegArg c{partial[2 * b], partial[2 * b + 1]};
+  if (threadIdx.x == 0) {
+    partial[2 * blockIdx.x] = best.d;
+    partial[2 * blockIdx.x + 1] = best.v;
+    __threadfence();
+    s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  best = DegArg{LLONG_MAX, LLONG_MAX};
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+    DegArg c{__ldcg(partial + 2 * b), __ldcg(partial + 2 * b + 1)};
     if (deg_less(c, best)) best = c;
   }
   best = block_min<256>(best);
   if (threadIdx.x == 0) {
+    *done = 0;  // for the next call on this stream
     st->dmin = best.d;
     st->argmin = best.v;
     if (initial) {
@@ -102,21 +113,20 @@ __global__ void min_final_k(const long long* __restrict__ partial, int nb, DevSt
   }
 }
 
-void bound_update_impl(const long long* deg, int64_t n, DevState* st, long long* partial, int initial,
+static void bound_impl(const long long* deg, int64_t n, DevState* st, long long* partial, unsigned* done, int initial,
                        cudaStream_t s) {
-  int nb = grid_for(n, 256, 512);
-  min_partial_k<<<nb, 256, 0, s>>>(deg, n, partial);
-  min_final_k<<<1, 256, 0, s>>>(partial, nb, st, initial);
-  count_launch(2);
+  min_deg_k<<<grid_for(n, 256, kMinBlocks), 256, 0, s>>>(deg, n, partial, done, st, initial);
+  count_launch();
   VC_CHECK_LAUNCH();
 }
 
-void bound_update(const long long* deg, int64_t n, DevState* st, long long* partial, cudaStream_t s) {
-  bound_update_impl(deg, n, st, partial, 0, s);
+void bound_update(const long long* deg, int64_t n, DevState* st, long long* partial, unsigned* done,
+                  cudaStream_t s) {
+  bound_impl(deg, n, st, partial, done, 0, s);
 }
 
-void bound_init(const long long* deg, int64_t n, DevState* st, long long* partial, cudaStream_t s) {
-  bound_update_impl(deg, n, st, partial, 1, s);
+void bound_init(const long long* deg, int64_t n, DevState* st, long long* partial, unsigned* done, cudaStream_t s) {
+  bound_impl(deg, n, st, partial, done, 1, s);
 }
 
 __global__ void snapshot_k(const int32_t* __restrict__ cur1, int64_t n1, unsigned char* __restrict__ side1,
@@ -191,14 +201,15 @@ void side_bits2(const int32_t* orig_map, int64_t n, const unsigned char* side1, 
   VC_CHECK_LAUNCH();
 }
 
-__global__ void trace_push_k(DevState* st, TraceStep* trace, int cap, int kind, int level) {
+__global__ void trace_push_k(DevState* st, TraceStep* trace, int cap, int kind, int level, long long n) {
+  if (n >= 0) st->n = n;
   int i = st->trace_len;
   if (i < cap) trace[i] = TraceStep{kind, level, st->n, st->nnz, st->lambda_hat};
   st->trace_len = i + 1;
 }
 
-void trace_push(DevState* st, TraceStep* trace, int cap, int kind, int level, cudaStream_t s) {
-  trace_push_k<<<1, 1, 0, s>>>(st, trace, cap, kind, level);
+void trace_push(DevState* st, TraceStep* trace, int cap, int kind, int level, int64_t n, cudaStream_t s) {
+  trace_push_k<<<1, 1, 0, s>>>(st, trace, cap, kind, level, n);
   count_launch();
   VC_CHECK_LAUNCH();
 }

@@ -101,7 +101,6 @@ __global__ void build_pairs_long_k(const int64_t* __restrict__ off, const int32_
 
 void build_pairs(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int bits, int64_t pairs,
                  const LongLists& longs, unsigned long long* keys, long long* vals, cudaStream_t s) {
-  if (longs.item) VC_CUDA(cudaMemsetAsync(longs.n, 0, sizeof(int), s));
   const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
   if (pairs <= 2 * g.n)
     build_pairs_k<1><<<grid_for(g.n, 256, kSMs * 8), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals, longs);
@@ -1179,7 +1178,7 @@ __global__ void giant_count_k(int ng, const int32_t* __restrict__ glist, const l
     dcount[glist[j]] = (int32_t)(hpos[gstart[j + 1]] - hpos[gstart[j]]);
 }
 
-static void giant_merge(const GiantScratch& G, int64_t c, const long long* cbase, int32_t* seg_key,
+static void giant_merge(GiantScratch G, int64_t c, const long long* cbase, int32_t* seg_key,
                         long long* seg_val, int32_t* dcount, long long* scan_scr, cudaStream_t s) {
   VC_CUDA(cudaMemsetAsync(G.gcount, 0, sizeof(int), s));
   giant_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, G.gcount, G.glist, G.gT);
@@ -1259,18 +1258,15 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
                    int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, bool big, bool sort_first,
                    const GiantScratch* giant, int32_t* blist, int* blist_n, cudaStream_t s, const SparseCtx* sp,
                    const LongLists& longs) {
-  exclusive_scan<int, long long>(ccount, cbase, c, cbase + c, cs.scan_scr, s);
-  VC_CUDA(cudaMemcpyAsync(cursor, cbase, sizeof(long long) * c, cudaMemcpyDeviceToDevice, s));
+  exclusive_scan<int, long long>(ccount, cbase, c, cbase + c, cs.scan_scr, s, cursor);
   const int gv = grid_for(g.n, 256, kSMs * 8), gc = grid_for(c, 8, kSMs * 16);
   const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
-  if (longs.item) VC_CUDA(cudaMemsetAsync(longs.n, 0, sizeof(int), s));
   cluster_scatter_k<<<gv, 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, cursor, seg_key, seg_val, longs);
   if (longs.item) {
     cluster_scatter_long_k<<<kSMs * 4, 256, 0, s>>>(g.off, cs.cnt, in, seg_key, seg_val, longs);
     count_launch();
   }
   if (sp) {
-    VC_CUDA(cudaMemsetAsync(sp->list_n, 0, sizeof(int), s));
     warp_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, sp->list, sp->list_n);
     count_launch();
   }
@@ -1280,8 +1276,8 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
   VC_CHECK_LAUNCH();
   if (big) {
     // the clusters of kMergeMax < T <= kMergeBlockMax pairs listed first, so that the
-    // blocks visit only them (blist: n ints no longer needed once the scatter ran)
-    VC_CUDA(cudaMemsetAsync(blist_n, 0, sizeof(int), s));
+    // blocks visit only them (blist: n ints no longer needed once the scatter ran; its count,
+    // like the other lists' here, starts from zero)
     block_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, blist, blist_n);
     const int smem = merge_block_smem();
     cluster_merge_block_k<<<kSMs, 256, smem, s>>>(c, cbase, seg_key, seg_val, ccount, blist, blist_n);
@@ -1290,18 +1286,18 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
   }
   if (giant && giant->ngiant > 0) giant_merge(*giant, c, cbase, seg_key, seg_val, ccount, cs.scan_scr, s);
   if (sp) sparse_finish_degrees(g, cid, sp->sdeg, ccount, sp->clean, c, s);
-  exclusive_scan<int, long long>(ccount, (long long*)coff, c, (long long*)coff + c, cs.scan_scr, s);
-  if (longs.item) VC_CUDA(cudaMemsetAsync(longs.n, 0, sizeof(int), s));
+  exclusive_scan<int, long long>(ccount, (long long*)coff, c, (long long*)coff + c, cs.scan_scr, s, nullptr, nnz_dev);
+  LongLists place = longs;
+  place.n = longs.n + 1;  // a count of its own, the items no longer needed
   cluster_place_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, coff, seg_key, seg_val, cadj, cw, csrc,
-                                                               sp ? sp->clean : nullptr, longs);
+                                                               sp ? sp->clean : nullptr, place);
   if (longs.item) {
-    cluster_place_long_k<<<kSMs * 4, 256, 0, s>>>(cbase, coff, seg_key, seg_val, cadj, cw, csrc, longs);
+    cluster_place_long_k<<<kSMs * 4, 256, 0, s>>>(cbase, coff, seg_key, seg_val, cadj, cw, csrc, place);
     count_launch();
   }
   count_launch();
   VC_CHECK_LAUNCH();
   if (sp) sparse_copy(g, sp->cidm, sp->sdeg, sp->dirty, coff, cadj, cw, csrc, s);
-  VC_CUDA(cudaMemcpyAsync(nnz_dev, coff + c, sizeof(long long), cudaMemcpyDeviceToDevice, s));
 }
 
 

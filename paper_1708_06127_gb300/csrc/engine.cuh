@@ -1,6 +1,7 @@
 // Host-side engine pieces shared by the single-graph driver and the batch driver:
 // grow-only device buffers and the workspace of device arrays one run needs.
 #pragma once
+#include <stddef.h>
 #include <string.h>
 
 #include <algorithm>
@@ -62,15 +63,26 @@ struct Buf {
 
 struct Counters {
   int c;
+  // from here to the end of nlong cleared by every contraction before it counts
   int maxt;  // largest pre-merged pair count of one cluster
   long long pairs;
-  int changed;
-  int ngiant;         // clusters of more than kMergeBlockMax pairs
-  long long gpairs;   // their pairs
+  long long gpairs;   // the pairs of clusters of more than kMergeBlockMax pairs
+  int ngiant;         // those clusters
   int blist_n;        // clusters listed for the block-level merge
-  int nlist;          // vertices or clusters listed (flag_list, the sparse contraction's merge)
-  int nlong;          // lists left to a grid's blocks to share (LongLists, PrLong)
+  int nlist;          // clusters listed for the sparse contraction's merge
+  int nlong[2];       // lists left to a grid's blocks to share (LongLists)
+  int nflag;          // vertices listed by flag_list
+  int nprlong;        // pairs listed by pass B (PrLong)
   int nab[2];         // vertices whose list is new for pass A, for pass B
+  int changed;
+};
+
+// What the host reads at its decision points, in one copy.
+struct Record {
+  DevState st;
+  Counters c;
+  int bins[8], dbins[8];  // Bins::counts
+  unsigned blocks_done;   // bound_init, bound_update
 };
 
 enum Phase { kPhLP = 0, kPhContract, kPhPR, kPhNOI, kPhOther, kPhCount };
@@ -80,7 +92,7 @@ struct Workspace {
   cudaStream_t s = nullptr;
   // vertex-sized
   Buf deg, labA, labB, map0, cidT, cur1, side1, flags, rank, cnt, pos, scan64, scan32, hv;
-  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, longV, longAt, longHit, slist, rlist, mlist, blist, glist, bl1, bcounts, noi_r;
+  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, longV, longAt, longHit, slist, rlist, mlist, blist, glist, bl1, noi_r;
   // entry-sized
   Buf tmpK, tmpV, cmpK, cmpV;
   // pair-sized
@@ -93,7 +105,8 @@ struct Workspace {
   // exact step
   Buf M0, M1, curK, sideK;
   // state
-  Buf state, trace, partial, counters;
+  Buf state, trace, partial;  // state: a Record
+  Record* h_rec = nullptr;    // page-locked
   DevState* h_state = nullptr;
   Counters* h_counters = nullptr;
   int trace_cap = 4096;
@@ -110,21 +123,21 @@ struct Workspace {
   long long ct_bytes_acc = 0, pm_bytes_acc = 0, ct_count = 0;
 
   Workspace() {
-    VC_CUDA(cudaMallocHost(&h_state, sizeof(DevState)));
-    VC_CUDA(cudaMallocHost(&h_counters, sizeof(Counters)));
-    state.ensure(sizeof(DevState));
+    VC_CUDA(cudaMallocHost(&h_rec, sizeof(Record)));
+    memset((void*)h_rec, 0, sizeof(Record));
+    h_state = &h_rec->st;
+    h_counters = &h_rec->c;
+    state.ensure(sizeof(Record));
     trace.ensure_n<TraceStep>(trace_cap);
     partial.ensure_n<long long>(2 * 1024);
-    counters.ensure(sizeof(Counters));
-    bcounts.ensure_n<int>(8);
   }
   ~Workspace() {
-    if (h_state) cudaFreeHost(h_state);
-    if (h_counters) cudaFreeHost(h_counters);
+    if (h_rec) cudaFreeHost(h_rec);
     for (auto e : ev_pool) cudaEventDestroy(e);
   }
-  DevState* st() { return state.as<DevState>(); }
-  Counters* ctr() { return counters.as<Counters>(); }
+  Record* rec() { return state.as<Record>(); }
+  DevState* st() { return &rec()->st; }
+  Counters* ctr() { return &rec()->c; }
 
   void ensure_vertices(int64_t n) {
     deg.ensure_n<long long>(n);
@@ -166,9 +179,15 @@ struct Workspace {
 
   void sync() { VC_CUDA(cudaStreamSynchronize(s)); }
   void read_state() {
-    VC_CUDA(cudaMemcpyAsync(h_state, st(), sizeof(DevState), cudaMemcpyDeviceToHost, s));
-    VC_CUDA(cudaMemcpyAsync(h_counters, ctr(), sizeof(Counters), cudaMemcpyDeviceToHost, s));
+    VC_CUDA(cudaMemcpyAsync(h_rec, rec(), sizeof(Record), cudaMemcpyDeviceToHost, s));
     sync();
+  }
+  // The record of a run's start: everything zero but the shape.
+  void write_state(int64_t n, int64_t nnz) {
+    memset((void*)h_rec, 0, sizeof(Record));
+    h_state->n = n;
+    h_state->nnz = nnz;
+    VC_CUDA(cudaMemcpyAsync(rec(), h_rec, sizeof(Record), cudaMemcpyHostToDevice, s));
   }
 
   // ---------------------------------------------------------------- timing
@@ -264,12 +283,10 @@ struct Workspace {
   Bins bins;
   bool bins_valid = false;
 
-  // Reads the class counts of bins b (and counts[6] into *extra when given) and sizes
-  // the global-class tables for its longest list.
-  void read_bins(Bins& b, int* extra = nullptr) {
-    int hc[7];
-    VC_CUDA(cudaMemcpyAsync(hc, b.counts, (extra ? 7 : 6) * sizeof(int), cudaMemcpyDeviceToHost, s));
-    sync();
+  // Takes the class counts of bins b from the record just read (and counts[6] into *extra
+  // when given) and sizes the global-class tables for its longest list.
+  void take_bins(Bins& b, int* extra = nullptr) {
+    const int* hc = b.counts == rec()->bins ? h_rec->bins : h_rec->dbins;
     b.h_mid = hc[0];
     b.h_block = hc[1];
     b.h_global = hc[2];
@@ -288,16 +305,23 @@ struct Workspace {
       gt.blocks = blocks;
     }
   }
+  void read_bins(Bins& b, int* extra = nullptr) {
+    read_state();
+    take_bins(b, extra);
+  }
 
-  void build_bins(const GraphView& g) {
+  void launch_bins(const GraphView& g) {
     bins.small_list = slist.as<int32_t>();
     bins.reg_list = rlist.as<int32_t>();
     bins.mid_list = mlist.as<int32_t>();
     bins.block_list = blist.as<int32_t>();
     bins.global_list = glist.as<int32_t>();
     bins.bail_list = bl1.as<int32_t>();
-    bins.counts = bcounts.as<int>();
+    bins.counts = rec()->bins;
     bins_build(g, bins, s);
+  }
+  void build_bins(const GraphView& g) {
+    launch_bins(g);
     read_bins(bins);
     bins_valid = true;
   }
@@ -323,8 +347,8 @@ struct Workspace {
                        prflag2.as<unsigned char>()};
       int32_t* list = prlist.ensure_n<int32_t>(nf);
       pr_carry(nf, cid, sdeg.as<int32_t>(), sdirty.as<unsigned char>(), from, to, h.n, s);
-      flag_list(h.n, to.flag, kListNew, list, &ctr()->nlist, ctr()->nab, s);
-      pr_partners(h, to.partner, to.pw, to.deg, s, list, &ctr()->nlist, to.flag);
+      flag_list(h.n, to.flag, kListNew, list, &ctr()->nflag, ctr()->nab, s);
+      pr_partners(h, to.partner, to.pw, to.deg, s, list, &ctr()->nflag, to.flag);
       partner.swap(partner2);
       pw.swap(pw2);
       deg.swap(deg2);
@@ -346,7 +370,7 @@ struct Workspace {
     L.v = longV.ensure_n<int32_t>(cap);
     L.sum = longAt.ensure_n<unsigned long long>(cap);
     L.pr3 = longHit.ensure_n<int>(cap);
-    L.n = &ctr()->nlong;
+    L.n = &ctr()->nprlong;
     return L;
   }
   void pr_new_read() {
@@ -361,7 +385,7 @@ struct Workspace {
   // dbins holds their bins.
   bool last_sparse = false;  // the last contraction was a sparse one
   Bins dbins;
-  Buf smflag, scidm, sdirty, sdeg, sclean, sdlist, dsl, drl, dml, dbl, dgl, dbail, dcounts;
+  Buf smflag, scidm, sdirty, sdeg, sclean, sdlist, dsl, drl, dml, dbl, dgl, dbail;
   // dbins' lists, for at most n listed vertices
   void prepare_dbins(int64_t n) {
     dbins.small_list = dsl.ensure_n<int32_t>(n);
@@ -370,7 +394,7 @@ struct Workspace {
     dbins.block_list = dbl.ensure_n<int32_t>(n);
     dbins.global_list = dgl.ensure_n<int32_t>(n);
     dbins.bail_list = dbail.ensure_n<int32_t>(n);
-    dbins.counts = dcounts.ensure_n<int>(8);
+    dbins.counts = rec()->dbins;
   }
 
   bool mark_sparse(const GraphView& g, const int32_t* labels, const int32_t* cid) {
@@ -569,14 +593,10 @@ struct Workspace {
     cudaEvent_t e0 = mark();
     emit_cross(g, B, gt, cid_out, po, cs.cnt, s, tune);
     if (timing && !sparse) pm_spans.push_back({e0, mark()});  // the whole graph's pre-merge only
-    VC_CUDA(cudaMemsetAsync(&ctr()->maxt, 0, sizeof(int), s));
-    VC_CUDA(cudaMemsetAsync(&ctr()->pairs, 0, sizeof(long long), s));
-    VC_CUDA(cudaMemsetAsync(&ctr()->ngiant, 0, sizeof(int), s));
-    VC_CUDA(cudaMemsetAsync(&ctr()->gpairs, 0, sizeof(long long), s));
+    VC_CUDA(cudaMemsetAsync(&ctr()->maxt, 0, offsetof(Counters, nflag) - offsetof(Counters, maxt), s));
     cluster_stats(g.n, ccount, &ctr()->maxt, &ctr()->pairs, &ctr()->ngiant, &ctr()->gpairs, s);
     if (timing) ct_spans.push_back({t0, mark()});
-    VC_CUDA(cudaMemcpyAsync(h_counters, ctr(), sizeof(Counters), cudaMemcpyDeviceToHost, s));
-    sync();
+    read_state();
     cudaEvent_t t1 = mark();
     const int64_t c = h_counters->c;
     const int64_t P = h_counters->pairs;
@@ -601,7 +621,7 @@ struct Workspace {
     if (ng) {
       longs.item = longV.ensure_n<int32_t>(long_list_cap(P));
       longs.at = longAt.ensure_n<long long>(long_list_cap(P));
-      longs.n = &ctr()->nlong;
+      longs.n = ctr()->nlong;
     }
     if (2 * GP <= P || sparse) {
       long long* cbase = pos.as<long long>();  // n + 1 >= c + 1 entries

@@ -216,7 +216,8 @@ struct GridShare {
 // Lists of more than kLongList pieces are left by the kernels that copy a list with a warp
 // to a second one in which the grid's blocks share them (a hub that absorbed many vertices
 // holds a tenth of a graph's entries: 3 ms by one warp).  item[*n] receives the vertex or
-// cluster, at[*n] where its list goes; both hold long_list_cap(pairs) entries.
+// cluster, at[*n] where its list goes; both hold long_list_cap(pairs) entries.  A contraction
+// gets two counts, n[0] and n[1], zero.
 constexpr int kLongList = 4096;
 inline int64_t long_list_cap(int64_t pairs) { return pairs / kLongList + 1; }
 struct LongLists {
@@ -290,10 +291,11 @@ void reduce_pairs(const unsigned long long* keys, const long long* vals, int64_t
 // ------------------------------------------------------------------ bounds
 void degrees(const GraphView& g, long long* deg, cudaStream_t s);
 // Minimum degree with smallest argmin; if below st->lambda_hat the bound improves
-// and st->improved is set (st->argmin/dmin always written).  partial: >= 1024 slots.
-void bound_update(const long long* deg, int64_t n, DevState* st, long long* partial, cudaStream_t s);
+// and st->improved is set (st->argmin/dmin always written).  partial: 1024 slots; *done
+// (a count of blocks) is zero before and after.
+void bound_update(const long long* deg, int64_t n, DevState* st, long long* partial, unsigned* done, cudaStream_t s);
 // Initial bound on the input graph: lambda-hat = minimum degree, best = its argmin.
-void bound_init(const long long* deg, int64_t n, DevState* st, long long* partial, cudaStream_t s);
+void bound_init(const long long* deg, int64_t n, DevState* st, long long* partial, unsigned* done, cudaStream_t s);
 // On improvement: side1[j] = (cur1[j] == st->argmin) and best_kind = 1.
 void snapshot_side(const int32_t* cur1, int64_t n1, unsigned char* side1, DevState* st, cudaStream_t s);
 void compose_map(int32_t* cur1, int64_t n1, const int32_t* cid, cudaStream_t s);
@@ -301,7 +303,8 @@ void iota(int32_t* x, int64_t n, cudaStream_t s);
 // Final side bitmap of the input vertices (see side_of in bound.cu).
 void side_bits2(const int32_t* orig_map, int64_t n, const unsigned char* side1, const int32_t* cur1,
                 const unsigned char* sideK, const DevState* st, unsigned long long* bits, cudaStream_t s);
-void trace_push(DevState* st, TraceStep* trace, int cap, int kind, int level, cudaStream_t s);
+// n >= 0: the graph's vertex count, stored in the state first.
+void trace_push(DevState* st, TraceStep* trace, int cap, int kind, int level, int64_t n, cudaStream_t s);
 
 // ------------------------------------------------------------------ Padberg-Rinaldi
 // Degree, partner and partner weight of every vertex, or of the listed ones only (list,

@@ -1,4 +1,6 @@
 // Device-wide exclusive scan and stable LSD radix sort (reduce-then-scan design).
+#include <utility>
+
 #include "prims.cuh"
 
 namespace vc {
@@ -41,7 +43,8 @@ __global__ void scan_reduce_k(const In* __restrict__ in, int64_t n, Out* __restr
 
 // Single block: exclusive scan of partial[0..nb) in place; total to *total.
 template <typename Out>
-__global__ void scan_partials_k(Out* __restrict__ partial, int64_t nb, Out* __restrict__ total) {
+__global__ void scan_partials_k(Out* __restrict__ partial, int64_t nb, Out* __restrict__ total,
+                                Out* __restrict__ total2) {
   __shared__ Out wsum[32];
   __shared__ Out carry_s;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -67,11 +70,12 @@ __global__ void scan_partials_k(Out* __restrict__ partial, int64_t nb, Out* __re
     __syncthreads();
   }
   if (threadIdx.x == 0 && total) *total = carry_s;
+  if (threadIdx.x == 0 && total2) *total2 = carry_s;
 }
 
 template <typename In, typename Out>
 __global__ void scan_apply_k(const In* __restrict__ in, Out* __restrict__ out, int64_t n,
-                             const Out* __restrict__ partial) {
+                             const Out* __restrict__ partial, Out* __restrict__ out2) {
   __shared__ Out tile[kScanTile];
   __shared__ Out wsum[kScanThreads / 32];
   int64_t base = (int64_t)blockIdx.x * kScanTile;
@@ -107,29 +111,93 @@ __global__ void scan_apply_k(const In* __restrict__ in, Out* __restrict__ out, i
   for (int i = 0; i < kScanItems; ++i) {
     int idx = i * kScanThreads + threadIdx.x;
     int64_t k = base + idx;
-    if (k < n) out[k] = tile[idx];
+    if (k < n) {
+      out[k] = tile[idx];
+      if (out2) out2[k] = tile[idx];
+    }
+  }
+}
+
+// At most kScanOneMax elements: one block, tile after tile.  At 16,384 elements a launch of
+// about 4 us takes the place of three of 2 to 3 us each and the gaps between them; above,
+// one block would be the longer way.
+constexpr int64_t kScanOneMax = 16384;
+constexpr int kScanOneItems = 4;
+template <typename In, typename Out>
+__global__ void __launch_bounds__(1024) scan_one_k(const In* __restrict__ in, Out* __restrict__ out, int n,
+                                                   Out* __restrict__ total, Out* __restrict__ out2,
+                                                   Out* __restrict__ total2) {
+  __shared__ Out tile[1024 * kScanOneItems];
+  __shared__ Out wsum[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  Out carry = 0;  // the same in every thread
+  for (int base = 0; base < n; base += 1024 * kScanOneItems) {
+#pragma unroll
+    for (int i = 0; i < kScanOneItems; ++i) {
+      const int k = i * 1024 + threadIdx.x;
+      tile[k] = base + k < n ? (Out)in[base + k] : (Out)0;
+    }
+    __syncthreads();
+    Out loc[kScanOneItems], sum = 0;
+#pragma unroll
+    for (int i = 0; i < kScanOneItems; ++i) {
+      loc[i] = sum;
+      sum += tile[threadIdx.x * kScanOneItems + i];
+    }
+    const Out inc = warp_incl_scan(sum);
+    if (lane == 31) wsum[wid] = inc;
+    __syncthreads();
+    const Out v = warp_incl_scan(wsum[lane]);  // by every warp: the sums of warps up to its lane
+    const Out before = carry + __shfl_sync(0xffffffffu, v, wid) - __shfl_sync(0xffffffffu, inc, 31) + inc - sum;
+    carry += __shfl_sync(0xffffffffu, v, 31);
+#pragma unroll
+    for (int i = 0; i < kScanOneItems; ++i) tile[threadIdx.x * kScanOneItems + i] = before + loc[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kScanOneItems; ++i) {
+      const int k = i * 1024 + threadIdx.x;
+      if (base + k < n) {
+        out[base + k] = tile[k];
+        if (out2) out2[base + k] = tile[k];
+      }
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    if (total) *total = carry;
+    if (total2) *total2 = carry;
   }
 }
 
 int64_t scan_scratch_elems(int64_t n) { return (n + kScanTile - 1) / kScanTile + 1; }
 
 template <typename In, typename Out>
-void exclusive_scan(const In* in, Out* out, int64_t n, Out* total, Out* scratch, cudaStream_t s) {
+void exclusive_scan(const In* in, Out* out, int64_t n, Out* total, Out* scratch, cudaStream_t s, Out* out2,
+                    Out* total2) {
   if (n <= 0) {
     if (total) VC_CUDA(cudaMemsetAsync(total, 0, sizeof(Out), s));
+    if (total2) VC_CUDA(cudaMemsetAsync(total2, 0, sizeof(Out), s));
+    return;
+  }
+  if (n <= kScanOneMax) {
+    scan_one_k<In, Out><<<1, 1024, 0, s>>>(in, out, (int)n, total, out2, total2);
+    count_launch();
+    VC_CHECK_LAUNCH();
     return;
   }
   int64_t nb = (n + kScanTile - 1) / kScanTile;
   scan_reduce_k<In, Out><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, scratch);
-  scan_partials_k<Out><<<1, 1024, 0, s>>>(scratch, nb, total);
-  scan_apply_k<In, Out><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, scratch);
+  scan_partials_k<Out><<<1, 1024, 0, s>>>(scratch, nb, total, total2);
+  scan_apply_k<In, Out><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, scratch, out2);
   count_launch(3);
   VC_CHECK_LAUNCH();
 }
 
-template void exclusive_scan<int, long long>(const int*, long long*, int64_t, long long*, long long*, cudaStream_t);
-template void exclusive_scan<long long, long long>(const long long*, long long*, int64_t, long long*, long long*, cudaStream_t);
-template void exclusive_scan<int, int>(const int*, int*, int64_t, int*, int*, cudaStream_t);
+template void exclusive_scan<int, long long>(const int*, long long*, int64_t, long long*, long long*, cudaStream_t,
+                                             long long*, long long*);
+template void exclusive_scan<long long, long long>(const long long*, long long*, int64_t, long long*, long long*,
+                                                   cudaStream_t, long long*, long long*);
+template void exclusive_scan<int, int>(const int*, int*, int64_t, int*, int*, cudaStream_t, int*, int*);
 
 // ------------------------------------------------------------------- radix sort
 constexpr int kRadixBits = 8;
@@ -231,29 +299,23 @@ __global__ void radix_scatter_k(const unsigned long long* __restrict__ keys,
   }
 }
 
-void radix_sort_pairs(unsigned long long* keys, long long* vals, unsigned long long* keys_alt,
-                      long long* vals_alt, int64_t n, int bits, long long* hist, cudaStream_t s) {
+void radix_sort_pairs(unsigned long long*& keys, long long*& vals, unsigned long long*& keys_alt,
+                      long long*& vals_alt, int64_t n, int bits, long long* hist, cudaStream_t s) {
   if (n <= 1 || bits <= 0) return;
   int64_t nb = (n + kRTile - 1) / kRTile;
   long long* scan_scr = hist + nb * kBuckets;
-  unsigned long long *src_k = keys, *dst_k = keys_alt;
-  long long *src_v = vals, *dst_v = vals_alt;
   int passes = (bits + kRadixBits - 1) / kRadixBits;
   for (int p = 0; p < passes; ++p) {
     int shift = p * kRadixBits;
-    radix_hist_k<<<(unsigned)nb, kRThreads, 0, s>>>(src_k, n, shift, nb, hist);
+    radix_hist_k<<<(unsigned)nb, kRThreads, 0, s>>>(keys, n, shift, nb, hist);
     count_launch();
     VC_CHECK_LAUNCH();
     exclusive_scan<long long, long long>(hist, hist, nb * kBuckets, nullptr, scan_scr, s);
-    radix_scatter_k<<<(unsigned)nb, kRThreads, 0, s>>>(src_k, src_v, n, shift, nb, hist, dst_k, dst_v);
+    radix_scatter_k<<<(unsigned)nb, kRThreads, 0, s>>>(keys, vals, n, shift, nb, hist, keys_alt, vals_alt);
     count_launch();
     VC_CHECK_LAUNCH();
-    std::swap(src_k, dst_k);
-    std::swap(src_v, dst_v);
-  }
-  if (src_k != keys) {
-    VC_CUDA(cudaMemcpyAsync(keys, src_k, sizeof(unsigned long long) * n, cudaMemcpyDeviceToDevice, s));
-    VC_CUDA(cudaMemcpyAsync(vals, src_v, sizeof(long long) * n, cudaMemcpyDeviceToDevice, s));
+    std::swap(keys, keys_alt);
+    std::swap(vals, vals_alt);
   }
 }
 

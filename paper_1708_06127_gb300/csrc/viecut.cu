@@ -35,8 +35,6 @@ bool take_injected_alloc_failure() {
   return false;
 }
 
-__global__ void set_n_k(DevState* st, long long n) { st->n = n; }
-
 __global__ void validate_k(int64_t n, int64_t m, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                            const int32_t* __restrict__ w, int* err) {
   int bad = 0;
@@ -181,11 +179,7 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
   const unsigned long long launches0 = g_launches;
   W.reset_timing();
   cudaEvent_t t_start = W.mark();
-  DevState init{};
-  init.n = H.n;
-  init.nnz = H.m;
-  VC_CUDA(cudaMemcpyAsync(W.st(), &init, sizeof(DevState), cudaMemcpyHostToDevice, s));
-  VC_CUDA(cudaMemsetAsync(W.ctr(), 0, sizeof(Counters), s));
+  W.write_state(H.n, H.m);
   DevState* st = W.st();
   TraceStep* tr = W.trace.as<TraceStep>();
   const int tcap = W.trace_cap;
@@ -204,10 +198,16 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
 
   cudaEvent_t a = W.mark();
   degrees(G, W.deg.as<long long>(), s);
-  bound_init(W.deg.as<long long>(), G.n, st, W.partial.as<long long>(), s);
-  trace_push(st, tr, tcap, 0, 0, s);
+  bound_init(W.deg.as<long long>(), G.n, st, W.partial.as<long long>(), &W.rec()->blocks_done, s);
+  trace_push(st, tr, tcap, 0, 0, -1, s);
   W.span(kPhOther, a);
+  // the first level's bins with the same read
+  if (G.n > H.n0) W.launch_bins(G);
   W.read_state();
+  if (G.n > H.n0) {
+    W.take_bins(W.bins);
+    W.bins_valid = true;
+  }
 
   int level = 0;
   int slot = -1;          // coarse buffer holding G (-1: the input)
@@ -231,8 +231,6 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
     // the sparse contraction for Padberg-Rinaldi passes and for levels the last one did
     // not halve (most vertices keep their own label there)
     GraphView h = W.contract(G, labels, cid, dst, kind == 1 && H.correct, kind >= 2 || W.tune.mid_bail);
-    set_n_k<<<1, 1, 0, s>>>(st, h.n);
-    count_launch();
     if (!contracted) {
       n1 = h.n;
       iota(W.cur1.as<int32_t>(), n1, s);
@@ -251,10 +249,10 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
       // pass reads (the same scan of the changed lists)
       W.contracted_partners(G, fine.n, cid, had_partners);
       partners_ok = true;
-      bound_update(W.deg.as<long long>(), G.n, st, W.partial.as<long long>(), s);
+      bound_update(W.deg.as<long long>(), G.n, st, W.partial.as<long long>(), &W.rec()->blocks_done, s);
       snapshot_side(W.cur1.as<int32_t>(), n1, W.side1.as<unsigned char>(), st, s);
     }
-    trace_push(st, tr, tcap, kind, level, s);
+    trace_push(st, tr, tcap, kind, level, G.n, s);
     W.span(kPhOther, a1);
     W.read_state();
     W.pr_new_read();
@@ -264,8 +262,7 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
   };
 
   auto read_changed = [&]() -> int {
-    VC_CUDA(cudaMemcpyAsync(&W.h_counters->changed, &W.ctr()->changed, sizeof(int), cudaMemcpyDeviceToHost, s));
-    W.sync();
+    W.read_state();
     return W.h_counters->changed;
   };
 
@@ -276,7 +273,7 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
     // a graph the last level did not halve is weakly clustered: its lists carry many labels
     W.tune.mid_bail = n_prev_level > 0 && 2 * n_start > n_prev_level;
     n_prev_level = n_start;
-    W.build_bins(G);
+    if (!W.bins_valid) W.build_bins(G);
     int32_t* labels = nullptr;
     cudaEvent_t a0 = W.mark();
     if (lp_iters > 0) {
@@ -301,9 +298,9 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
         unsigned char* flag = W.prflag.as<unsigned char>();
         if (pass == 0 && few) {
           int32_t* list = W.prlist.ensure_n<int32_t>(G.n);
-          flag_list(G.n, flag, kListA, list, &W.ctr()->nlist, nullptr, s);
+          flag_list(G.n, flag, kListA, list, &W.ctr()->nflag, nullptr, s);
           pr_pass_a_lists(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), st, list,
-                          &W.ctr()->nlist, W.parent.as<int32_t>(), lab, &W.ctr()->changed, s);
+                          &W.ctr()->nflag, W.parent.as<int32_t>(), lab, &W.ctr()->changed, s);
         } else if (pass == 0) {
           pr_pass_a(G, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), st,
                     W.parent.as<int32_t>(), lab, &W.ctr()->changed, s);
@@ -810,8 +807,7 @@ struct StepCtx {
     ws->s = s;
     ws->ensure_vertices(g.n);
     ws->ensure_entries(g.nnz, g.n);
-    VC_CUDA(cudaMemsetAsync(ws->state.p, 0, sizeof(vc::DevState), s));
-    VC_CUDA(cudaMemsetAsync(ws->counters.p, 0, sizeof(vc::Counters), s));
+    VC_CUDA(cudaMemsetAsync(ws->state.p, 0, sizeof(vc::Record), s));
   }
   ~StepCtx() {
     if (s) cudaStreamSynchronize(s);
