@@ -377,12 +377,70 @@ __global__ void cluster_scatter_long_k(const int64_t* __restrict__ off, const in
   }
 }
 
+// ---- sorting pairs by target: a bitonic network over packed elements (target << kIdxBits |
+// place of the pair), E of them in the registers of each thread.  Element i = thread E + r,
+// so that strides below E stay in a thread, strides up to 16 E are one shuffle and only a
+// block's longest strides go through shared memory; the pairs' sums never move.
+constexpr int kIdxBits = 12;  // places below kMergeBlockMax
+static_assert((1 << kIdxBits) >= kMergeBlockMax, "a pair's place fits beside its target");
+constexpr unsigned long long kSortPad = ~0ull;
+
+__device__ __forceinline__ void sort_pair(unsigned long long& a, unsigned long long& b, bool up) {
+  const unsigned long long lo = a < b ? a : b, hi = a < b ? b : a;
+  a = up ? lo : hi;
+  b = up ? hi : lo;
+}
+
+// The strides below E of merge level k; `up` for levels of at least E.
+template <int E>
+__device__ __forceinline__ void sort_inside(unsigned long long (&x)[E], int k, bool up) {
+#pragma unroll
+  for (int j = E / 2; j > 0; j >>= 1)
+#pragma unroll
+    for (int r = 0; r < E; ++r)
+      if ((r & j) == 0 && j < k) sort_pair(x[r], x[r | j], k < E ? (r & k) == 0 : up);
+}
+
+// Sorts the T E elements of T threads (32: a warp, each warp for itself; more: the block, with
+// T E elements of shared memory).
+template <int E, int T>
+__device__ __forceinline__ void sort_elements(unsigned long long (&x)[E], unsigned long long* sh) {
+  const int t = T == 32 ? (threadIdx.x & 31) : threadIdx.x;
+#pragma unroll
+  for (int k = 2; k < E; k <<= 1) sort_inside<E>(x, k, true);
+  if (E > 1) sort_inside<E>(x, E, (t & 1) == 0);
+#pragma unroll 1
+  for (int h = 2; h <= T; h <<= 1) {  // merge level h E
+    const bool up = (t & h) == 0;
+#pragma unroll 1
+    for (int m = h >> 1; m > 0; m >>= 1) {  // stride m E
+      const bool keep_low = ((t & m) == 0) == up;
+      if (m >= 32) {
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < E; ++r) sh[r * T + t] = x[r];
+        __syncthreads();
+      }
+#pragma unroll
+      for (int r = 0; r < E; ++r) {
+        const unsigned long long y = m >= 32 ? sh[r * T + (t ^ m)] : __shfl_xor_sync(0xffffffffu, x[r], m);
+        x[r] = (y < x[r]) == keep_low ? y : x[r];
+      }
+    }
+    sort_inside<E>(x, h * E, up);
+  }
+}
+
+// Places of sorted elements in shared memory, padded so that threads writing their E
+// consecutive elements meet no bank conflicts (4-byte and 8-byte elements).
+__device__ __forceinline__ int pad4(int i) { return i + (i >> 5); }
+__device__ __forceinline__ int pad8(int i) { return i + (i >> 4); }
+
 // A warp per cluster of at most kMergeMax pairs, the distinct targets written back in
 // ascending order at the front of the segment; dcount[c] = their number.  The pairs go
 // into registers and the warp takes one step per distinct target (summing its
 // weights) while targets are few; a cluster reaching kMergeWarpKeys targets is sorted
-// instead, in the warp's shared-memory buffer (bitonic network), and every run head
-// sums its run (a step per target costs slots x compares, which only pays while
+// instead, and every run head sums its run (a step per target costs slots x compares, which only pays while
 // targets are few).  With sort_first (a contraction whose clusters are mostly one or
 // two vertices: nearly every pair its own target) a cluster of at least kMergeSortMin
 // pairs is sorted without walking first.  With a list (list_n not null) only the listed
@@ -397,11 +455,13 @@ __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long lon
                                                        const int32_t* __restrict__ list,
                                                        const int* __restrict__ list_n) {
   constexpr int S = kMergeMax / 32;
-  __shared__ int32_t sk_all[8][kMergeMax];
+  __shared__ int32_t sk_all[8][kMergeMax + kMergeMax / 32];
+  __shared__ uint16_t si_all[8][kMergeMax + kMergeMax / 32];
   __shared__ long long sv_all[8][kMergeMax];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int32_t* sk = sk_all[wid];
-  long long* sv = sv_all[wid];
+  int32_t* sk = sk_all[wid];   // sorted targets (at pad4),
+  uint16_t* si = si_all[wid];  // the places of their pairs,
+  long long* sv = sv_all[wid]; // the pairs' sums by place
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   if (list_n) c = *list_n;
   for (int64_t xi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; xi < c; xi += warps) {
@@ -473,50 +533,45 @@ __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long lon
         continue;
       }
     }
-    // many targets: sort the pairs (from registers) in shared memory; each stage of the
-    // bitonic network compares N / 2 pairs (i, i + j), i with bit j clear
-    int N = 32;
-    while (N < T) N <<= 1;
+    // many targets: sort the pairs
 #pragma unroll
-    for (int r = 0; r < S; ++r) {
-      const int i = lane + 32 * r;
-      if (i < N) {
-        sk[i] = i < T ? L.k[r] : INT_MAX;
-        sv[i] = i < T ? L.wt[r] : 0;
+    for (int r = 0; r < S; ++r)
+      if (32 * r < T && lane + 32 * r < T) sv[lane + 32 * r] = L.wt[r];
+    auto sorted = [&](auto size) {
+      constexpr int E = decltype(size)::value;
+      unsigned long long e[E];
+#pragma unroll
+      for (int r = 0; r < E; ++r) {
+        const int i = lane + 32 * r;
+        e[r] = i < T ? ((unsigned long long)(uint32_t)L.k[r] << kIdxBits | (unsigned)i) : kSortPad;
       }
-    }
+      sort_elements<E, 32>(e, nullptr);
+#pragma unroll
+      for (int r = 0; r < E; ++r) {
+        const int i = pad4(lane * E + r);
+        sk[i] = (int32_t)(e[r] >> kIdxBits);  // pads: beyond T
+        si[i] = (uint16_t)(e[r] & ((1u << kIdxBits) - 1u));
+      }
+    };
+    if (T <= 64) sorted(std::integral_constant<int, 2>());
+    else if (T <= 128) sorted(std::integral_constant<int, 4>());
+    else if (T <= 256) sorted(std::integral_constant<int, 8>());
+    else sorted(std::integral_constant<int, 16>());
     __syncwarp();
-    for (int k = 2; k <= N; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int p = lane; p < (N >> 1); p += 32) {
-          const int i = ((p & ~(j - 1)) << 1) | (p & (j - 1));
-          const int l = i | j;
-          const bool up = (i & k) == 0;
-          const int32_t a = sk[i], q = sk[l];
-          if (up ? a > q : a < q) {
-            sk[i] = q;
-            sk[l] = a;
-            const long long t = sv[i];
-            sv[i] = sv[l];
-            sv[l] = t;
-          }
-        }
-        __syncwarp();
-      }
-    }
     int out = 0;
     for (int c0 = 0; c0 < T; c0 += 32) {
       const int i = c0 + lane;
-      const bool head = i < T && (i == 0 || sk[i - 1] != sk[i]);
+      const int32_t key = i < T ? sk[pad4(i)] : 0;
+      const bool head = i < T && (i == 0 || sk[pad4(i - 1)] != key);
       long long sum = 0;
       if (head) {
-        sum = sv[i];
-        for (int j = i + 1; j < T && sk[j] == sk[i]; ++j) sum += sv[j];
+        sum = sv[si[pad4(i)]];
+        for (int j = i + 1; j < T && sk[pad4(j)] == key; ++j) sum += sv[si[pad4(j)]];
       }
       const unsigned bal = __ballot_sync(0xffffffffu, head);
       if (head) {
         const int at = out + __popc(bal & ((1u << lane) - 1u));
-        seg_key[b + at] = sk[i];
+        seg_key[b + at] = key;
         seg_val[b + at] = sum;
       }
       out += __popc(bal);
@@ -526,11 +581,69 @@ __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long lon
   }
 }
 
-// Clusters of kMergeMax < T <= kMergeBlockMax pairs: a block per cluster sorts the
-// pairs by target in shared memory (bitonic network over the next power of two,
-// padding keys INT_MAX), then every run head sums its run; the distinct targets are
-// written back in ascending order at the front of the segment.
+// Clusters of kMergeMax < T <= kMergeBlockMax pairs: a block per cluster sorts the pairs by
+// target (sort_elements, 4 to 16 elements per thread), then every run head sums its run; the
+// distinct targets are written back in ascending order at the front of the segment.
 // With a list (list_count not null) only the listed clusters are visited.
+constexpr int kMergeBlockSmem = (kMergeBlockMax + kMergeBlockMax / 16 + kMergeBlockMax) * 8;  // elements, sums
+
+template <int E>
+__device__ __forceinline__ int merge_block(long long b, int T, int32_t* __restrict__ seg_key,
+                                           long long* __restrict__ seg_val, unsigned long long* se, long long* sv,
+                                           int* s_warp) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  unsigned long long e[E];
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const int i = tid + 256 * r;
+    e[r] = i < T ? ((unsigned long long)(uint32_t)seg_key[b + i] << kIdxBits | (unsigned)i) : kSortPad;
+    if (i < T) sv[i] = seg_val[b + i];
+  }
+  sort_elements<E, 256>(e, se);
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < E; ++r) se[pad8(tid * E + r)] = e[r];
+  __syncthreads();
+  // run heads among this thread's consecutive elements, numbered by a block scan
+  const unsigned long long before0 = tid ? se[pad8(tid * E - 1)] >> kIdxBits : ~0ull;
+  unsigned heads = 0;
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const unsigned long long key = e[r] >> kIdxBits, prev = r ? e[r ? r - 1 : 0] >> kIdxBits : before0;
+    if (e[r] != kSortPad && key != prev) heads |= 1u << r;
+  }
+  const int cnt = __popc(heads);
+  int inc = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) s_warp[wid] = inc;
+  __syncthreads();
+  int before = 0, total = 0;
+  for (int w2 = 0; w2 < 8; ++w2) {
+    if (w2 < wid) before += s_warp[w2];
+    total += s_warp[w2];
+  }
+  int at = before + inc - cnt;
+  // the sorted copy and the sums are in shared memory, so the segment can be overwritten
+  for (unsigned m = heads; m; m &= m - 1u) {
+    const int i = tid * E + __ffs(m) - 1;
+    const unsigned long long x = se[pad8(i)], key = x >> kIdxBits;
+    long long sum = sv[x & ((1u << kIdxBits) - 1u)];
+    for (int j = i + 1; j < T; ++j) {
+      const unsigned long long y = se[pad8(j)];
+      if (y >> kIdxBits != key) break;
+      sum += sv[y & ((1u << kIdxBits) - 1u)];
+    }
+    seg_key[b + at] = (int32_t)key;
+    seg_val[b + at] = sum;
+    ++at;
+  }
+  return total;
+}
+
 __global__ void __launch_bounds__(256) cluster_merge_block_k(int64_t c, const long long* __restrict__ cbase,
                                                              int32_t* __restrict__ seg_key,
                                                              long long* __restrict__ seg_val,
@@ -538,74 +651,20 @@ __global__ void __launch_bounds__(256) cluster_merge_block_k(int64_t c, const lo
                                                              const int32_t* __restrict__ list = nullptr,
                                                              const int* __restrict__ list_count = nullptr) {
   extern __shared__ __align__(16) unsigned char mb_dyn[];
-  long long* sv = (long long*)mb_dyn;
-  int32_t* sk = (int32_t*)(sv + kMergeBlockMax);
+  unsigned long long* se = (unsigned long long*)mb_dyn;
+  long long* sv = (long long*)(se + kMergeBlockMax + kMergeBlockMax / 16);
   __shared__ int s_warp[8];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t total = list_count ? (int64_t)*list_count : c;
   for (int64_t xi = blockIdx.x; xi < total; xi += gridDim.x) {
     const int64_t x = list_count ? (int64_t)list[xi] : xi;
     const long long b = cbase[x];
     const int T = (int)(cbase[x + 1] - b);
     if (T <= kMergeMax || T > kMergeBlockMax) continue;  // the same in every thread of the block
-    int N = 1;
-    while (N < T) N <<= 1;
-    for (int i = tid; i < N; i += 256) {
-      sk[i] = i < T ? seg_key[b + i] : INT_MAX;
-      sv[i] = i < T ? seg_val[b + i] : 0;
-    }
-    __syncthreads();
-    for (int k = 2; k <= N; k <<= 1) {
-      for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int p = tid; p < (N >> 1); p += 256) {  // pair (i, i + j), i with bit j clear
-          const int i = ((p & ~(j - 1)) << 1) | (p & (j - 1));
-          const int l = i | j;
-          const bool up = (i & k) == 0;
-          const int32_t a = sk[i], bb = sk[l];
-          if (up ? a > bb : a < bb) {
-            sk[i] = bb;
-            sk[l] = a;
-            const long long t = sv[i];
-            sv[i] = sv[l];
-            sv[l] = t;
-          }
-        }
-        __syncthreads();
-      }
-    }
-    // run heads, numbered by a block scan; each head sums its run
-    constexpr int kPer = kMergeBlockMax / 256;
-    int cnt = 0;
-    for (int q = 0; q < kPer; ++q) {
-      const int i = tid * kPer + q;
-      if (i < N && sk[i] != INT_MAX && (i == 0 || sk[i] != sk[i - 1])) ++cnt;
-    }
-    int inc = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) s_warp[wid] = inc;
-    __syncthreads();
-    int before = 0, total = 0;
-    for (int w2 = 0; w2 < 8; ++w2) {
-      if (w2 < wid) before += s_warp[w2];
-      total += s_warp[w2];
-    }
-    int at = before + inc - cnt;
-    // the sorted copy is in shared memory, so the segment can be overwritten
-    for (int q = 0; q < kPer; ++q) {
-      const int i = tid * kPer + q;
-      if (i < N && sk[i] != INT_MAX && (i == 0 || sk[i] != sk[i - 1])) {
-        long long sum = sv[i];
-        for (int j = i + 1; j < N && sk[j] == sk[i]; ++j) sum += sv[j];
-        seg_key[b + at] = sk[i];
-        seg_val[b + at] = sum;
-        ++at;
-      }
-    }
-    if (tid == 0) dcount[x] = total;
+    int d;
+    if (T <= 1024) d = merge_block<4>(b, T, seg_key, seg_val, se, sv, s_warp);
+    else if (T <= 2048) d = merge_block<8>(b, T, seg_key, seg_val, se, sv, s_warp);
+    else d = merge_block<16>(b, T, seg_key, seg_val, se, sv, s_warp);
+    if (threadIdx.x == 0) dcount[x] = d;
     __syncthreads();
   }
 }
@@ -1217,7 +1276,7 @@ void cluster_stats(int64_t n, const int32_t* ccount, int* maxt, long long* pairs
 static int merge_block_smem() {
   static std::mutex mu;
   static std::unordered_map<int, bool> ready;  // per device: the shared-memory limit was raised
-  const int smem = kMergeBlockMax * (int)(sizeof(long long) + sizeof(int32_t));
+  const int smem = kMergeBlockSmem;
   int dev = 0;
   VC_CUDA(cudaGetDevice(&dev));
   std::lock_guard<std::mutex> lk(mu);
@@ -1280,7 +1339,7 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
     // like the other lists' here, starts from zero)
     block_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, blist, blist_n);
     const int smem = merge_block_smem();
-    cluster_merge_block_k<<<kSMs, 256, smem, s>>>(c, cbase, seg_key, seg_val, ccount, blist, blist_n);
+    cluster_merge_block_k<<<kSMs * 3, 256, smem, s>>>(c, cbase, seg_key, seg_val, ccount, blist, blist_n);
     count_launch(2);
     VC_CHECK_LAUNCH();
   }
