@@ -443,21 +443,26 @@ __device__ __forceinline__ int pad8(int i) { return i + (i >> 4); }
 // instead, and every run head sums its run (a step per target costs slots x compares, which only pays while
 // targets are few).  With sort_first (a contraction whose clusters are mostly one or
 // two vertices: nearly every pair its own target) a cluster of at least kMergeSortMin
-// pairs is sorted without walking first.  With a list (list_n not null) only the listed
-// clusters are visited (a sparse contraction leaves nearly all of them without pairs:
-// 0.75 ms for 3.5 million empty clusters, 0.04 ms to list the others).
+// pairs is sorted without walking first.  S slots per lane: clusters of at most
+// kMergeSmall pairs with four, the others with sixteen, whose registers would halve the
+// warps in flight for all.  With a list (list_n not null) only the listed clusters are
+// visited (a sparse contraction leaves nearly all of them without pairs: 0.75 ms for
+// 3.5 million empty clusters, 0.04 ms to list the others).
 constexpr int kMergeWarpKeys = 32;
 constexpr int kMergeSortMin = 12;
+constexpr int kMergeSmall = 128;
+constexpr int kMergeWarps = 4;
 
-__global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long long* __restrict__ cbase,
+template <int S>
+__global__ void __launch_bounds__(kMergeWarps * 32) cluster_merge_k(int64_t c, const long long* __restrict__ cbase,
                                                        int32_t* __restrict__ seg_key, long long* __restrict__ seg_val,
                                                        int32_t* __restrict__ dcount, bool sort_first,
                                                        const int32_t* __restrict__ list,
                                                        const int* __restrict__ list_n) {
-  constexpr int S = kMergeMax / 32;
-  __shared__ int32_t sk_all[8][kMergeMax + kMergeMax / 32];
-  __shared__ uint16_t si_all[8][kMergeMax + kMergeMax / 32];
-  __shared__ long long sv_all[8][kMergeMax];
+  constexpr int kMax = 32 * S;
+  __shared__ int32_t sk_all[kMergeWarps][kMax + S];
+  __shared__ uint16_t si_all[kMergeWarps][kMax + S];
+  __shared__ long long sv_all[kMergeWarps][kMax];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int32_t* sk = sk_all[wid];   // sorted targets (at pad4),
   uint16_t* si = si_all[wid];  // the places of their pairs,
@@ -468,7 +473,7 @@ __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long lon
     const int64_t x = list_n ? (int64_t)list[xi] : xi;
     const long long b = cbase[x];
     const int T = (int)(cbase[x + 1] - b);
-    if (T > kMergeMax) continue;  // the block kernel takes it
+    if (T > kMax) continue;  // another launch takes it
     RegList<long long, S> L;
     L.slots = (T + 31) >> 5;
     L.todo = 0;
@@ -553,10 +558,9 @@ __global__ void __launch_bounds__(256) cluster_merge_k(int64_t c, const long lon
         si[i] = (uint16_t)(e[r] & ((1u << kIdxBits) - 1u));
       }
     };
-    if (T <= 64) sorted(std::integral_constant<int, 2>());
-    else if (T <= 128) sorted(std::integral_constant<int, 4>());
-    else if (T <= 256) sorted(std::integral_constant<int, 8>());
-    else sorted(std::integral_constant<int, 16>());
+    // T > kMergeSmall in the launch of the larger clusters
+    if (2 * T <= kMax) sorted(std::integral_constant<int, S / 2>());
+    else sorted(std::integral_constant<int, S>());
     __syncwarp();
     int out = 0;
     for (int c0 = 0; c0 < T; c0 += 32) {
@@ -1295,15 +1299,15 @@ __global__ void block_class_list_k(int64_t c, const long long* __restrict__ cbas
   }
 }
 
-// The clusters of 1 to kMergeMax pairs.
-__global__ void warp_class_list_k(int64_t c, const long long* __restrict__ cbase, int32_t* __restrict__ list,
-                                  int* __restrict__ count) {
+// The clusters of lo + 1 to hi pairs.
+__global__ void warp_class_list_k(int64_t c, const long long* __restrict__ cbase, int lo, int hi,
+                                  int32_t* __restrict__ list, int* __restrict__ count) {
   const int lane = threadIdx.x & 31;
   for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; b < c;
        b += (int64_t)gridDim.x * blockDim.x) {
     const int64_t x = b + lane;
     const long long T = x < c ? cbase[x + 1] - cbase[x] : 0;
-    const bool in = T > 0 && T <= kMergeMax;
+    const bool in = T > lo && T <= hi;
     const unsigned bal = __ballot_sync(0xffffffffu, in);
     int at = 0;
     if (lane == 0 && bal) at = atomicAdd(count, __popc(bal));
@@ -1314,26 +1318,34 @@ __global__ void warp_class_list_k(int64_t c, const long long* __restrict__ cbase
 
 void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int32_t* ccount, int64_t c,
                    long long* cbase, long long* cursor, int32_t* seg_key, long long* seg_val, int64_t* coff,
-                   int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, bool big, bool sort_first,
-                   const GiantScratch* giant, int32_t* blist, int* blist_n, cudaStream_t s, const SparseCtx* sp,
+                   int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, int maxt, bool sort_first,
+                   const GiantScratch* giant, int32_t* blist, int* blist_n, const MergeLists& lists, cudaStream_t s,
+                   const SparseCtx* sp,
                    const LongLists& longs) {
   exclusive_scan<int, long long>(ccount, cbase, c, cbase + c, cs.scan_scr, s, cursor);
-  const int gv = grid_for(g.n, 256, kSMs * 8), gc = grid_for(c, 8, kSMs * 16);
+  const int gv = grid_for(g.n, 256, kSMs * 8), gc = grid_for(c, kMergeWarps, kSMs * 32);
   const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
   cluster_scatter_k<<<gv, 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, cursor, seg_key, seg_val, longs);
   if (longs.item) {
     cluster_scatter_long_k<<<kSMs * 4, 256, 0, s>>>(g.off, cs.cnt, in, seg_key, seg_val, longs);
     count_launch();
   }
+  const int gl = grid_for(c, 256, kSMs * 8);
   if (sp) {
-    warp_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, sp->list, sp->list_n);
+    warp_class_list_k<<<gl, 256, 0, s>>>(c, cbase, 0, kMergeSmall, lists.small, lists.n);
     count_launch();
   }
-  cluster_merge_k<<<gc, 256, 0, s>>>(c, cbase, seg_key, seg_val, ccount, sort_first, sp ? sp->list : nullptr,
-                                     sp ? sp->list_n : nullptr);
+  cluster_merge_k<kMergeSmall / 32><<<gc, kMergeWarps * 32, 0, s>>>(
+      c, cbase, seg_key, seg_val, ccount, sort_first, sp ? lists.small : nullptr, sp ? lists.n : nullptr);
   count_launch(2);
+  if (maxt > kMergeSmall) {
+    warp_class_list_k<<<gl, 256, 0, s>>>(c, cbase, kMergeSmall, kMergeMax, lists.large, lists.n + 1);
+    cluster_merge_k<kMergeMax / 32><<<gc, kMergeWarps * 32, 0, s>>>(c, cbase, seg_key, seg_val, ccount, sort_first,
+                                                                   lists.large, lists.n + 1);
+    count_launch(2);
+  }
   VC_CHECK_LAUNCH();
-  if (big) {
+  if (maxt > kMergeMax) {
     // the clusters of kMergeMax < T <= kMergeBlockMax pairs listed first, so that the
     // blocks visit only them (blist: n ints no longer needed once the scatter ran; its count,
     // like the other lists' here, starts from zero)

@@ -69,7 +69,7 @@ struct Counters {
   long long gpairs;   // the pairs of clusters of more than kMergeBlockMax pairs
   int ngiant;         // those clusters
   int blist_n;        // clusters listed for the block-level merge
-  int nlist;          // clusters listed for the sparse contraction's merge
+  int nlist[2];       // clusters listed for the warp-level merges
   int nlong[2];       // lists left to a grid's blocks to share (LongLists)
   int nflag;          // vertices listed by flag_list
   int nprlong;        // pairs listed by pass B (PrLong)
@@ -92,7 +92,7 @@ struct Workspace {
   cudaStream_t s = nullptr;
   // vertex-sized
   Buf deg, labA, labB, map0, cidT, cur1, side1, flags, rank, cnt, pos, scan64, scan32, hv;
-  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, longV, longAt, longHit, slist, rlist, mlist, blist, glist, bl1, noi_r;
+  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, longV, longAt, longHit, mergeS, mergeL, slist, rlist, mlist, blist, glist, bl1, noi_r;
   // entry-sized
   Buf tmpK, tmpV, cmpK, cmpV;
   // pair-sized
@@ -648,9 +648,10 @@ struct Workspace {
         gs.hist = hist.ensure_n<long long>(radix_hist_elems(GP));
       }
       const SparseCtx sp{scidm.as<int32_t>(), sdeg.as<int32_t>(), sclean.as<unsigned char>(),
-                         sdirty.as<unsigned char>(), sdlist.as<int32_t>(), &ctr()->nlist};
+                         sdirty.as<unsigned char>()};
+      const MergeLists ml{mergeS.ensure_n<int32_t>(c), mergeL.ensure_n<int32_t>(c), ctr()->nlist};
       cluster_merge(g, cid_out, cs, ccount, c, cbase, cur, sk, sv, co, ca, cwp, csp, &st()->nnz,
-                    h_counters->maxt > kMergeMax, 2 * c >= g.n, ng ? &gs : nullptr, cs.cnt, &ctr()->blist_n, s,
+                    h_counters->maxt, 2 * c >= g.n, ng ? &gs : nullptr, cs.cnt, &ctr()->blist_n, ml, s,
                     sparse ? &sp : nullptr, longs);
     } else {
       exclusive_scan<int, long long>(cs.cnt, cs.pos, g.n, &ctr()->pairs, cs.scan_scr, s);

@@ -237,8 +237,7 @@ struct LongLists {
 // (giant index, target).  The pre-merge fills ccount[cid] (PairOut::ccount);
 // cluster_stats reads its n entries (zero beyond the c clusters) into *maxt, *pairs and
 // the giant clusters' count and pairs; cluster_merge writes the coarse CSR (coff[c + 1],
-// sorted cadj, cw, entry sources csrc) and *nnz_dev; big = some cluster holds more than
-// kMergeMax pairs.
+// sorted cadj, cw, entry sources csrc) and *nnz_dev; maxt = the most pairs of a cluster.
 constexpr int kMergeMax = 512;
 constexpr int kMergeBlockMax = 4096;
 struct GiantScratch {
@@ -267,15 +266,19 @@ struct SparseCtx {
   const int32_t* sdeg;
   unsigned char* clean;
   const unsigned char* dirty;  // 1: left to the pre-merge; 2: a lone list with no entry into a merged group
-  int32_t* list;               // scratch: c ids
-  int* list_n;
+};
+// Clusters by merge launch: up to 128 pairs (listed in sparse contractions only), up to
+// kMergeMax; room for c each, two counts, zero.
+struct MergeLists {
+  int32_t *small, *large;
+  int* n;
 };
 void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, unsigned char* mflag, int32_t* cidm,
                  unsigned char* dirty, int32_t* sdeg, int32_t* list, int* count, cudaStream_t s);
 void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int32_t* ccount, int64_t c,
                    long long* cbase, long long* cursor, int32_t* seg_key, long long* seg_val, int64_t* coff,
-                   int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, bool big, bool sort_first,
-                   const GiantScratch* giant, int32_t* blist, int* blist_n, cudaStream_t s,
+                   int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, int maxt, bool sort_first,
+                   const GiantScratch* giant, int32_t* blist, int* blist_n, const MergeLists& lists, cudaStream_t s,
                    const SparseCtx* sparse = nullptr, const LongLists& longs = LongLists());
 
 // Builds (cid[v] << bits | cu, weight) pairs from the pre-merged lists.
