@@ -13,6 +13,7 @@
 #include <limits.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
 #include <type_traits>
 #include <unordered_map>
@@ -800,35 +801,189 @@ __device__ __forceinline__ int sc_collect(int64_t beg, int64_t end, int lane, co
   return nm;
 }
 
+// A contraction that merges few vertices touches few lists: the neighbours of the merged
+// groups' members (every edge is in both lists), found from the members' own.  They are
+// marked so (touched) while at most a sixteenth of the vertices disappears, and pass 1 then
+// reads only those lists; otherwise it reads every list.  Planted 8 x 2^20, 392 million
+// entries: 1.25 ms a pass over every list, whatever the pass merged (one random gather per
+// entry, at 0.8 of one per SM and cycle); 31.0 -> 17.2 ms for its 25 contractions.  Below
+// kScPushMin entries a pass costs less than the marking: 8 x 60,000 (18.7 million entries)
+// took 1.9 ms with it, 1.6 ms without.
+constexpr int64_t kScPushMin = int64_t(1) << 25;
+__device__ __forceinline__ bool sc_few(int64_t n, const int* nclust) { return 16 * (n - __ldg(nclust)) <= n; }
+
+__global__ void __launch_bounds__(256) sc_push_k(int64_t n, const int* __restrict__ nclust,
+                                                 const int32_t* __restrict__ cidm, const int64_t* __restrict__ off,
+                                                 const int32_t* __restrict__ adj,
+                                                 unsigned char* __restrict__ touched, int32_t* __restrict__ longs,
+                                                 int* __restrict__ nlong) {
+  if (!sc_few(n, nclust)) return;
+  const int lane = threadIdx.x & 31;
+  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; b < n;
+       b += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = b + lane;
+    for (unsigned m = __ballot_sync(0xffffffffu, v < n && cidm[v] < 0); m; m &= m - 1u) {
+      const int64_t x = b + __ffs(m) - 1, beg = off[x], end = off[x + 1];
+      if (end - beg > kLongList) {
+        if (lane == 0) longs[atomicAdd(nlong, 1)] = (int32_t)x;
+        continue;
+      }
+#pragma unroll 4
+      for (int64_t e = beg + lane; e < end; e += 32) touched[__ldg(adj + e)] = 1;
+    }
+  }
+}
+
+// The lists sc_push_k left out (a hub's), shared by the blocks.
+__global__ void __launch_bounds__(256) sc_push_long_k(const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
+                                                      unsigned char* __restrict__ touched,
+                                                      const int32_t* __restrict__ longs,
+                                                      const int* __restrict__ nlong) {
+  const int n = *nlong;
+  const GridShare G(n);
+  for (int i = G.first; i < n; i += G.step) {
+    const int64_t beg = off[longs[i]], end = off[longs[i] + 1];
+#pragma unroll 4
+    for (int64_t e = beg + G.part * 256 + threadIdx.x; e < end; e += (int64_t)G.parts * 256) touched[__ldg(adj + e)] = 1;
+  }
+}
+
 // Pass 1: the coarse degree of every lone vertex handled here (sdeg[v], else -1), and in
 // dirty the vertices left to the pre-merge (1) and the lists with no entry into a merged
-// group (2).
-__global__ void __launch_bounds__(256) sc_count_k(int64_t n, const int32_t* __restrict__ cidm,
-                                                  const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                                                  int32_t* __restrict__ sdeg, unsigned char* __restrict__ dirty) {
+// group (2).  A warp per `per` vertices, the lists to read one after another: 32 where most
+// are not read (touched), else 1.
+__global__ void __launch_bounds__(256) sc_count_k(int64_t n, const int* __restrict__ nclust,
+                                                  const int32_t* __restrict__ cidm, const int64_t* __restrict__ off,
+                                                  const int32_t* __restrict__ adj,
+                                                  const unsigned char* __restrict__ touched,
+                                                  int32_t* __restrict__ sdeg, unsigned char* __restrict__ dirty,
+                                                  int per) {
   __shared__ int32_t s_mk[8][kScMaxM];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-    const int64_t beg = off[v], end = off[v + 1];
-    if (cidm[v] < 0) {  // a member of a merged group
-      if (lane == 0) { sdeg[v] = -1; dirty[v] = 1; }
-      continue;
+  const bool few = touched && sc_few(n, nclust);
+  for (int64_t b = ((int64_t)blockIdx.x * 8 + wid) * per; b < n; b += (int64_t)gridDim.x * 8 * per) {
+    const int64_t v = lane < per ? b + lane : n;
+    int64_t beg = 0, end = 0;
+    bool read = false;
+    int32_t deg = -1;         // a member of a merged group
+    unsigned char state = 1;
+    if (v < n) {
+      beg = off[v];
+      end = off[v + 1];
+      if (cidm[v] >= 0) {
+        read = !few || touched[v];
+        deg = (int32_t)(end - beg);
+        state = 2;
+      }
     }
-    const int nm = sc_collect<false>(beg, end, lane, adj, (const UnitW*)nullptr, cidm, s_mk[wid], nullptr);
-    if (nm > kScMaxM) {
-      if (lane == 0) { sdeg[v] = -1; dirty[v] = 1; }
-      continue;
+    for (unsigned m = __ballot_sync(0xffffffffu, read); m; m &= m - 1u) {
+      const int j = __ffs(m) - 1;
+      const int64_t lb = __shfl_sync(0xffffffffu, beg, j), le = __shfl_sync(0xffffffffu, end, j);
+      const int nm = sc_collect<false>(lb, le, lane, adj, (const UnitW*)nullptr, cidm, s_mk[wid], nullptr);
+      int nd = nm;
+      if (nm > 1 && nm <= kScMaxM) {  // the same in every lane
+        const bool have = lane < nm;
+        const int32_t key = have ? s_mk[wid][lane] : -1 - lane;
+        const unsigned peers = __match_any_sync(0xffffffffu, key);
+        nd = __popc(__ballot_sync(0xffffffffu, have && (__ffs(peers) - 1) == lane));
+      }
+      if (lane == j && nm > 0) {
+        deg = nm > kScMaxM ? -1 : deg - nm + nd;
+        state = nm > kScMaxM ? 1 : 0;
+      }
+      __syncwarp();
     }
-    int nd = nm;
-    if (nm > 1) {  // the same in every lane
-      const bool have = lane < nm;
-      const int32_t key = have ? s_mk[wid][lane] : -1 - lane;
-      const unsigned peers = __match_any_sync(0xffffffffu, key);
-      nd = __popc(__ballot_sync(0xffffffffu, have && (__ffs(peers) - 1) == lane));
+    if (v < n) {
+      sdeg[v] = deg;
+      dirty[v] = state;
     }
-    if (lane == 0) { sdeg[v] = (int32_t)(end - beg - nm + nd); dirty[v] = nm == 0 ? 2 : 0; }
-    __syncwarp();
+  }
+}
+
+// Pass 2 of the lists with no entry into a merged group, where at most one vertex in 512
+// disappears: most runs of 2^shift consecutive ids then lose none, and their new ids are the
+// old ones less one offset.  The offsets of all runs (tab; -1: some id is gone) fit shared
+// memory, and only entries into the other runs gather their new id.  What is left is a
+// stream: 12 bytes read and 16 written per entry (392 million entries, 1800 of 4.4 million
+// vertices gone: 3.5 ms -> 2.4 ms here and 0.4 ms in sc_write_k; 15,800 gone, over one in
+// 512: too few whole runs).  From kScPushMin entries on: at 18.7 million it gained nothing.
+constexpr int kScTab = 16384;  // runs at most
+constexpr int kScCopyThreads = 512;
+static int sc_shift(int64_t n) { return std::max(8, ceil_log2(n) - 14); }
+
+__global__ void sc_table_k(int64_t n, int64_t c, int shift, const int32_t* __restrict__ rank,
+                           int32_t* __restrict__ tab) {
+  const int64_t runs = (n + (1LL << shift) - 1) >> shift;
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < runs; r += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t a = r << shift, z = (r + 1) << shift < n ? (r + 1) << shift : n;
+    const int64_t ra = rank[a], rz = z < n ? (int64_t)rank[z] : c;
+    tab[r] = rz - ra == z - a ? (int32_t)(a - ra) : -1;
+  }
+}
+
+template <typename WT>
+__global__ void __launch_bounds__(kScCopyThreads) sc_copy_k(int64_t n, int shift, const int32_t* __restrict__ tab,
+                                                            const int32_t* __restrict__ cidm,
+                                                            const int64_t* __restrict__ off,
+                                                            const int32_t* __restrict__ adj,
+                                                            const WT* __restrict__ w,
+                                                            const unsigned char* __restrict__ dirty,
+                                                            const int64_t* __restrict__ coff,
+                                                            int32_t* __restrict__ cadj, long long* __restrict__ cw,
+                                                            int32_t* __restrict__ csrc) {
+  extern __shared__ int32_t s_tab[];
+  const int lane = threadIdx.x & 31;
+  const int runs = (int)((n + (1LL << shift) - 1) >> shift);
+  for (int i = threadIdx.x; i < runs; i += kScCopyThreads) s_tab[i] = tab[i];
+  __syncthreads();
+  const int64_t warps = (int64_t)gridDim.x * (kScCopyThreads / 32);
+  int64_t v = ((int64_t)blockIdx.x * kScCopyThreads + threadIdx.x) >> 5;
+  if (v >= n) return;
+  // the next list's header is read ahead
+  int64_t beg = off[v], to = 0;
+  int len = dirty[v] == 2 ? (int)(off[v + 1] - beg) : 0;  // a strictly increasing list: below 2^31 entries
+  int32_t x = cidm[v];
+  for (;;) {
+    const int64_t vn = v + warps;
+    int64_t nbeg = 0;
+    int nlen = 0;
+    int32_t xn = 0;
+    if (vn < n) {
+      nbeg = off[vn];
+      nlen = dirty[vn] == 2 ? (int)(off[vn + 1] - nbeg) : 0;
+      xn = cidm[vn];
+    }
+    if (len > 0) {
+      to = coff[x];
+      const int32_t* a = adj + beg;
+      for (int b = lane; b - lane < len; b += 32 * kScUnroll) {
+        int32_t u[kScUnroll];
+        long long wt[kScUnroll];
+#pragma unroll
+        for (int q = 0; q < kScUnroll; ++q) {
+          u[q] = b + 32 * q < len ? __ldg(a + b + 32 * q) : -1;
+          wt[q] = b + 32 * q < len ? ldw(w, beg + b + 32 * q) : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < kScUnroll; ++q)
+          if (u[q] >= 0) {
+            const int32_t d = s_tab[u[q] >> shift];
+            u[q] = d >= 0 ? u[q] - d : __ldg(cidm + u[q]) & 0x7fffffff;
+          }
+#pragma unroll
+        for (int q = 0; q < kScUnroll; ++q)
+          if (u[q] >= 0) {
+            cadj[to + b + 32 * q] = u[q];
+            cw[to + b + 32 * q] = wt[q];
+            csrc[to + b + 32 * q] = x;
+          }
+      }
+    }
+    if (vn >= n) break;
+    v = vn;
+    beg = nbeg;
+    len = nlen;
+    x = xn;
   }
 }
 
@@ -850,10 +1005,11 @@ constexpr int kScChunk = 512;
 template <typename WT>
 __global__ void __launch_bounds__(256) sc_write_k(int64_t n, const int32_t* __restrict__ cidm,
                                                   const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                                                  const WT* __restrict__ w, const int32_t* __restrict__ sdeg,
+                                                  const WT* __restrict__ w,
                                                   const unsigned char* __restrict__ dirty,
                                                   const int64_t* __restrict__ coff, int32_t* __restrict__ cadj,
-                                                  long long* __restrict__ cw, int32_t* __restrict__ csrc) {
+                                                  long long* __restrict__ cw, int32_t* __restrict__ csrc,
+                                                  bool copied) {
   __shared__ int32_t s_mk[8][kScMaxM];
   __shared__ long long s_mw[8][kScMaxM];
   __shared__ int32_t s_dk[8][kScMaxM];
@@ -869,11 +1025,12 @@ __global__ void __launch_bounds__(256) sc_write_k(int64_t n, const int32_t* __re
   uint16_t* at = s_at[wid];
   unsigned* bits = s_bits[wid];
   for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-    if (sdeg[v] < 0) continue;  // the same in every lane
+    const unsigned char state = dirty[v];
+    if (state == 1 || (state == 2 && copied)) continue;  // the same in every lane
     const int64_t beg = off[v], end = off[v + 1];
     const int32_t x = cidm[v];  // lone: no sign bit
     int64_t o = coff[x];
-    if (dirty[v] == 2) {  // no entry into a merged cluster: the list renumbered in place
+    if (state == 2) {  // no entry into a merged cluster: the list renumbered in place
       for (int64_t b = beg; b < end; b += 32 * kScUnroll) {
         int32_t u[kScUnroll];
         long long wt[kScUnroll];
@@ -884,7 +1041,7 @@ __global__ void __launch_bounds__(256) sc_write_k(int64_t n, const int32_t* __re
           wt[q] = e < end ? ldw(w, e) : 0;
         }
 #pragma unroll
-        for (int q = 0; q < kScUnroll; ++q) u[q] = u[q] >= 0 ? __ldg(cidm + u[q]) : -1;
+        for (int q = 0; q < kScUnroll; ++q) u[q] = u[q] >= 0 ? __ldg(cidm + u[q]) & 0x7fffffff : -1;
 #pragma unroll
         for (int q = 0; q < kScUnroll; ++q)
           if (u[q] >= 0) {
@@ -1046,18 +1203,30 @@ static void sc_by_weight(const GraphView& g, F f) {
   else f((const long long*)g.w);
 }
 
-void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, unsigned char* mflag, int32_t* cidm,
-                 unsigned char* dirty, int32_t* sdeg, int32_t* list, int* count, cudaStream_t s) {
+void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, const int* nclust, unsigned char* mflag,
+                 unsigned char* touched, int32_t* cidm, unsigned char* dirty, int32_t* sdeg, int32_t* list, int* count,
+                 cudaStream_t s) {
   VC_CUDA(cudaMemsetAsync(mflag, 0, (size_t)g.n, s));
   VC_CUDA(cudaMemsetAsync(count, 0, sizeof(int), s));
   const int grid = grid_for(g.n, 256, kSMs * 8);
   sc_merged_k<<<grid, 256, 0, s>>>(g.n, lab, cid, mflag);
   sc_pack_k<<<grid, 256, 0, s>>>(g.n, cid, mflag, cidm);
-  sc_count_k<<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, cidm, g.off, g.adj, sdeg, dirty);
+  if (touched) {
+    VC_CUDA(cudaMemsetAsync(touched, 0, (size_t)g.n, s));
+    sc_push_k<<<grid, 256, 0, s>>>(g.n, nclust, cidm, g.off, g.adj, touched, list, count);
+    sc_push_long_k<<<kSMs * 4, 256, 0, s>>>(g.off, g.adj, touched, list, count);
+    VC_CUDA(cudaMemsetAsync(count, 0, sizeof(int), s));
+    count_launch(2);
+  }
+  const int per = touched ? 32 : 1;
+  sc_count_k<<<grid_for(g.n, 8 * per, kSMs * (touched ? 64 : 16)), 256, 0, s>>>(g.n, nclust, cidm, g.off, g.adj,
+                                                                                touched, sdeg, dirty, per);
   sc_list_k<<<grid, 256, 0, s>>>(g.n, dirty, list, count);
   count_launch(4);
   VC_CHECK_LAUNCH();
 }
+
+bool sparse_touches(const GraphView& g) { return g.nnz >= kScPushMin; }
 
 static void sparse_finish_degrees(const GraphView& g, const int32_t* cid, const int32_t* sdeg, int32_t* ccount,
                                   unsigned char* clean, int64_t c, cudaStream_t s) {
@@ -1067,12 +1236,38 @@ static void sparse_finish_degrees(const GraphView& g, const int32_t* cid, const 
   VC_CHECK_LAUNCH();
 }
 
-static void sparse_copy(const GraphView& g, const int32_t* cidm, const int32_t* sdeg, const unsigned char* dirty,
-                        const int64_t* coff, int32_t* cadj, long long* cw, int32_t* csrc, cudaStream_t s) {
+// Opts a copy kernel into its table, once per kernel and device.
+template <typename F>
+static void sc_copy_smem(F kfn) {
+  static std::mutex mu;
+  static std::map<std::pair<const void*, int>, bool> ready;
+  int dev = 0;
+  VC_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  bool& done = ready[{(const void*)kfn, dev}];
+  if (!done)
+    VC_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, kScTab * (int)sizeof(int32_t)));
+  done = true;
+}
+
+static void sparse_copy(const GraphView& g, int64_t c, const SparseCtx& sp, const int64_t* coff, int32_t* cadj,
+                        long long* cw, int32_t* csrc, cudaStream_t s) {
+  const bool table = 512 * (g.n - c) <= g.n && g.nnz >= kScPushMin;
+  const int shift = sc_shift(g.n), runs = (int)((g.n + (int64_t(1) << shift) - 1) >> shift);
+  if (table) {
+    sc_table_k<<<grid_for(runs, 256, kSMs), 256, 0, s>>>(g.n, c, shift, sp.rank, sp.tab);
+    count_launch();
+  }
   sc_by_weight(g, [&](auto wp) {
     using WT = std::remove_cv_t<std::remove_pointer_t<decltype(wp)>>;
-    sc_write_k<WT><<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, cidm, g.off, g.adj, wp, sdeg, dirty, coff, cadj,
-                                                               cw, csrc);
+    if (table) {
+      sc_copy_smem(sc_copy_k<WT>);
+      sc_copy_k<WT><<<grid_for(g.n, kScCopyThreads / 32, kSMs * 8), kScCopyThreads, sizeof(int32_t) * runs, s>>>(
+          g.n, shift, sp.tab, sp.cidm, g.off, g.adj, wp, sp.dirty, coff, cadj, cw, csrc);
+      count_launch();
+    }
+    sc_write_k<WT><<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, sp.cidm, g.off, g.adj, wp, sp.dirty, coff, cadj,
+                                                               cw, csrc, table);
   });
   count_launch();
   VC_CHECK_LAUNCH();
@@ -1368,7 +1563,7 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
   }
   count_launch();
   VC_CHECK_LAUNCH();
-  if (sp) sparse_copy(g, sp->cidm, sp->sdeg, sp->dirty, coff, cadj, cw, csrc, s);
+  if (sp) sparse_copy(g, c, *sp, coff, cadj, cw, csrc, s);
 }
 
 

@@ -385,7 +385,7 @@ struct Workspace {
   // dbins holds their bins.
   bool last_sparse = false;  // the last contraction was a sparse one
   Bins dbins;
-  Buf smflag, scidm, sdirty, sdeg, sclean, sdlist, dsl, drl, dml, dbl, dgl, dbail;
+  Buf stouch, stab, smflag, scidm, sdirty, sdeg, sclean, sdlist, dsl, drl, dml, dbl, dgl, dbail;
   // dbins' lists, for at most n listed vertices
   void prepare_dbins(int64_t n) {
     dbins.small_list = dsl.ensure_n<int32_t>(n);
@@ -401,7 +401,8 @@ struct Workspace {
     const int64_t n = g.n;
     prepare_dbins(n);
     int32_t* list = sdlist.ensure_n<int32_t>(n);
-    sparse_mark(g, labels, cid, smflag.ensure_n<unsigned char>(n), scidm.ensure_n<int32_t>(n),
+    sparse_mark(g, labels, cid, &ctr()->c, smflag.ensure_n<unsigned char>(n),
+                sparse_touches(g) ? stouch.ensure_n<unsigned char>(n) : nullptr, scidm.ensure_n<int32_t>(n),
                 sdirty.ensure_n<unsigned char>(n), sdeg.ensure_n<int32_t>(n), list, dbins.counts + 6, s);
     bins_build(g, dbins, s, list, dbins.counts + 6);
     int ndirty = 0;
@@ -648,7 +649,7 @@ struct Workspace {
         gs.hist = hist.ensure_n<long long>(radix_hist_elems(GP));
       }
       const SparseCtx sp{scidm.as<int32_t>(), sdeg.as<int32_t>(), sclean.as<unsigned char>(),
-                         sdirty.as<unsigned char>()};
+                         sdirty.as<unsigned char>(), cs.rank, stab.ensure_n<int32_t>(16384)};
       const MergeLists ml{mergeS.ensure_n<int32_t>(c), mergeL.ensure_n<int32_t>(c), ctr()->nlist};
       cluster_merge(g, cid_out, cs, ccount, c, cbase, cur, sk, sv, co, ca, cwp, csp, &st()->nnz,
                     h_counters->maxt, 2 * c >= g.n, ng ? &gs : nullptr, cs.cnt, &ctr()->blist_n, ml, s,

@@ -266,6 +266,8 @@ struct SparseCtx {
   const int32_t* sdeg;
   unsigned char* clean;
   const unsigned char* dirty;  // 1: left to the pre-merge; 2: a lone list with no entry into a merged group
+  const int32_t* rank;         // ids that stay below each id (relabel)
+  int32_t* tab;                // scratch: 16384 ints
 };
 // Clusters by merge launch: up to 128 pairs (listed in sparse contractions only), up to
 // kMergeMax; room for c each, two counts, zero.
@@ -273,8 +275,11 @@ struct MergeLists {
   int32_t *small, *large;
   int* n;
 };
-void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, unsigned char* mflag, int32_t* cidm,
-                 unsigned char* dirty, int32_t* sdeg, int32_t* list, int* count, cudaStream_t s);
+// nclust: the cluster count, on the device; touched: scratch, n bytes, where sparse_touches.
+bool sparse_touches(const GraphView& g);
+void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, const int* nclust, unsigned char* mflag,
+                 unsigned char* touched, int32_t* cidm, unsigned char* dirty, int32_t* sdeg, int32_t* list, int* count,
+                 cudaStream_t s);
 void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int32_t* ccount, int64_t c,
                    long long* cbase, long long* cursor, int32_t* seg_key, long long* seg_val, int64_t* coff,
                    int32_t* cadj, long long* cw, int32_t* csrc, long long* nnz_dev, int maxt, bool sort_first,
