@@ -195,6 +195,119 @@ void reduce_pairs(const unsigned long long* keys, const long long* vals, int64_t
   VC_CHECK_LAUNCH();
 }
 
+// ---------------------------------------------------------------- merge in a table
+// Few clusters and many pairs: the pairs are added up in a table of c x c sums (additions in
+// L2 that return nothing), which is then read row by row into the coarse lists.  No pair is
+// sorted or moved, and a cluster's size does not matter.  A sum of 0 is no entry, unless a
+// pair of weight 0 or below went into it (inputs that nothing checked): those are noted in a
+// bit per sum (zero, 32 columns a word).
+__host__ __device__ inline int64_t table_words(int64_t c) { return (c + 31) >> 5; }
+
+
+// W lanes per fine vertex add its pre-merged list to its cluster's row.
+template <int W>
+__global__ void __launch_bounds__(256) table_add_k(int64_t n, const int64_t* __restrict__ off,
+                                                   const int32_t* __restrict__ cid, const int32_t* __restrict__ cnt,
+                                                   PairOut in, int64_t c, long long* __restrict__ sums,
+                                                   unsigned* __restrict__ zero) {
+  const int lane = threadIdx.x & (W - 1);
+  const int64_t groups = (int64_t)gridDim.x * (256 / W);
+  for (int64_t v = ((int64_t)blockIdx.x * 256 + threadIdx.x) / W; v < n; v += groups) {
+    const int32_t x = cid[v];
+    const int k = x >= 0 ? cnt[v] : 0;
+    if (k == 0) continue;
+    const int64_t src = off[v], row = (int64_t)x * c;
+#pragma unroll 4
+    for (int j = lane; j < k; j += W) {
+      int32_t key;
+      long long w;
+      in.get(v, src, j, &key, &w);
+      atomicAdd((unsigned long long*)(sums + row + key), (unsigned long long)w);
+      if (w <= 0) atomicOr(zero + x * table_words(c) + (key >> 5), 1u << (key & 31));
+    }
+  }
+}
+
+// A warp per row: f of each entry, and then of the row.
+constexpr int kTableUnroll = 8;
+template <typename F>
+__device__ __forceinline__ void table_rows(int64_t c, const long long* sums, const unsigned* zero, F f) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < c; x += warps) {
+    const long long* row = sums + x * c;
+    const unsigned* zrow = zero + x * table_words(c);
+    int64_t made = 0;
+    for (int64_t b = 0; b < c; b += 32 * kTableUnroll) {
+      long long w[kTableUnroll];
+      unsigned z[kTableUnroll];
+#pragma unroll
+      for (int q = 0; q < kTableUnroll; ++q) {
+        w[q] = b + 32 * q + lane < c ? row[b + 32 * q + lane] : 0;
+        z[q] = b + 32 * q < c ? zrow[(b >> 5) + q] : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < kTableUnroll; ++q) {
+        const bool in = w[q] != 0 || (z[q] >> lane & 1u);
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        if (in) f(x, made + __popc(bal & ((1u << lane) - 1u)), b + 32 * q + lane, w[q]);
+        made += __popc(bal);
+      }
+    }
+    f(x, made);
+  }
+}
+struct TableCount {
+  int32_t* count;
+  __device__ __forceinline__ void operator()(int64_t, int64_t, int64_t, long long) const {}
+  __device__ __forceinline__ void operator()(int64_t x, int64_t made) const {
+    if ((threadIdx.x & 31) == 0) count[x] = (int32_t)made;
+  }
+};
+struct TableWrite {
+  const int64_t* coff;
+  int32_t* cadj;
+  long long* cw;
+  int32_t* csrc;
+  __device__ __forceinline__ void operator()(int64_t x, int64_t i, int64_t y, long long w) const {
+    const int64_t to = coff[x] + i;
+    cadj[to] = (int32_t)y;
+    cw[to] = w;
+    csrc[to] = (int32_t)x;
+  }
+  __device__ __forceinline__ void operator()(int64_t, int64_t) const {}
+};
+template <typename F>
+__global__ void __launch_bounds__(256) table_rows_k(int64_t c, const long long* __restrict__ sums,
+                                                    const unsigned* __restrict__ zero, F f) {
+  table_rows(c, sums, zero, f);
+}
+
+int64_t table_elems(int64_t c) { return c * c + (c * table_words(c) + 1) / 2; }
+bool table_merge_fits(int64_t c, int64_t pairs) {
+  return c > 0 && c <= (int64_t(1) << 30) && c * c <= 2 * pairs && pairs <= std::max<int64_t>(64 * c * c, 1 << 16);
+}
+
+void table_merge(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int64_t c, int64_t pairs,
+                 long long* sums, int32_t* ccount, int64_t* coff, int32_t* cadj, long long* cw, int32_t* csrc,
+                 long long* nnz_dev, cudaStream_t s) {
+  const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
+  VC_CUDA(cudaMemsetAsync(sums, 0, sizeof(long long) * table_elems(c), s));
+  unsigned* zero = (unsigned*)(sums + c * c);
+  if (pairs <= 2 * g.n)
+    table_add_k<1><<<grid_for(g.n, 256, kSMs * 8), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, c, sums, zero);
+  else if (pairs <= 16 * g.n)
+    table_add_k<8><<<grid_for(g.n, 32, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, c, sums, zero);
+  else
+    table_add_k<32><<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, in, c, sums, zero);
+  const int grid = grid_for(c, 8, kSMs * 8);
+  table_rows_k<<<grid, 256, 0, s>>>(c, sums, zero, TableCount{ccount});
+  exclusive_scan<int, long long>(ccount, (long long*)coff, c, (long long*)coff + c, cs.scan_scr, s, nullptr, nnz_dev);
+  table_rows_k<<<grid, 256, 0, s>>>(c, sums, zero, TableWrite{coff, cadj, cw, csrc});
+  count_launch(3);
+  VC_CHECK_LAUNCH();
+}
+
 // ---------------------------------------------------------------- cluster merge
 // Warp-level grouping of the lanes whose vertices share a cluster (consecutive
 // vertices often do), so that one atomic per group and warp moves its counter.

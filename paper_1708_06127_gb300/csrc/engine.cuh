@@ -624,7 +624,10 @@ struct Workspace {
       longs.at = longAt.ensure_n<long long>(long_list_cap(P));
       longs.n = ctr()->nlong;
     }
-    if (2 * GP <= P || sparse) {
+    if (!sparse && table_merge_fits(c, P)) {
+      auto* sums = (long long*)keysA.ensure_n<unsigned long long>(table_elems(c));
+      table_merge(g, cid_out, cs, c, P, sums, ccount, co, ca, cwp, csp, &st()->nnz, s);
+    } else if (2 * GP <= P || sparse) {
       long long* cbase = pos.as<long long>();  // n + 1 >= c + 1 entries
       long long* cur = ccur.ensure_n<long long>(std::max<int64_t>(c, 1));
       auto* sk = (int32_t*)keysA.ensure_n<unsigned long long>(std::max<int64_t>(P, 1));

@@ -83,3 +83,39 @@ def test_exact_step_batch_classes():
     for g, cut, side in zip(graphs, cuts, bits):
         ref = oracle.viecut(g.offsets, g.adj, g.w, seed=3, lp_iters=2, n0=1 << 40)
         assert cut == ref.cut and np.array_equal(side, ref.side_bits), g.n
+
+
+def check_contract(G, labels):
+    """One contraction against the oracle's, element by element; returns the coarse graph."""
+    labels = np.ascontiguousarray(labels, np.int32)
+    d = vc.viecut_graph_upload(G.offsets, G.adj, G.w)
+    out = None
+    try:
+        out, cid = vc.viecut_step_contract(d, labels)
+        off, adj, w = vc.viecut_graph_download(out)
+        ref, rcid = oracle.contract(G, labels)
+        assert np.array_equal(cid, rcid)
+        assert np.array_equal(off, ref.offsets)
+        assert np.array_equal(adj, ref.adj)
+        assert np.array_equal(w, ref.w)
+        return ref
+    finally:
+        vc.viecut_graph_free(d)
+        if out is not None:
+            vc.viecut_graph_free(out)
+
+
+@pytest.mark.parametrize("n,deg,clusters", [
+    (2000, 300, 2), (2000, 300, 31), (2000, 300, 33), (2000, 300, 255), (2000, 300, 257),  # the table
+    (40, 20, 5), (300, 3, 9),                      # of few pairs; one lane per list
+    (40000, 4, 2), (70000, 4, 2), (70000, 4, 40),  # few sums: up to 65,536 pairs, above, 64 per sum
+    (700, 300, 690)])                              # more sums than pairs would fill
+def test_contract_to_few_clusters(n, deg, clusters):
+    """The merge in a table and both sides of the line where it is taken; one vertex in ten
+    with weights of 0, which leave an entry of weight 0."""
+    g = gg.er(n, deg, 3 + clusters, 1, 100)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    labels = np.random.default_rng(clusters).integers(0, clusters, n)
+    check_contract(G, labels)
+    src = np.repeat(np.arange(n), np.diff(g.offsets))
+    check_contract(oracle.CsrGraph(G.offsets, G.adj, np.where((src % 10 == 0) | (G.adj % 10 == 0), 0, G.w)), labels)
