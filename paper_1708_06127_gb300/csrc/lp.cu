@@ -279,17 +279,31 @@ int64_t global_table_cap(int maxdeg) {
   return c < 64 ? 64 : c;
 }
 
+// Adds x to a sum in shared memory.  32-bit additions with the carry passed on (the upper one
+// is mostly not needed) instead of a 64-bit one: 516 -> 499 us of lp_block_k on 16,001 lists of
+// 1522 entries, 19.8 -> 19.5 ms of lp_warp_k on planted 8 x 2^20.
+__device__ __forceinline__ void shared_add(unsigned* p, unsigned x) { atomicAdd(p, x); }
+__device__ __forceinline__ void shared_add(unsigned long long* p, unsigned long long x) {
+  unsigned* h = (unsigned*)p;
+  const unsigned lo = (unsigned)x, old = atomicAdd(h, lo);
+  const unsigned hi = (unsigned)(x >> 32) + (old + lo < old ? 1u : 0u);
+  if (hi) atomicAdd(h + 1, hi);
+}
+
 // Adds wt to the slot of key k (linear probing; capacity >= 2 x distinct keys, so a
 // free slot always exists and the loop ends within one pass over the table).
 // Returns the slot index if this call created the key, otherwise -1.
-template <typename ACC>
+template <typename ACC, bool GLOBAL = false>
 __device__ __forceinline__ int tbl_add(int* tk, ACC* tv, int lg, int k, long long wt) {
   const uint32_t mask = (1u << lg) - 1u;
   uint32_t h = slot_hash(k, lg);
   for (uint32_t probe = 0; probe <= mask; ++probe) {
     int prev = atomicCAS(&tk[h], kEmptyKey, k);
     if (prev == kEmptyKey || prev == k) {
-      atomicAdd(&tv[h], (ACC)wt);
+      if (GLOBAL)
+        atomicAdd(&tv[h], (ACC)wt);
+      else
+        shared_add(&tv[h], (ACC)wt);
       return prev == kEmptyKey ? (int)h : -1;
     }
     h = (h + 1) & mask;
@@ -317,18 +331,11 @@ struct Chunk {
   long long sum;
 };
 
-template <typename WT, int MODE, bool FIRST>
-__device__ __forceinline__ Chunk load_chunk(int64_t e, int64_t end, const int32_t* __restrict__ adj,
-                                            const WT* __restrict__ w, const int32_t* __restrict__ lab, int32_t own,
-                                            long long* sw, int lane) {
+template <typename WT>
+__device__ __forceinline__ Chunk group_chunk(int32_t k, bool use, long long wt, long long* sw, int lane) {
   Chunk c;
-  c.k = 0;
-  c.use = false;
-  long long wt = 0;
-  if (e < end) {
-    c.use = entry_key<MODE, FIRST>(lab, __ldg(adj + e), own, &c.k);
-    wt = ldw(w, e);
-  }
+  c.k = k;
+  c.use = use;
   // unused lanes get a unique negative key so they form singleton groups
   const int32_t km = c.use ? c.k : (-2 - lane);
   const unsigned peers = __match_any_sync(0xffffffffu, km);
@@ -345,6 +352,20 @@ __device__ __forceinline__ Chunk load_chunk(int64_t e, int64_t end, const int32_
     c.sum = s;
   }
   return c;
+}
+
+template <typename WT, int MODE, bool FIRST>
+__device__ __forceinline__ Chunk load_chunk(int64_t e, int64_t end, const int32_t* __restrict__ adj,
+                                            const WT* __restrict__ w, const int32_t* __restrict__ lab, int32_t own,
+                                            long long* sw, int lane) {
+  int32_t k = 0;
+  bool use = false;
+  long long wt = 0;
+  if (e < end) {
+    use = entry_key<MODE, FIRST>(lab, __ldg(adj + e), own, &k);
+    wt = ldw(w, e);
+  }
+  return group_chunk<WT>(k, use, wt, sw, lane);
 }
 
 // Per-lane running best over (sum, hash, -label); the tie hash of a label is read
@@ -372,6 +393,11 @@ struct LaneBest {
 };
 
 // ------------------------------------------------------------------ warp classes
+// The table kernels gather the labels of several chunks before they add the first: the
+// gathers, not the additions, set their time (lists of 129 to 512 entries, planted
+// 8 x 2^20: 25.2 ms with 1, 19.5 ms with 4, 17.1 ms with 8).
+constexpr int kLpTableChunks = 8;
+
 // Label propagation with a per-warp table.  LISTED = false: every vertex of list
 // length <= CAP/2 (grid-stride over all vertices); LISTED = true: the listed vertices.
 // The slots a vertex creates are recorded, so the final argmax visits only them.
@@ -412,12 +438,27 @@ __global__ void __launch_bounds__(kAggThreads) lp_warp_k(
     }
     const int lg = ceil_log2(2 * (int64_t)d);
     int created = 0;  // warp-uniform count of recorded slots
-    for (int64_t base = beg; base < end; base += 32) {
-      Chunk c = load_chunk<WT, kModeLP, FIRST>(base + lane, end, adj, w, lab, 0, sw, lane);
-      const int slot = c.leader ? tbl_add<ACC>(tk, tv, lg, c.k, c.sum) : -1;
-      const unsigned bal = __ballot_sync(0xffffffffu, slot >= 0);
-      if (slot >= 0) slots[created + __popc(bal & ((1u << lane) - 1u))] = slot;
-      created += __popc(bal);
+    for (int64_t base = beg; base < end; base += 32 * kLpTableChunks) {
+      int32_t k[kLpTableChunks];
+      long long wt[kLpTableChunks];
+#pragma unroll
+      for (int q = 0; q < kLpTableChunks; ++q) {
+        const int64_t e = base + 32 * q + lane;
+        k[q] = e < end ? __ldg(adj + e) : -1;
+        wt[q] = e < end ? ldw(w, e) : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < kLpTableChunks; ++q)
+        if (!FIRST && k[q] >= 0) k[q] = __ldg(lab + k[q]);
+#pragma unroll
+      for (int q = 0; q < kLpTableChunks; ++q) {
+        if (base + 32 * q >= end) break;  // the same in every lane
+        const Chunk c = group_chunk<WT>(k[q], k[q] >= 0, wt[q], sw, lane);
+        const int slot = c.leader ? tbl_add<ACC>(tk, tv, lg, c.k, c.sum) : -1;
+        const unsigned bal = __ballot_sync(0xffffffffu, slot >= 0);
+        if (slot >= 0) slots[created + __popc(bal & ((1u << lane) - 1u))] = slot;
+        created += __popc(bal);
+      }
     }
     __syncwarp();
     LaneBest lb;
@@ -1222,16 +1263,23 @@ __global__ void __launch_bounds__(kAggThreads) emit_split_k(const int32_t* __res
 
 // --------------------------------------------------------- block / global classes
 // Label propagation, one block per listed vertex; the table lives in shared memory
-// (GLOBAL = false) or in this block's region of global scratch (GLOBAL = true).
+// (GLOBAL = false) or in this block's region of global scratch (GLOBAL = true).  In shared
+// memory the table's 96 KB admit two blocks per SM, so they have 16 warps each, and most
+// lists are kLpBlockChunks chunks per warp or fewer: 16,001 lists of 1522 entries 714 us with
+// 8 warps and a chunk at a time, 500 us (560 us with 8 chunks, whose registers and tests go
+// unused).  Half the slots (1.25 per entry) took 684 us in probes, twice as many 514 us.
+constexpr int lp_block_threads(bool global) { return global ? kAggThreads : 512; }
+constexpr int kLpBlockChunks = 4;
 template <typename WT, typename ACC, bool FIRST, bool GLOBAL>
-__global__ void __launch_bounds__(kAggThreads) lp_block_k(
+__global__ void __launch_bounds__(lp_block_threads(GLOBAL)) lp_block_k(
     const int32_t* __restrict__ list, const int* __restrict__ count_ptr, const int64_t* __restrict__ off,
     const int32_t* __restrict__ adj, const WT* __restrict__ w, const int32_t* __restrict__ lab,
     int32_t* __restrict__ lab_out, const unsigned long long* __restrict__ hv, int32_t* __restrict__ gkeys,
     long long* __restrict__ gvals, int64_t gcap, const unsigned char* __restrict__ vact) {
   extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ Cand s_best[kWarpsPerBlock];
-  __shared__ long long s_w[kWarpsPerBlock][32];
+  constexpr int BT = lp_block_threads(GLOBAL), NW = BT / 32;
+  __shared__ Cand s_best[NW];
+  __shared__ long long s_w[NW][32];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   int* tk;
   ACC* tv;
@@ -1246,7 +1294,7 @@ __global__ void __launch_bounds__(kAggThreads) lp_block_k(
     table_cap = kBlockCap;
   }
   long long* sw = s_w[wib];
-  for (int64_t i = threadIdx.x; i < table_cap; i += kAggThreads) { tk[i] = kEmptyKey; tv[i] = 0; }
+  for (int64_t i = threadIdx.x; i < table_cap; i += BT) { tk[i] = kEmptyKey; tv[i] = 0; }
   __syncthreads();
   const int count = *count_ptr;
   for (int idx = blockIdx.x; idx < count; idx += gridDim.x) {
@@ -1256,13 +1304,28 @@ __global__ void __launch_bounds__(kAggThreads) lp_block_k(
     const int64_t d = end - beg;
     const int lg = ceil_log2(2 * d);
     const int64_t cap = (int64_t)1 << lg;
-    for (int64_t base = beg + 32 * wib; base < end; base += 32 * kWarpsPerBlock) {
-      Chunk c = load_chunk<WT, kModeLP, FIRST>(base + lane, end, adj, w, lab, 0, sw, lane);
-      if (c.leader) tbl_add<ACC>(tk, tv, lg, c.k, c.sum);
+    for (int64_t base = beg + 32 * wib; base < end; base += 32 * NW * kLpBlockChunks) {
+      int32_t k[kLpBlockChunks];
+      long long wt[kLpBlockChunks];
+#pragma unroll
+      for (int q = 0; q < kLpBlockChunks; ++q) {
+        const int64_t e = base + 32 * NW * q + lane;
+        k[q] = e < end ? __ldg(adj + e) : -1;
+        wt[q] = e < end ? ldw(w, e) : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < kLpBlockChunks; ++q)
+        if (!FIRST && k[q] >= 0) k[q] = __ldg(lab + k[q]);
+#pragma unroll
+      for (int q = 0; q < kLpBlockChunks; ++q) {
+        if (base + 32 * NW * q >= end) break;  // the same in every lane
+        const Chunk c = group_chunk<WT>(k[q], k[q] >= 0, wt[q], sw, lane);
+        if (c.leader) tbl_add<ACC, GLOBAL>(tk, tv, lg, c.k, c.sum);
+      }
     }
     __syncthreads();
     LaneBest lb;
-    for (int64_t i = threadIdx.x; i < cap; i += kAggThreads) {
+    for (int64_t i = threadIdx.x; i < cap; i += BT) {
       const int L = tk[i];
       if (L != kEmptyKey) {
         lb.add((long long)tv[i], L, hv);
@@ -1275,7 +1338,7 @@ __global__ void __launch_bounds__(kAggThreads) lp_block_k(
     __syncthreads();
     if (threadIdx.x == 0) {
       Cand b = s_best[0];
-      for (int q = 1; q < kWarpsPerBlock; ++q)
+      for (int q = 1; q < NW; ++q)
         if (better(s_best[q], b)) b = s_best[q];
       lab_out[v] = b.l;
     }
@@ -1328,8 +1391,8 @@ void launch_lp(const GraphView& g, const Bins& b, const GlobalTables& gt, const 
     const size_t smem = (size_t)kBlockCap * (sizeof(ACC) + sizeof(int));
     auto kfn = lp_block_k<WT, ACC, FIRST, false>;
     set_smem(kfn, smem);
-    kfn<<<grid_for(b.h_block, 1, kSMs * 2), kAggThreads, smem, s>>>(b.block_list, b.counts + 1, g.off, g.adj, w,
-                                                                   lab, lab_out, key, nullptr, nullptr, 0, g.vact);
+    kfn<<<grid_for(b.h_block, 1, kSMs * 2), lp_block_threads(false), smem, s>>>(
+        b.block_list, b.counts + 1, g.off, g.adj, w, lab, lab_out, key, nullptr, nullptr, 0, g.vact);
     count_launch();
     VC_CHECK_LAUNCH();
   }
