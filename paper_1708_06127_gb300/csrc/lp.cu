@@ -1051,18 +1051,8 @@ __global__ void __launch_bounds__(kAggThreads) lp_first_simple_block_k(const int
 // the first lane holding the id writes the pair; the cluster merge that follows merges
 // equal ids across chunks and across vertices.  `next_slot` yields the pair's index.
 template <typename WT, int G, typename SLOT>
-__device__ __forceinline__ void emit_chunk(int64_t e, int64_t end, const int32_t* __restrict__ adj,
-                                           const WT* __restrict__ w, const int32_t* __restrict__ cid, int32_t own,
-                                           int lane, unsigned gmask, const PairOut& out, int64_t v, int64_t beg,
-                                           SLOT next_slot) {
-  int32_t k = -1;
-  long long wt = 0;
-  bool use = false;
-  if (e < end) {
-    k = __ldg(cid + __ldg(adj + e));
-    use = k != own;
-    wt = ldw(w, e);
-  }
+__device__ __forceinline__ void emit_chunk(int32_t k, bool use, long long wt, int lane, unsigned gmask,
+                                           const PairOut& out, int64_t v, int64_t beg, SLOT next_slot) {
   unsigned todo = __ballot_sync(gmask, use) & gmask;
   while (todo) {
     const int leader = __ffs(todo) - 1;
@@ -1088,18 +1078,8 @@ __device__ __forceinline__ void emit_chunk(int64_t e, int64_t end, const int32_t
 // distinct keys of the chunk (lists whose neighbours are nearly all in clusters of their
 // own).  `reserve(k)` returns the index of the chunk's first of k pairs.
 template <typename WT, int G, typename RESERVE>
-__device__ __forceinline__ void emit_chunk_rows(int64_t e, int64_t end, const int32_t* __restrict__ adj,
-                                                const WT* __restrict__ w, const int32_t* __restrict__ cid,
-                                                int32_t own, int lane, unsigned gmask, const PairOut& out, int64_t v,
-                                                int64_t beg, RESERVE reserve) {
-  int32_t k = -1;
-  long long wt = 0;
-  bool use = false;
-  if (e < end) {
-    k = __ldg(cid + __ldg(adj + e));
-    use = k != own;
-    wt = ldw(w, e);
-  }
+__device__ __forceinline__ void emit_chunk_rows(int32_t k, bool use, long long wt, int lane, unsigned gmask,
+                                                const PairOut& out, int64_t v, int64_t beg, RESERVE reserve) {
   const unsigned long long tag = use ? (unsigned long long)(uint32_t)k : (0xffffffff00000000ull | (unsigned)lane);
   const unsigned peers = __match_any_sync(gmask, tag);
   const bool lead = use && (__ffs(peers) - 1) == lane;
@@ -1137,6 +1117,33 @@ __device__ __forceinline__ bool emit_many_keys(int64_t e, int64_t end, const int
   return __popc(__ballot_sync(gmask, use && (__ffs(peers) - 1) == lane) & gmask) > kEmitWalkKeys;
 }
 
+// f(k, use, wt) for every chunk of a list from entry e on, `step` entries apart: the cluster
+// ids of kEmitChunks chunks are gathered before the first is worked on (16,001 lists of 1522
+// entries: 363 -> 344 us, 2326 coarse ones of 1345: 152 -> 130 us).
+constexpr int kEmitChunks = 4;
+template <typename WT, typename F>
+__device__ __forceinline__ void emit_chunks(int64_t base, int glane, int64_t end, int64_t step,
+                                            const int32_t* __restrict__ adj, const WT* __restrict__ w,
+                                            const int32_t* __restrict__ cid, int32_t own, F f) {
+  for (; base < end; base += kEmitChunks * step) {
+    int32_t k[kEmitChunks];
+    long long wt[kEmitChunks];
+#pragma unroll
+    for (int q = 0; q < kEmitChunks; ++q) {
+      const int64_t e = base + q * step + glane;
+      k[q] = e < end ? __ldg(adj + e) : -1;
+      wt[q] = e < end ? ldw(w, e) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < kEmitChunks; ++q) k[q] = k[q] >= 0 ? __ldg(cid + k[q]) : own;
+#pragma unroll
+    for (int q = 0; q < kEmitChunks; ++q) {
+      if (base + q * step >= end) break;  // the same in every lane of the group
+      f(k[q], k[q] != own, wt[q]);
+    }
+  }
+}
+
 // Listed vertices (the mid and block classes), G lanes per vertex: 32 / G vertices
 // per warp, each group walking its list in G-entry chunks.
 template <typename WT, int G>
@@ -1158,16 +1165,17 @@ __global__ void __launch_bounds__(kAggThreads) emit_warp_k(const int32_t* __rest
     int made = 0;  // group-uniform
     if (own >= 0) {
       if (rows || emit_many_keys<G>(beg + glane, end, adj, cid, own, lane, gmask))
-        for (int64_t base = beg; base < end; base += G)
-          emit_chunk_rows<WT, G>(base + glane, end, adj, w, cid, own, lane, gmask, out, v, beg, [&](int k) {
+        emit_chunks(beg, glane, end, G, adj, w, cid, own, [&](int32_t k, bool use, long long wt) {
+          emit_chunk_rows<WT, G>(k, use, wt, lane, gmask, out, v, beg, [&](int pairs) {
             const int at = made;
-            made += k;
+            made += pairs;
             return at;
           });
+        });
       else
-        for (int64_t base = beg; base < end; base += G)
-          emit_chunk<WT, G>(base + glane, end, adj, w, cid, own, lane, gmask, out, v, beg,
-                            [&](int) { return made++; });
+        emit_chunks(beg, glane, end, G, adj, w, cid, own, [&](int32_t k, bool use, long long wt) {
+          emit_chunk<WT, G>(k, use, wt, lane, gmask, out, v, beg, [&](int) { return made++; });
+        });
     }
     if (glane == 0) {
       cnt[v] = made;
@@ -1195,19 +1203,21 @@ __global__ void __launch_bounds__(kAggThreads) emit_block_k(const int32_t* __res
     __syncthreads();
     if (own >= 0) {
       if (rows || emit_many_keys<32>(beg + 32 * wib + lane, end, adj, cid, own, lane, 0xffffffffu))
-        for (int64_t base = beg + 32 * wib; base < end; base += 32 * kWarpsPerBlock)
-          emit_chunk_rows<WT, 32>(base + lane, end, adj, w, cid, own, lane, 0xffffffffu, out, v, beg, [&](int k) {
+        emit_chunks(beg + 32 * wib, lane, end, kAggThreads, adj, w, cid, own, [&](int32_t k, bool use, long long wt) {
+          emit_chunk_rows<WT, 32>(k, use, wt, lane, 0xffffffffu, out, v, beg, [&](int pairs) {
             int at = 0;
-            if (lane == 0) at = atomicAdd(&s_made, k);
+            if (lane == 0) at = atomicAdd(&s_made, pairs);
             return __shfl_sync(0xffffffffu, at, 0);
           });
+        });
       else
-        for (int64_t base = beg + 32 * wib; base < end; base += 32 * kWarpsPerBlock)
-          emit_chunk<WT, 32>(base + lane, end, adj, w, cid, own, lane, 0xffffffffu, out, v, beg, [&](int leader) {
+        emit_chunks(beg + 32 * wib, lane, end, kAggThreads, adj, w, cid, own, [&](int32_t k, bool use, long long wt) {
+          emit_chunk<WT, 32>(k, use, wt, lane, 0xffffffffu, out, v, beg, [&](int leader) {
             int at = 0;
             if (lane == leader) at = atomicAdd(&s_made, 1);
             return __shfl_sync(0xffffffffu, at, leader);
           });
+        });
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1245,16 +1255,17 @@ __global__ void __launch_bounds__(kAggThreads) emit_split_k(const int32_t* __res
     if (own < 0) continue;  // the same in every thread
     if (threadIdx.x == 0) s_made = 0;
     __syncthreads();
-    for (int64_t base = beg + 32 * ((int64_t)G.part * kWarpsPerBlock + wib); base < end;
-         base += 32 * (int64_t)kWarpsPerBlock * G.parts)
-      emit_chunk_rows<WT, 32>(base + lane, end, adj, w, cid, own, lane, 0xffffffffu, out, v, beg, [&](int k) {
-        int at = 0;
-        if (lane == 0) {
-          at = atomicAdd(cnt + v, k);
-          atomicAdd(&s_made, k);
-        }
-        return __shfl_sync(0xffffffffu, at, 0);
-      });
+    emit_chunks(beg + 32 * ((int64_t)G.part * kWarpsPerBlock + wib), lane, end, (int64_t)kAggThreads * G.parts, adj, w,
+                cid, own, [&](int32_t k, bool use, long long wt) {
+                  emit_chunk_rows<WT, 32>(k, use, wt, lane, 0xffffffffu, out, v, beg, [&](int pairs) {
+                    int at = 0;
+                    if (lane == 0) {
+                      at = atomicAdd(cnt + v, pairs);
+                      atomicAdd(&s_made, pairs);
+                    }
+                    return __shfl_sync(0xffffffffu, at, 0);
+                  });
+                });
     __syncthreads();
     if (threadIdx.x == 0 && out.ccount && s_made) atomicAdd(&out.ccount[own], s_made);
     __syncthreads();
