@@ -119,3 +119,139 @@ def test_contract_to_few_clusters(n, deg, clusters):
     check_contract(G, labels)
     src = np.repeat(np.arange(n), np.diff(g.offsets))
     check_contract(oracle.CsrGraph(G.offsets, G.adj, np.where((src % 10 == 0) | (G.adj % 10 == 0), 0, G.w)), labels)
+
+
+LENGTHS = (1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65, 127, 128, 129, 257, 511, 512, 513, 1025, 2049, 4095, 4096,
+           4097)
+
+
+def lengths_graph(weights):
+    """Vertices of exactly the list lengths at the edges of the kernels' classes, over 12,000
+    leaves that form a ring."""
+    rng = np.random.default_rng(len(weights))
+    n, first = 12000 + len(LENGTHS), 12000
+    pairs = [(v, (v + 1) % 12000) for v in range(12000)]
+    for i, d in enumerate(LENGTHS):
+        pairs += [(int(u), first + i) for u in rng.choice(12000, d, replace=False)]
+    return gg.from_edges(n, [(a, b, int(x)) for (a, b), x in zip(pairs, rng.choice(weights, len(pairs)))])
+
+
+@pytest.mark.parametrize("weights", [(1,), (1, 2, 9), (1 << 20, 1 << 30)])
+def test_list_lengths(weights):
+    """Label rounds (from the identity, from others' labels with few and with many distinct
+    ones) and contractions by them; whole runs, which take input weights in 32 bits."""
+    g = lengths_graph(weights)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    key = oracle.level_key(4, 0)
+    rng = np.random.default_rng(8)
+    for start in (np.arange(G.n), rng.integers(0, 3, G.n), rng.permutation(G.n)):
+        start = start.astype(np.int32)
+        ref = oracle.lp_round(G, start, key)
+        d = vc.viecut_graph_upload(G.offsets, G.adj, G.w)
+        try:
+            assert np.array_equal(vc.viecut_step_lp(d, start, key, 1)[0], ref)
+        finally:
+            vc.viecut_graph_free(d)
+        check_contract(G, ref)
+    for n0 in (10, 1000):
+        ref = oracle.viecut(g.offsets, g.adj, g.w, seed=5, lp_iters=2, n0=n0)
+        with vc.MinCut(g.offsets, g.adj, g.w, n0=n0) as mc:
+            cut, bits = mc.run(5, 2)
+            assert mc.trace() == ref.trace
+        assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
+
+
+PAIRS = (2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 2047, 2048, 2049,
+         4095, 4096, 4097, 5000)
+
+
+@pytest.mark.parametrize("sparse", [True, False])
+def test_contract_cluster_pairs(sparse):
+    """Clusters of two vertices with exactly the pair counts at the edges of the merge's
+    classes, half of the targets in both lists; the other clusters single vertices, under
+    their own ids or another's."""
+    rng = np.random.default_rng(2)
+    leaves, edges = 9000, []
+    for i, t in enumerate(PAIRS):
+        us = rng.choice(leaves, t // 2 + t % 2, replace=False)
+        a = leaves + 2 * i
+        edges += [(int(u), a, int(rng.integers(1, 50))) for u in us]
+        vs = np.concatenate([us[:t // 4], rng.choice(np.setdiff1d(np.arange(leaves), us), t // 2 - t // 4,
+                                                     replace=False)])
+        edges += [(int(u), a + 1, int(rng.integers(1, 50))) for u in vs]
+    n = leaves + 2 * len(PAIRS)
+    g = gg.from_edges(n, edges + [(v, (v + 1) % leaves, 3) for v in range(leaves)])
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    labels = np.arange(n) if sparse else np.roll(np.arange(n), 1)
+    labels[leaves + 1::2] = labels[leaves::2]
+    check_contract(G, labels)
+
+
+@pytest.mark.parametrize("n", [16383, 16384, 16385, 32767, 32769])
+def test_contract_vertex_counts(n):
+    """Vertex counts at the edge of the one-block scan."""
+    g = ring_graph(n, 5, 1, 9)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    near = np.arange(n)
+    near[1::400] = near[0::400][:len(near[1::400])]
+    for labels in (near, np.random.default_rng(1).permutation(n) // 2, np.arange(n) // 3):
+        check_contract(G, labels)
+
+
+def test_contract_large_near_identity():
+    """Graphs of more than 2^25 entries where few vertices merge: the lists next to a merged
+    group are the only ones read (up to a sixteenth of the vertices), the others renumbered by
+    the run (up to one in 512), also those of a hub and of vertices under another's id."""
+    g = gg.er(700_000, 50, 3, 1, 100)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    n = G.n
+    assert G.nnz >= 1 << 25
+    rng = np.random.default_rng(6)
+    labels = np.arange(n)
+    labels[rng.choice(n, 200, replace=False)] = 77
+    hub = check_contract(G, labels)  # 77: a list of about 10,000 entries
+    assert np.diff(hub.offsets).max() > 4096
+    for gone in (hub.n // 512 - 8, hub.n // 512 + 8, hub.n // 16 + 8):
+        labels = np.arange(hub.n)
+        pick = rng.choice(hub.n, 2 * gone, replace=False)
+        labels[pick[:gone]] = labels[pick[gone:]]
+        labels[pick[0]] = int(np.diff(hub.offsets).argmax())
+        check_contract(hub, labels)
+    labels = np.arange(hub.n)
+    a, b = rng.choice(hub.n, (2, 50), replace=False)
+    labels[a], labels[b] = b, a
+    check_contract(hub, labels)
+
+
+def test_run_of_changed_lists_and_hubs():
+    """A graph whose levels run many passes over the lists that the last one changed, with
+    hubs of more than 4096 entries from merges, both ends of some pairs long."""
+    g = gg.planted(4, 1 << 15, 24, 8, 3)
+    ref = oracle.viecut(g.offsets, g.adj, g.w, seed=2, lp_iters=2, n0=1000)
+    with vc.MinCut(g.offsets, g.adj, g.w, n0=1000) as mc:
+        for _ in range(2):  # the second run finds every workspace in place
+            cut, bits = mc.run(2, 2)
+            assert mc.trace() == ref.trace
+            assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+def test_converging_rounds_with_a_hub(weighted):
+    """Rounds over the neighbours of changed vertices only, a hub among them."""
+    base = gg.core_lcc(gg.rhg(1 << 16, 16, 12), 0)
+    if weighted:
+        base = gg.with_pair_weights(base, 4, 1, 9)
+    src = np.repeat(np.arange(base.n), np.diff(base.offsets))
+    hub = np.random.default_rng(3).choice(base.n, 6000, replace=False)
+    one = np.ones(6000, np.int32)
+    a = np.concatenate([src, hub, np.full(6000, base.n)])
+    b = np.concatenate([base.adj, np.full(6000, base.n), hub])
+    w = np.concatenate([base.w, one, one])
+    order = np.lexsort((b, a))
+    off = np.concatenate([[0], np.cumsum(np.bincount(a, minlength=base.n + 1))]).astype(np.int64)
+    adj, w = b[order].astype(np.int32), w[order].astype(np.int32)
+    ref = oracle.viecut(off, adj, w, seed=3, lp_iters=25, n0=500, converge=True)
+    with vc.MinCut(off, adj, w, n0=500, lp_converge=True) as mc:
+        cut, bits = mc.run(3, 25)
+        assert mc.trace() == ref.trace
+    assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
