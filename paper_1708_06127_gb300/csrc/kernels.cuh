@@ -402,7 +402,7 @@ struct BatchNoi {
   int trace_cap;
   const int* level;
 };
-// Blocks per SM of the batches' dense exact step (512 threads and 32 registers each).
+// Blocks per SM that the batches' dense exact step is launched for, each with matrices of its own.
 constexpr int kNoiDenseBlocksPerSM = 4;
 // Dense rounds for the listed graphs of a union u (vertex range [vbase[g], +nv[g])),
 // `blocks` persistent blocks with 2 x mcap matrix entries and kDenseMax curK each;

@@ -301,12 +301,14 @@ __global__ void pr_a_edge_k(int64_t n, const int32_t* __restrict__ src, const in
 // Union-find start for pass A on sorted lists: each vertex points at its smallest
 // marked neighbour below it (or at itself).  Every such pointer is a union of a
 // marked edge towards a smaller id, so this is a valid forest with min-id roots,
-// shallow from the start; the per-entry pass then finds short paths.  Eight lanes per
-// vertex read its list in rows of eight ascending entries (four rows at a time) and stop
-// at the first row holding a marked entry below v or an entry at or above v.
+// shallow from the start; the per-entry pass then finds short paths.  A start is only a
+// start: eight lanes per vertex look at the first 32 entries of its list, in four rows of
+// eight, and a vertex without a marked neighbour among them stays its own.  Each further 32
+// entries cost three dependent loads and the per-entry pass is no slower without them
+// (planted 8 x 2^20, 12 passes: 9.7 ms with 1024 entries, 7.4 with 128, 3.8 with 32, the
+// per-entry pass 11.0 to 11.5 ms each time; 2326 vertices of 1345 entries: 100, 16, 7 us).
 constexpr int kInitMinG = 8;
 constexpr int kInitMinRows = 4;
-constexpr int kInitMinReach = 1024;
 template <typename WT>
 __global__ void uf_init_min_k(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
                               const WT* __restrict__ w, const DevState* st, int32_t* __restrict__ parent,
@@ -320,37 +322,25 @@ __global__ void uf_init_min_k(int64_t n, const int64_t* __restrict__ off, const 
     long long lam;
     const int64_t beg = off[v], end = off[v + 1];
     if (end - beg >= 2 && pr_graph(bc, st, v, &lam)) {
-      bool found = false;
-      // a start is only a start: a vertex without a marked neighbour among its first
-      // kInitMinReach stays its own (a hub's eight lanes would walk on alone)
-      const int64_t reach = end - beg > kInitMinReach ? beg + kInitMinReach : end;
-      for (int64_t b = beg; b < reach && !found; b += kInitMinRows * G) {
-        // kInitMinRows rows in flight: ids, then the weights of the entries below v,
-        // then the list lengths of the heavy ones
-        int u[kInitMinRows];
-        bool mk[kInitMinRows];
+      // the rows in flight: ids, then the weights of the entries below v, then the list
+      // lengths of the heavy ones
+      int u[kInitMinRows];
+      bool mk[kInitMinRows];
 #pragma unroll
-        for (int r = 0; r < kInitMinRows; ++r) {
-          const int64_t e = b + r * G + glane;
-          u[r] = e < end ? adj[e] : INT_MAX;
-        }
+      for (int r = 0; r < kInitMinRows; ++r) {
+        const int64_t e = beg + r * G + glane;
+        u[r] = e < end ? adj[e] : INT_MAX;
+      }
 #pragma unroll
-        for (int r = 0; r < kInitMinRows; ++r) mk[r] = u[r] < v && (long long)w[b + r * G + glane] >= lam;
+      for (int r = 0; r < kInitMinRows; ++r) mk[r] = u[r] < v && (long long)w[beg + r * G + glane] >= lam;
 #pragma unroll
-        for (int r = 0; r < kInitMinRows; ++r) mk[r] = mk[r] && off[u[r] + 1] - off[u[r]] >= 2;
+      for (int r = 0; r < kInitMinRows; ++r) mk[r] = mk[r] && off[u[r] + 1] - off[u[r]] >= 2;
 #pragma unroll
-        for (int r = 0; r < kInitMinRows; ++r) {
-          const unsigned mb = __ballot_sync(gmask, mk[r]);
-          const unsigned past = __ballot_sync(gmask, !(u[r] < v));
-          if (mb) {  // sorted: the lowest marked lane holds the smallest marked neighbour
-            p = __shfl_sync(gmask, u[r], __ffs(mb) - 1);
-            found = true;
-            break;
-          }
-          if (past) {  // no smaller neighbour follows
-            found = true;
-            break;
-          }
+      for (int r = 0; r < kInitMinRows; ++r) {
+        const unsigned mb = __ballot_sync(gmask, mk[r]);
+        if (mb) {  // sorted: the lowest marked lane holds the smallest marked neighbour
+          p = __shfl_sync(gmask, u[r], __ffs(mb) - 1);
+          break;
         }
       }
     }
