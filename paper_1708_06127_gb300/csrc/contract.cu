@@ -921,7 +921,7 @@ __device__ __forceinline__ int sc_collect(int64_t beg, int64_t end, int lane, co
 // entries: 1.25 ms a pass over every list, whatever the pass merged (one random gather per
 // entry, at 0.8 of one per SM and cycle); 31.0 -> 17.2 ms for its 25 contractions.  Below
 // kScPushMin entries a pass costs less than the marking: 8 x 60,000 (18.7 million entries)
-// took 1.9 ms with it, 1.6 ms without.
+// took 1.6 ms with it, 1.4 ms without.
 constexpr int64_t kScPushMin = int64_t(1) << 25;
 __device__ __forceinline__ bool sc_few(int64_t n, const int* nclust) { return 16 * (n - __ldg(nclust)) <= n; }
 

@@ -900,7 +900,7 @@ void launch_lp_bailed(const GraphView& g, const Bins& b, const WT* w, const int3
 // slots per lane, where a step per distinct label is costly) with many distinct labels
 // go on to the hash-table kernel (the bail list and counts[7] are free during label
 // propagation: the pre-merge uses them later).  Lists of at most 128 entries keep the
-// walk: four slots per lane make each step cheap, and measured, the table kernel did not
+// walk: few slots per lane make each step cheap, and measured, the table kernel did not
 // beat it there.
 template <typename WT, typename ACC, bool FIRST>
 void launch_lp_reg(const GraphView& g, const Bins& b, const WT* w, const int32_t* lab, int32_t* lab_out,
