@@ -16,6 +16,7 @@ struct GraphView {
   int wbytes = 8;
   bool unit = false;
   bool simple = false;  // every list strictly increasing (no parallel entries)
+  bool wraps = false;   // 64-bit weights nothing checked: their sums may leave 64 bits
   // batches: label propagation touches only vertices v with vact[v] != 0 (null: all)
   const unsigned char* vact = nullptr;
   // source vertex of every entry (contracted graphs; null when not built)

@@ -89,6 +89,12 @@ __device__ __forceinline__ int warp_argmax_unseen(const long long* r, const int*
 // is raised to 0 when it is chosen), so that one addition tests, raises and takes, and
 // the untaken vertex of largest attachment holds the largest r read as unsigned.
 //
+// A vertex is taken at most once whatever the weights, so the queue (n places) never
+// overflows: a weight above lam counts as lam (which crosses it as the weight itself does),
+// and so does a negative one, which only an input that nothing checked can hold; and on
+// graphs whose sums may leave 64 bits (GraphView::wraps) a taken vertex is not added to any
+// more, so that r cannot come back below 0 around the end of its range either.
+//
 // Measured (RHG n = 8191, average degree 32, unit weights: 612 runs, 2174 levels): 1.66 ms a
 // round, about 1400 cycles a level (450 of them the lists' L2 access) and 1100 a choice,
 // against 4.47 ms for one warp over the same state.  8 and 4 warps take 1.70 and 2.05 ms;
@@ -103,8 +109,8 @@ struct NoiShared {
 };
 
 // The state in shared memory.  R = int serves graphs in which lam x entries stays below
-// 2^31: weights are cut to lam (which crosses it as the weight itself does), so no sum
-// wraps.  kOff: the list offsets are kept too (they are read from goff otherwise).
+// 2^31, so no sum of weights of at most lam wraps.  kOff: the list offsets are kept too
+// (they are read from goff otherwise).
 template <typename RT, typename OT, bool kOff>
 struct ClosureSmem {
   using R = RT;
@@ -176,10 +182,22 @@ __device__ __forceinline__ bool noi_fits32(long long lam, int64_t entries) {
   return lam < INT_MAX && entries < INT_MAX && (lam > 1 ? lam : 1) * entries < INT_MAX;
 }
 
-// Shared-memory additions of either width (the 64-bit one is declared unsigned).
+// Additions of either width (the 64-bit one is declared unsigned); the value before.  WRAPS:
+// a value that is no longer negative stays as it is (each failed exchange is another's
+// addition, so the loop ends).
+template <bool WRAPS>
 __device__ __forceinline__ int noi_add(int* p, int x) { return atomicAdd(p, x); }
+template <bool WRAPS>
 __device__ __forceinline__ long long noi_add(long long* p, long long x) {
-  return (long long)atomicAdd((unsigned long long*)p, (unsigned long long)x);
+  unsigned long long* q = (unsigned long long*)p;
+  if constexpr (!WRAPS) return (long long)atomicAdd(q, (unsigned long long)x);
+  unsigned long long old = atomicAdd(q, 0ull);
+  while ((long long)old < 0) {
+    const unsigned long long seen = atomicCAS(q, old, old + (unsigned long long)x);
+    if (seen == old) break;
+    old = seen;
+  }
+  return (long long)old;
 }
 
 constexpr int kNoiUnroll = 4;  // rows of a list in flight per warp while relaxing
@@ -187,7 +205,7 @@ constexpr int kNoiUnroll = 4;  // rows of a list in flight per warp while relaxi
 // One round by a block of NW warps (a power of two), one graph at a time.  put(x, m)
 // receives every vertex x with the smallest id m of its run.  Returns, in every thread,
 // whether some run holds two or more vertices.  Ends with a barrier.
-template <int NW, typename WT, typename ST, typename PUT>
+template <int NW, bool WRAPS = false, typename WT, typename ST, typename PUT>
 __device__ __forceinline__ bool noi_closure_block(int32_t lo, int n, const int32_t* __restrict__ adj,
                                                   const WT* __restrict__ w, long long lam_in, const ST& S,
                                                   NoiShared& sh, PUT put) {
@@ -281,7 +299,7 @@ __device__ __forceinline__ bool noi_closure_block(int32_t lo, int n, const int32
             if (e < len) {
               y[q] = __ldg(a + e) - lo;
               const long long x64 = ldw(w, e0 + beg + e);
-              c[q] = (sizeof(R) == 4 && x64 > (long long)lam) ? lam : (R)x64;
+              c[q] = (unsigned long long)x64 > (unsigned long long)lam ? lam : (R)x64;
             }
           }
 #pragma unroll
@@ -289,10 +307,10 @@ __device__ __forceinline__ bool noi_closure_block(int32_t lo, int n, const int32
             if (row + q * P * 32 >= len) break;  // the same in every lane
             bool join = false;
             if (y[q] >= 0) {
-              const R old = noi_add(&S.r[y[q]], c[q]), now = old + c[q];
+              const R old = noi_add<WRAPS>(&S.r[y[q]], c[q]), now = (R)((U)old + (U)c[q]);
               join = old < 0 && now >= 0;  // the addition that crosses lam takes the vertex
               if constexpr (ST::kBounds)
-                if (now < 0) atomicMax(&S.cmax[y[q] >> 5], (U)now);
+                if ((old & now) < 0) atomicMax(&S.cmax[y[q] >> 5], (U)now);
             }
             const unsigned b = __ballot_sync(0xffffffffu, join);
             if (b) {
@@ -725,7 +743,7 @@ __host__ __device__ constexpr size_t noi_round_smem(int ncap) { return (size_t)(
 // The listed graphs (list null: the one graph of n1 vertices with bound st->lambda_hat),
 // a block at a time each.  Graphs of at most ncap vertices keep their state in shared
 // memory; the others in r (values at the vertex), cmax (chunk bounds) and queue.
-template <typename WT, int NW>
+template <typename WT, int NW, bool WRAPS>
 __global__ void __launch_bounds__(NW * 32) noi_round_k(
     const int32_t* __restrict__ list, int count, int64_t n1, const DevState* st, const long long* __restrict__ vbase,
     const long long* __restrict__ nv, const long long* __restrict__ glam, const int64_t* __restrict__ off,
@@ -744,7 +762,7 @@ __global__ void __launch_bounds__(NW * 32) noi_round_k(
     bool any;
     if (n > ncap) {
       const ClosureGlobal S{r + lo, cmax + lo, queue + lo, goff, e0};
-      any = noi_closure_block<NW>((int32_t)lo, n, adj, w, lam, S, sh, put);
+      any = noi_closure_block<NW, WRAPS>((int32_t)lo, n, adj, w, lam, S, sh, put);
     } else if (noi_fits32(lam, goff[n] - e0)) {
       ClosureSmem<int, int32_t, true> S;
       S.r = (int*)noi_rs;
@@ -752,7 +770,7 @@ __global__ void __launch_bounds__(NW * 32) noi_round_k(
       S.queue = (uint16_t*)(S.soff + n + 1);
       S.goff = goff;
       S.e0 = e0;
-      any = noi_closure_block<NW>((int32_t)lo, n, adj, w, lam, S, sh, put);
+      any = noi_closure_block<NW, WRAPS>((int32_t)lo, n, adj, w, lam, S, sh, put);
     } else {
       ClosureSmem<long long, int64_t, false> S;
       S.r = (long long*)noi_rs;
@@ -760,18 +778,18 @@ __global__ void __launch_bounds__(NW * 32) noi_round_k(
       S.queue = (uint16_t*)(S.r + ((n + 3) & ~3));
       S.goff = goff;
       S.e0 = e0;
-      any = noi_closure_block<NW>((int32_t)lo, n, adj, w, lam, S, sh, put);
+      any = noi_closure_block<NW, WRAPS>((int32_t)lo, n, adj, w, lam, S, sh, put);
     }
     if (any && threadIdx.x == 0) atomicOr(list ? changed + g : changed, 1);
   }
 }
 
-template <int NW, typename WT>
+template <int NW, typename WT, bool WRAPS = false>
 static void noi_round_launch(const GraphView& u, const int32_t* list, int count, const DevState* st,
                              const long long* vbase, const long long* nv, const long long* glam, long long* r,
                              int32_t* queue, int32_t* labels, int* changed, int ncap, cudaStream_t s) {
-  noi_set_smem(noi_round_k<WT, NW>, noi_round_smem(kNoiSmemRoundMaxN));
-  noi_round_k<WT, NW><<<std::min(count, kSMs * 8), NW * 32, noi_round_smem(ncap), s>>>(
+  noi_set_smem(noi_round_k<WT, NW, WRAPS>, noi_round_smem(kNoiSmemRoundMaxN));
+  noi_round_k<WT, NW, WRAPS><<<std::min(count, kSMs * 8), NW * 32, noi_round_smem(ncap), s>>>(
       list, count, u.n, st, vbase, nv, glam, u.off, u.adj, (const WT*)u.w, r, (unsigned long long*)r + u.n, queue,
       labels, changed, ncap);
   count_launch();
@@ -794,7 +812,11 @@ void noi_round_sparse(const GraphView& g, const DevState* st, long long* r, int3
                       int* changed, cudaStream_t s) {
   // parent (n entries) holds the queue of taken vertices
   const int ncap = (int)std::min<int64_t>(g.n, kNoiSmemRoundMaxN);
-  noi_round_by_weight<16>(g, nullptr, 1, st, nullptr, nullptr, nullptr, r, parent, labels, changed, ncap, s);
+  if (g.wraps)
+    noi_round_launch<16, long long, true>(g, nullptr, 1, st, nullptr, nullptr, nullptr, r, parent, labels, changed,
+                                          ncap, s);
+  else
+    noi_round_by_weight<16>(g, nullptr, 1, st, nullptr, nullptr, nullptr, r, parent, labels, changed, ncap, s);
 }
 
 void noi_round_batch(const GraphView& u, const int32_t* list, int count, const long long* vbase, const long long* nv,

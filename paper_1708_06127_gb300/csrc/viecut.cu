@@ -429,6 +429,7 @@ struct StepGraph {
   int64_t n = 0, nnz = 0;
   bool simple = false;
   bool unit = false;  // every weight is 1: the kernels that can then read no weights
+  bool wraps = false; // sums of the weights may leave 64 bits
   Buf off, adj, w;
   GraphView view() const {
     GraphView g;
@@ -440,6 +441,7 @@ struct StepGraph {
     g.wbytes = 8;
     g.simple = simple;
     g.unit = unit;
+    g.wraps = wraps;
     return g;
   }
 };
@@ -752,6 +754,11 @@ int viecut_graph_upload(viecut_graph** g, const int64_t* offsets, const int32_t*
         if (adj[e + 1] <= adj[e]) { x->g.simple = false; break; }
     x->g.unit = true;
     for (int64_t e = 0; e < nnz && x->g.unit; ++e) x->g.unit = weights[e] == 1;
+    uint64_t sum = 0;  // of the weights' magnitudes, until it passes 2^61
+    for (int64_t e = 0; e < nnz && !x->g.unit && !x->g.wraps; ++e) {
+      const uint64_t a = weights[e] < 0 ? 0 - (uint64_t)weights[e] : (uint64_t)weights[e];
+      x->g.wraps = a >> 61 || (sum += a) >> 61;
+    }
     VC_CUDA(cudaMemcpy(x->g.off.ensure_n<int64_t>(n + 1), offsets, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice));
     x->g.adj.ensure_n<int32_t>(nnz);
     x->g.w.ensure_n<long long>(nnz);
@@ -889,6 +896,7 @@ int viecut_step_contract(viecut_graph* g, const int32_t* labels, viecut_graph** 
     x->g.n = h.n;
     x->g.nnz = nnz;
     x->g.simple = true;
+    x->g.wraps = g->g.wraps;
     VC_CUDA(cudaMemcpyAsync(x->g.off.ensure_n<int64_t>(h.n + 1), h.off, sizeof(int64_t) * (h.n + 1),
                             cudaMemcpyDeviceToDevice, c.s));
     VC_CUDA(cudaMemcpyAsync(x->g.adj.ensure_n<int32_t>(nnz), h.adj, sizeof(int32_t) * nnz, cudaMemcpyDeviceToDevice, c.s));

@@ -1,5 +1,7 @@
 """Kernels at the edges of their size and value ranges, against the oracle (every value a
 whole number, compared exactly)."""
+import heapq
+
 import numpy as np
 import pytest
 
@@ -46,6 +48,56 @@ def test_exact_round_sizes_and_weights(n, wlo, whi):
             assert ch == (1 if cnt > 0 else 0)
     finally:
         vc.viecut_graph_free(d)
+
+
+def any_round(G, lam):
+    """A round in whole numbers of any size (maximum-adjacency order, ties to the smallest id):
+    every vertex's smallest joined id."""
+    r, seen, parent = [0] * G.n, [False] * G.n, list(range(G.n))
+
+    def find(x):
+        while parent[x] != x:
+            parent[x] = x = parent[parent[x]]
+        return x
+
+    off, adj, w = G.offsets.tolist(), G.adj.tolist(), G.w.tolist()
+    heap = [(0, v) for v in range(G.n)]
+    while heap:
+        rx, x = heapq.heappop(heap)
+        if seen[x] or -rx != r[x]:
+            continue
+        seen[x] = True
+        for e in range(off[x], off[x + 1]):
+            y = adj[e]
+            if seen[y]:
+                continue
+            r[y] += w[e]
+            heapq.heappush(heap, (-r[y], y))
+            if r[y] >= lam:
+                a, b = sorted((find(x), find(y)))
+                parent[b] = a
+    return [find(v) for v in range(G.n)]
+
+
+@pytest.mark.parametrize("n", [2, 40, 513, 4000, 16384, 16390])
+def test_exact_round_unchecked_weights(n):
+    """A step takes any 64-bit weights: those below 0 count as the bound, sums may pass 2^63,
+    and every vertex is still taken exactly once."""
+    g = ring_graph(n, 3 + n, 1, 9)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    src = np.repeat(np.arange(n), np.diff(G.offsets))
+    mixed = np.where((src * 7 + G.adj * 7) % 5 < 2, -G.w, G.w)
+    huge = (1 << 60) * np.minimum(G.w, 7)
+    for w, bounds in ((mixed, (1, 5, 20, 1 << 40)), (huge, (1, 1 << 60, (1 << 62) + 5, (1 << 63) - 1))):
+        d = vc.viecut_graph_upload(G.offsets, G.adj, w)
+        try:
+            for lam in bounds:
+                ref = any_round(oracle.CsrGraph(G.offsets, G.adj, np.where(w < 0, lam, w)), lam)
+                got, ch = vc.viecut_step_noi_round(d, lam)
+                assert np.array_equal(got, ref), lam
+                assert ch == int(any(ref[v] != v for v in range(n)))
+        finally:
+            vc.viecut_graph_free(d)
 
 
 @pytest.mark.parametrize("wlo,whi", [(1, 1), (1, 9), (1 << 20, 1 << 30)])
