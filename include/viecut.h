@@ -59,7 +59,10 @@ typedef struct viecut_opts {
   void* stream;        /* cudaStream_t for all work; NULL = the library creates one */
   int32_t validate;    /* 0 = trust input; 1 = range/loop/weight/offset checks, one pass on
                           the device (default); 2 = the same checks plus symmetry, on the
-                          host (create from host arrays; O(m log m)) */
+                          host (create from host arrays; O(m log m)).  With 0 and 1 it is the
+                          caller who sees to it that every edge appears in both directions:
+                          with 0 nothing looks, and with 1 a graph that is not symmetric is
+                          accepted, but the cut it gets stands for nothing */
   int32_t timing;      /* 1 = record per-phase CUDA-event times (viecut_get_stats) */
   int32_t lp_group;    /* lanes per vertex of the first-round label-propagation kernel:
                           8, 16 or 32, or 0 = pick by timing once per handle (default);

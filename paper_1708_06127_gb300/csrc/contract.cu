@@ -915,7 +915,8 @@ __device__ __forceinline__ int sc_collect(int64_t beg, int64_t end, int lane, co
 }
 
 // A contraction that merges few vertices touches few lists: the neighbours of the merged
-// groups' members (every edge is in both lists), found from the members' own.  They are
+// groups' members (every edge is in both lists: GraphView::symmetric), found from the
+// members' own.  They are
 // marked so (touched) while at most a sixteenth of the vertices disappears, and pass 1 then
 // reads only those lists; otherwise it reads every list.  Planted 8 x 2^20, 392 million
 // entries: 1.25 ms a pass over every list, whatever the pass merged (one random gather per
@@ -1339,7 +1340,7 @@ void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, con
   VC_CHECK_LAUNCH();
 }
 
-bool sparse_touches(const GraphView& g) { return g.nnz >= kScPushMin; }
+bool sparse_touches(const GraphView& g) { return g.symmetric && g.nnz >= kScPushMin; }
 
 static void sparse_finish_degrees(const GraphView& g, const int32_t* cid, const int32_t* sdeg, int32_t* ccount,
                                   unsigned char* clean, int64_t c, cudaStream_t s) {

@@ -75,6 +75,7 @@ struct Counters {
   int nprlong;        // pairs listed by pass B (PrLong)
   int nab[2];         // vertices whose list is new for pass A, for pass B
   int changed;
+  unsigned long long asym;  // validation: 0 where every entry has its reverse
 };
 
 // What the host reads at its decision points, in one copy.
@@ -470,7 +471,7 @@ struct Workspace {
   // n / 10000 labels (one count and host read per round).  A vertex's choice follows from its
   // neighbours' labels alone, so from the first round on that changed few labels (one vertex in
   // kFewChanged at most) only the neighbours of those vertices choose again: each edge is in
-  // both lists, so they are found from the changed vertices' own.  RHG n = 300,000, average
+  // both lists (GraphView::symmetric), so they are found from the changed vertices' own.  RHG n = 300,000, average
   // degree 32, 24 rounds: 2.75 ms a run over all vertices each round, 2.44 ms so (what is left
   // of a round is launches and the host's read).
   static constexpr int64_t kFewChanged = 32;  // 1 / 32
@@ -519,7 +520,7 @@ struct Workspace {
         sync();
         const long long changed = h_counters->gpairs;
         if (changed * 10000 <= g.n) break;
-        if (!few && changed * kFewChanged <= g.n && r + 1 < rounds) {
+        if (!few && g.symmetric && changed * kFewChanged <= g.n && r + 1 < rounds) {
           few = true;
           mark_ = smflag.ensure_n<unsigned char>(g.n);
           VC_CUDA(cudaMemsetAsync(mark_, 0, (size_t)g.n, s));
@@ -683,6 +684,7 @@ struct Workspace {
     h.src = csp;
     h.wbytes = 8;
     h.simple = true;
+    h.symmetric = g.symmetric;
     bins_valid = false;
     return h;
   }

@@ -16,6 +16,9 @@ struct GraphView {
   int wbytes = 8;
   bool unit = false;
   bool simple = false;  // every list strictly increasing (no parallel entries)
+  // Every entry has its reverse.  False only where something relies on it (sparse_touches,
+  // converging label rounds) and the input was found otherwise; those then read every list.
+  bool symmetric = true;
   bool wraps = false;   // 64-bit weights nothing checked: their sums may leave 64 bits
   // batches: label propagation touches only vertices v with vact[v] != 0 (null: all)
   const unsigned char* vact = nullptr;
@@ -276,7 +279,8 @@ struct MergeLists {
   int32_t *small, *large;
   int* n;
 };
-// nclust: the cluster count, on the device; touched: scratch, n bytes, where sparse_touches.
+// nclust: the cluster count, on the device; touched: scratch, n bytes, where sparse_touches
+// (the lists next to a merged group are then found from its members' own).
 bool sparse_touches(const GraphView& g);
 void sparse_mark(const GraphView& g, const int32_t* lab, const int32_t* cid, const int* nclust, unsigned char* mflag,
                  unsigned char* touched, int32_t* cidm, unsigned char* dirty, int32_t* sdeg, int32_t* list, int* count,

@@ -35,9 +35,13 @@ bool take_injected_alloc_failure() {
   return false;
 }
 
+// asym (may be null): *asym += a hash of every entry's unordered pair, taken from the lower id's
+// list and subtracted from the higher one's: 0 where every entry has its reverse (as many times),
+// and otherwise with a chance of 2^-64.
 __global__ void validate_k(int64_t n, int64_t m, const int64_t* __restrict__ off, const int32_t* __restrict__ adj,
-                           const int32_t* __restrict__ w, int* err) {
+                           const int32_t* __restrict__ w, int* err, unsigned long long* asym) {
   int bad = 0;
+  unsigned long long pairs = 0;
   const int64_t T = (int64_t)gridDim.x * blockDim.x;
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t0 == 0 && (off[0] != 0 || off[n] != m)) bad |= 1;
@@ -53,6 +57,11 @@ __global__ void validate_k(int64_t n, int64_t m, const int64_t* __restrict__ off
       int32_t u = adj[e];
       if (u < 0 || u >= n) bad |= 4;
       else if (u == v) bad |= 8;
+      if (asym) {
+        const uint64_t lo = u < v ? (uint32_t)u : (uint64_t)v, hi = u < v ? (uint64_t)v : (uint32_t)u;
+        const uint64_t x = mix64(lo << 32 | hi);
+        pairs += u < v ? 0 - x : x;
+      }
       if (w) {  // null: the weights are checked apart (weight_check_k)
         if (w[e] < 1) bad |= 16;
         if (w[e] != 1) bad |= 32;  // not an error: the weights are not all 1
@@ -61,6 +70,10 @@ __global__ void validate_k(int64_t n, int64_t m, const int64_t* __restrict__ off
     }
   }
   if (bad) atomicOr(err, bad);
+  if (asym) {
+    pairs = warp_sum(pairs);
+    if (lane == 0 && pairs) atomicAdd(asym, pairs);
+  }
 }
 
 // Weights alone, an entry per thread: 16 = a weight < 1, 32 = not all weights 1.
@@ -88,6 +101,7 @@ struct Handle {
   int lp_async = 0;          // asynchronous rounds in shuffled blocks (2: with the first round's restriction)
   bool unit = false;    // every input weight is 1 (found by validation)
   bool simple = false;  // every input list strictly increasing (found by validation)
+  bool symmetric = true;  // GraphView::symmetric (false only as found by validation)
   bool host_input = false;  // the graph was copied from host arrays into in_*
   bool bound = false;       // a graph passed validation and may run
   cudaStream_t cstream = nullptr;  // viecut_solve: the weights' copy and check
@@ -108,20 +122,30 @@ struct Handle {
   }
 };
 
+// Whether a run on an m-entry graph would rely on every entry having its reverse.
+static bool relies_on_symmetry(int64_t m, bool lp_converge) {
+  GraphView g;
+  g.nnz = m;
+  return lp_converge || sparse_touches(g);
+}
+
 // with_weights = false: the weights are checked apart (viecut_solve); unit is then
 // left as the caller set it.
 static void device_validate(Handle& H, bool with_weights = true) {
   Workspace& W = *H.ws;
   int* err = &W.ctr()->changed;
+  unsigned long long* asym = relies_on_symmetry(H.m, H.lp_converge) ? &W.ctr()->asym : nullptr;
   VC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), H.stream));
+  VC_CUDA(cudaMemsetAsync(&W.ctr()->asym, 0, sizeof(unsigned long long), H.stream));
   validate_k<<<grid_for(H.n, 256, kSMs * 8), 256, 0, H.stream>>>(H.n, H.m, H.off0, H.adj0,
-                                                                with_weights ? H.w0 : nullptr, err);
+                                                                with_weights ? H.w0 : nullptr, err, asym);
   count_launch();
   VC_CHECK_LAUNCH();
   W.read_state();
   int bad = W.h_counters->changed;
   if (with_weights) H.unit = (bad & 32) == 0;
   H.simple = (bad & 64) == 0;
+  H.symmetric = W.h_counters->asym == 0;
   bad &= ~(32 | 64);
   if (bad) {
     std::string why;
@@ -193,6 +217,7 @@ static void run_impl(Handle& H, uint64_t seed, int lp_iters, long long* d_cut, u
   G.wbytes = 4;
   G.unit = H.unit;
   G.simple = H.simple;
+  G.symmetric = H.symmetric;
   W.bins_valid = false;
   W.flags_ok = W.carried = false;
 
@@ -428,6 +453,7 @@ struct StepGraph {
   int device = 0;
   int64_t n = 0, nnz = 0;
   bool simple = false;
+  bool symmetric = true;
   bool unit = false;  // every weight is 1: the kernels that can then read no weights
   bool wraps = false; // sums of the weights may leave 64 bits
   Buf off, adj, w;
@@ -440,6 +466,7 @@ struct StepGraph {
     g.w = w.p;
     g.wbytes = 8;
     g.simple = simple;
+    g.symmetric = symmetric;
     g.unit = unit;
     g.wraps = wraps;
     return g;
@@ -513,6 +540,7 @@ static void bind_graph(vc::Handle& H, bool host_input, const int64_t* off, const
   H.m = m;
   H.unit = unit;
   H.simple = simple;
+  H.symmetric = true;
   H.host_input = host_input;
   if (host_input) {
     H.off0 = H.in_off.ensure_n<int64_t>(n + 1);
@@ -766,6 +794,19 @@ int viecut_graph_upload(viecut_graph** g, const int64_t* offsets, const int32_t*
       VC_CUDA(cudaMemcpy(x->g.adj.p, adj, sizeof(int32_t) * nnz, cudaMemcpyHostToDevice));
       VC_CUDA(cudaMemcpy(x->g.w.p, weights, sizeof(int64_t) * nnz, cudaMemcpyHostToDevice));
     }
+    if (vc::relies_on_symmetry(nnz, false)) {
+      vc::Buf found;
+      unsigned long long* asym = found.ensure_n<unsigned long long>(2);
+      VC_CUDA(cudaMemset(asym, 0, 2 * sizeof(unsigned long long)));
+      vc::validate_k<<<vc::grid_for(n, 256, vc::kSMs * 8), 256>>>(n, nnz, x->g.off.as<int64_t>(),
+                                                                  x->g.adj.as<int32_t>(), nullptr, (int*)(asym + 1),
+                                                                  asym);
+      vc::count_launch();
+      VC_CHECK_LAUNCH();
+      unsigned long long a = 0;
+      VC_CUDA(cudaMemcpy(&a, asym, sizeof(a), cudaMemcpyDeviceToHost));
+      x->g.symmetric = a == 0;
+    }
   } catch (...) {
     delete x;
     throw;
@@ -897,6 +938,7 @@ int viecut_step_contract(viecut_graph* g, const int32_t* labels, viecut_graph** 
     x->g.nnz = nnz;
     x->g.simple = true;
     x->g.wraps = g->g.wraps;
+    x->g.symmetric = g->g.symmetric;
     VC_CUDA(cudaMemcpyAsync(x->g.off.ensure_n<int64_t>(h.n + 1), h.off, sizeof(int64_t) * (h.n + 1),
                             cudaMemcpyDeviceToDevice, c.s));
     VC_CUDA(cudaMemcpyAsync(x->g.adj.ensure_n<int32_t>(nnz), h.adj, sizeof(int32_t) * nnz, cudaMemcpyDeviceToDevice, c.s));

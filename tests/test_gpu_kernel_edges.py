@@ -307,3 +307,33 @@ def test_converging_rounds_with_a_hub(weighted):
         cut, bits = mc.run(3, 25)
         assert mc.trace() == ref.trace
     assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
+
+
+def dropped(g, share, seed):
+    """The graph without a random share of its entries, so that some edges are in one list only."""
+    keep = np.random.default_rng(seed).random(len(g.adj)) >= share
+    off = np.concatenate([[0], np.cumsum(keep)])[g.offsets].astype(np.int64)
+    return off, g.adj[keep], g.w[keep]
+
+
+def test_contract_large_not_symmetric():
+    """More than 2^25 entries, some edges in one list only: a list next to a merged group cannot
+    be found from the group's own."""
+    G = oracle.as_csr64(*dropped(gg.er(700_000, 60, 3, 1, 100), 0.15, 1))
+    assert G.nnz >= 1 << 25
+    rng = np.random.default_rng(6)
+    for gone in (200, G.n // 16 - 8):
+        labels = np.arange(G.n)
+        pick = rng.choice(G.n, 2 * gone, replace=False)
+        labels[pick[:gone]] = labels[pick[gone:]]
+        G = check_contract(G, labels)
+
+
+def test_converging_rounds_not_symmetric():
+    """Converging rounds where a vertex may follow one that does not list it."""
+    off, adj, w = dropped(gg.core_lcc(gg.rhg(1 << 18, 24, 12), 0), 0.2, 2)
+    ref = oracle.viecut(off, adj, w, seed=3, lp_iters=25, n0=500, pr_runs_max=0, converge=True)
+    with vc.MinCut(off, adj, w, n0=500, pr_runs_max=0, lp_converge=True) as mc:
+        cut, bits = mc.run(3, 25)
+        assert mc.trace() == ref.trace
+    assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
