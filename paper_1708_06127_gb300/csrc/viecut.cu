@@ -971,6 +971,11 @@ static int step_labels(viecut_graph* g, int64_t lambda_hat, int32_t* labels, int
     else
       vc::pr_pass_b(v, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), W.st(), lab, chg, c.s);
   } else {
+    // every entry reaches a bound below 1, one of weight 0 too: as unit weights reach 1
+    if (lambda_hat < 1) {
+      v.unit = true;
+      v.wraps = false;
+    }
     W.noi_r.ensure_n<long long>(vc::noi_round_scratch(v.n));
     vc::noi_round_sparse(v, W.st(), W.noi_r.as<long long>(), W.parent.as<int32_t>(),
                          lab, chg, c.s);

@@ -100,6 +100,25 @@ def test_exact_round_unchecked_weights(n):
             vc.viecut_graph_free(d)
 
 
+@pytest.mark.parametrize("n", [2, 40, 513, 3000, 16390])
+def test_exact_round_zero_weights(n):
+    """Entries of weight 0: they join their ends where the bound is below 1, and only there."""
+    g = ring_graph(n, 5 + n, 1, 9)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    src = np.repeat(np.arange(n), np.diff(G.offsets))
+    for w in (np.where((src + G.adj) % 3 == 0, G.w, 0), np.zeros(G.nnz, np.int64)):
+        Z = oracle.CsrGraph(G.offsets, G.adj, w)
+        d = vc.viecut_graph_upload(Z.offsets, Z.adj, Z.w)
+        try:
+            for lam in (-3, 0, 1, 2, 12):
+                got, ch = vc.viecut_step_noi_round(d, lam)
+                ref, cnt = oracle.noi_round(Z, lam)
+                assert np.array_equal(got, ref), lam
+                assert ch == (1 if cnt > 0 else 0)
+        finally:
+            vc.viecut_graph_free(d)
+
+
 @pytest.mark.parametrize("wlo,whi", [(1, 1), (1, 9), (1 << 20, 1 << 30)])
 @pytest.mark.parametrize("n", [2, 5, 33, 150, 151, 400, 512, 600])
 def test_exact_step_whole(n, wlo, whi):
