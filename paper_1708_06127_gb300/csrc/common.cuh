@@ -7,6 +7,8 @@
 #include <atomic>
 #include <string>
 
+#include "smem_limit.h"
+
 namespace vc {
 
 // ------------------------------------------------------------ error handling
@@ -38,6 +40,18 @@ inline int grid_for(int64_t work, int per_block, int max_blocks) {
 // reported beside timings.
 extern std::atomic<unsigned long long> g_launches;  // host threads of servers count too
 inline void count_launch(int k = 1) { g_launches += (unsigned long long)k; }
+
+// Opts a kernel into `bytes` of dynamic shared memory (above the 48 KB every kernel may use)
+// on the current device.
+extern SmemLimits g_smem_limits;
+template <typename F>
+inline void set_smem(F kfn, size_t bytes) {
+  int dev = 0;
+  VC_CUDA(cudaGetDevice(&dev));
+  g_smem_limits.require((const void*)kfn, dev, bytes, [&] {
+    VC_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  });
+}
 
 // ------------------------------------------------------------ device helpers
 // SplitMix64 output function (Steele, Lea, Flood 2014).

@@ -13,10 +13,7 @@
 #include <limits.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <type_traits>
-#include <unordered_map>
 
 #include "kernels.cuh"
 #include "prims.cuh"
@@ -1350,20 +1347,6 @@ static void sparse_finish_degrees(const GraphView& g, const int32_t* cid, const 
   VC_CHECK_LAUNCH();
 }
 
-// Opts a copy kernel into its table, once per kernel and device.
-template <typename F>
-static void sc_copy_smem(F kfn) {
-  static std::mutex mu;
-  static std::map<std::pair<const void*, int>, bool> ready;
-  int dev = 0;
-  VC_CUDA(cudaGetDevice(&dev));
-  std::lock_guard<std::mutex> lk(mu);
-  bool& done = ready[{(const void*)kfn, dev}];
-  if (!done)
-    VC_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, kScTab * (int)sizeof(int32_t)));
-  done = true;
-}
-
 static void sparse_copy(const GraphView& g, int64_t c, const SparseCtx& sp, const int64_t* coff, int32_t* cadj,
                         long long* cw, int32_t* csrc, cudaStream_t s) {
   const bool table = 512 * (g.n - c) <= g.n && g.nnz >= kScPushMin;
@@ -1375,7 +1358,7 @@ static void sparse_copy(const GraphView& g, int64_t c, const SparseCtx& sp, cons
   sc_by_weight(g, [&](auto wp) {
     using WT = std::remove_cv_t<std::remove_pointer_t<decltype(wp)>>;
     if (table) {
-      sc_copy_smem(sc_copy_k<WT>);
+      set_smem(sc_copy_k<WT>, kScTab * sizeof(int32_t));
       sc_copy_k<WT><<<grid_for(g.n, kScCopyThreads / 32, kSMs * 8), kScCopyThreads, sizeof(int32_t) * runs, s>>>(
           g.n, shift, sp.tab, sp.cidm, g.off, g.adj, wp, sp.dirty, coff, cadj, cw, csrc);
       count_launch();
@@ -1585,21 +1568,6 @@ void cluster_stats(int64_t n, const int32_t* ccount, int* maxt, long long* pairs
   VC_CHECK_LAUNCH();
 }
 
-// Opts cluster_merge_block_k into its shared-memory size, once per device.
-static int merge_block_smem() {
-  static std::mutex mu;
-  static std::unordered_map<int, bool> ready;  // per device: the shared-memory limit was raised
-  const int smem = kMergeBlockSmem;
-  int dev = 0;
-  VC_CUDA(cudaGetDevice(&dev));
-  std::lock_guard<std::mutex> lk(mu);
-  if (!ready[dev]) {
-    VC_CUDA(cudaFuncSetAttribute(cluster_merge_block_k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    ready[dev] = true;
-  }
-  return smem;
-}
-
 __global__ void block_class_list_k(int64_t c, const long long* __restrict__ cbase, int32_t* __restrict__ list,
                                    int* __restrict__ count) {
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < c; x += (int64_t)gridDim.x * blockDim.x) {
@@ -1659,8 +1627,8 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
     // blocks visit only them (blist: n ints no longer needed once the scatter ran; its count,
     // like the other lists' here, starts from zero)
     block_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, blist, blist_n);
-    const int smem = merge_block_smem();
-    cluster_merge_block_k<<<kSMs * 3, 256, smem, s>>>(c, cbase, seg_key, seg_val, ccount, blist, blist_n);
+    set_smem(cluster_merge_block_k, kMergeBlockSmem);
+    cluster_merge_block_k<<<kSMs * 3, 256, kMergeBlockSmem, s>>>(c, cbase, seg_key, seg_val, ccount, blist, blist_n);
     count_launch(2);
     VC_CHECK_LAUNCH();
   }

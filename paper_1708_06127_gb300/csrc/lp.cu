@@ -18,9 +18,7 @@
 #include <limits.h>
 
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
-#include <unordered_map>
 
 #include "kernels.cuh"
 #include "prims.cuh"
@@ -880,8 +878,6 @@ __global__ void __launch_bounds__(kAggThreads) emit_reg_k(const int32_t* __restr
 
 template <int CAP, typename ACC>
 constexpr size_t warp_smem();
-template <typename F>
-void set_smem(F kfn, size_t bytes);
 
 // The vertices a register-class kernel handed on: a warp per vertex with a hash table of
 // CAP slots in shared memory (the bail list and its count are read on the device).
@@ -1355,18 +1351,6 @@ __global__ void __launch_bounds__(lp_block_threads(GLOBAL)) lp_block_k(
     }
     __syncthreads();
   }
-}
-
-// Opts a kernel into more than 48 KB of dynamic shared memory, once per kernel.
-template <typename F>
-void set_smem(F kfn, size_t bytes) {
-  static std::mutex mu;
-  static std::unordered_map<const void*, size_t> done;
-  std::lock_guard<std::mutex> lock(mu);
-  auto it = done.find((const void*)kfn);
-  if (it != done.end() && it->second >= bytes) return;
-  VC_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  done[(const void*)kfn] = bytes;
 }
 
 template <int CAP, typename ACC>

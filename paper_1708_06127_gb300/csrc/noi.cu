@@ -10,7 +10,6 @@
 #include <limits.h>
 
 #include <algorithm>
-#include <map>
 #include <mutex>
 #include <string>
 #include <type_traits>
@@ -603,25 +602,12 @@ __global__ void __launch_bounds__(kNoiThreads) noi_dense_k(int n, const int64_t*
 // (beside the body's own arrays, below the 227 KB of a block).
 constexpr int kNoiDenseSmem = 150 * 150;
 
-// Opts a kernel into its dynamic shared memory, once per kernel and device.
-template <typename F>
-static void noi_set_smem(F kfn, size_t bytes) {
-  static std::mutex mu;
-  static std::map<std::pair<const void*, int>, bool> ready;
-  int dev = 0;
-  VC_CUDA(cudaGetDevice(&dev));
-  std::lock_guard<std::mutex> lk(mu);
-  bool& done = ready[{(const void*)kfn, dev}];
-  if (!done) VC_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  done = true;
-}
-
 template <typename WT>
 static void noi_dense_launch(const GraphView& g, long long* M0, long long* M1, int32_t* curK, unsigned char* sideK,
                              DevState* st, TraceStep* trace, int trace_cap, int level, cudaStream_t s) {
   const int n = (int)g.n;
   const int scap = std::min(n * n, kNoiDenseSmem);
-  noi_set_smem(noi_dense_k<WT>, sizeof(long long) * kNoiDenseSmem);
+  set_smem(noi_dense_k<WT>, sizeof(long long) * kNoiDenseSmem);
   noi_dense_k<WT><<<1, kNoiThreads, sizeof(long long) * scap, s>>>(n, g.off, g.adj, (const WT*)g.w, M0, M1, curK,
                                                                    sideK, st, trace, trace_cap, level, scap);
   count_launch();
@@ -788,7 +774,7 @@ template <int NW, typename WT, bool WRAPS = false>
 static void noi_round_launch(const GraphView& u, const int32_t* list, int count, const DevState* st,
                              const long long* vbase, const long long* nv, const long long* glam, long long* r,
                              int32_t* queue, int32_t* labels, int* changed, int ncap, cudaStream_t s) {
-  noi_set_smem(noi_round_k<WT, NW, WRAPS>, noi_round_smem(kNoiSmemRoundMaxN));
+  set_smem(noi_round_k<WT, NW, WRAPS>, noi_round_smem(kNoiSmemRoundMaxN));
   noi_round_k<WT, NW, WRAPS><<<std::min(count, kSMs * 8), NW * 32, noi_round_smem(ncap), s>>>(
       list, count, u.n, st, vbase, nv, glam, u.off, u.adj, (const WT*)u.w, r, (unsigned long long*)r + u.n, queue,
       labels, changed, ncap);

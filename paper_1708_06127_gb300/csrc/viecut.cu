@@ -18,6 +18,7 @@
 namespace vc {
 
 std::atomic<unsigned long long> g_launches{0};
+SmemLimits g_smem_limits;
 static thread_local std::string t_last_error;
 void set_last_error(const std::string& msg) { t_last_error = msg; }
 

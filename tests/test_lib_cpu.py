@@ -128,3 +128,46 @@ def test_fault_injection_arguments(lib):
     assert vc.lib().viecut_debug_fail_device_allocs(-1, 1) == vc.VIECUT_EINVAL
     assert vc.lib().viecut_debug_fail_device_allocs(0, -1) == vc.VIECUT_EINVAL
     assert vc.lib().viecut_debug_fail_device_allocs(0, 0) == vc.VIECUT_OK
+
+
+def test_shared_memory_limit_is_raised_per_device(tmp_path):
+    """A kernel's shared-memory limit belongs to one device: each device that runs the kernel
+    raises it, once, and a raise that failed is tried again."""
+    src = tmp_path / "limits.cpp"
+    src.write_text("""
+#include <cassert>
+#include <stdexcept>
+#include "smem_limit.h"
+int main() {
+  vc::SmemLimits limits;
+  int a = 0, b = 0, calls = 0;
+  auto require = [&](const void* kernel, int device, size_t bytes) {
+    const int before = calls;
+    limits.require(kernel, device, bytes, [&] { ++calls; });
+    return calls - before;
+  };
+  assert(require(&a, 0, 1000) == 1 && require(&a, 0, 1000) == 0 && require(&a, 0, 999) == 0);
+  assert(require(&a, 1, 1000) == 1 && require(&a, 1, 1000) == 0);
+  assert(require(&b, 0, 1000) == 1 && require(&b, 1, 500) == 1);
+  assert(require(&a, 0, 2000) == 1 && require(&a, 1, 1000) == 0 && require(&a, 1, 2000) == 1);
+  bool thrown = false;
+  try {
+    limits.require(&b, 2, 1000, [] { throw std::runtime_error("no"); });
+  } catch (const std::runtime_error&) {
+    thrown = true;
+  }
+  assert(thrown && require(&b, 2, 1000) == 1 && require(&b, 2, 1000) == 0);
+}
+""")
+    import subprocess
+    exe = tmp_path / "limits"
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_1708_06127_gb300", "csrc"), str(src), "-o",
+                    str(exe), "-lpthread"], check=True)
+    subprocess.run([str(exe)], check=True)
+
+
+def test_shared_memory_limits_are_raised_in_one_place():
+    """Every opt-in goes through the helper that keeps them by device."""
+    csrc = os.path.join(ROOT, "paper_1708_06127_gb300", "csrc")
+    found = {f: open(os.path.join(csrc, f)).read().count("cudaFuncSetAttribute(") for f in os.listdir(csrc)}
+    assert {f: k for f, k in found.items() if k} == {"common.cuh": 1}
