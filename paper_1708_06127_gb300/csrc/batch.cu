@@ -1035,10 +1035,14 @@ struct Server {
   int64_t solo_completed = 0;
 };
 
-static int64_t request_estimate(int64_t n, int64_t m) {
-  // union CSR + workspace share per entry and per vertex (see DESIGN: memory layout)
-  return 96 * (m + n) + 112 * n + (1 << 16);
-}
+// Device memory of one request.  Per vertex, every array of that size on a solo lane (which has
+// the most): the workspace's own 145 bytes, the sparse contraction's marks and lists 40, the
+// arrays carried between Padberg-Rinaldi passes 26, two coarse graphs' offsets 16, the cluster
+// merge's lists and cursor 16, the exact step's values and bounds 16, the input's offsets and the
+// side's bits 9 (a union's slot has 4 + 9 more of its own and neither marks nor carried arrays).
+// Per entry: the input 8, the pre-merged pairs 12, two coarse graphs 32, and the merge of the
+// pairs that are left between clusters.
+static int64_t request_estimate(int64_t n, int64_t m) { return 96 * m + 272 * n + (1 << 16); }
 
 static int64_t arena_alloc(Server& S, int64_t n) {
   for (;;) {
