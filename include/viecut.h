@@ -108,7 +108,7 @@ typedef struct viecut_stats {
                             8(n+1) offsets + nnz (4 id + weight bytes + 4 label gather,
                             no gather in a level's first round) + 4n label writes; a round
                             of lp_converge over the neighbours of changed vertices alone
-                            counts no entries (lp_nnz neither) */
+                            counts their entries as nnz (so does lp_nnz) */
   int32_t first_group;   /* lanes per vertex of the first-round label-propagation kernel
                             (8, 16 or 32; picked once per handle by timing each choice) */
   int32_t emit_group;    /* lanes per vertex of the contraction's pre-merge kernel (same) */

@@ -76,6 +76,7 @@ struct Counters {
   int nab[2];         // vertices whose list is new for pass A, for pass B
   int changed;
   unsigned long long asym;  // validation: 0 where every entry has its reverse
+  unsigned long long lp_entries;  // entries of a level's label rounds over marked vertices (timing)
 };
 
 // What the host reads at its decision points, in one copy.
@@ -492,7 +493,8 @@ struct Workspace {
       cudaEvent_t a = mark();
       if (few) {
         prepare_dbins(g.n);
-        bins_build(g, dbins, s, nullptr, nullptr, KeepLabels{mark_, in, out});
+        bins_build(g, dbins, s, nullptr, nullptr,
+                   KeepLabels{mark_, in, out, timing ? &ctr()->lp_entries : nullptr});
         dbins.h_small = bins.h_small;  // no class grows: enough for the launches
         dbins.h_reg = bins.h_reg;
         dbins.h_mid = bins.h_mid;
@@ -503,7 +505,7 @@ struct Workspace {
       if (timing) {
         lp_spans.push_back({a, mark()});
         long long gather = in ? 4 : 0;
-        const int64_t entries = few ? 0 : g.nnz;  // how many of them a restricted round reads stays on the device
+        const int64_t entries = few ? 0 : g.nnz;  // those of restricted rounds are counted on the device
         lp_bytes_acc += 8 * (g.n + 1) + entries * (4 + (g.unit ? 0 : g.wbytes) + gather) + 4 * g.n;
         lp_nnz_acc += entries;
         lp_n_acc += g.n;
@@ -524,9 +526,16 @@ struct Workspace {
           few = true;
           mark_ = smflag.ensure_n<unsigned char>(g.n);
           VC_CUDA(cudaMemsetAsync(mark_, 0, (size_t)g.n, s));
+          if (timing) VC_CUDA(cudaMemsetAsync(&ctr()->lp_entries, 0, sizeof(unsigned long long), s));
           count_changed(g, prev, out, cnt, mark_, s);  // this round's marks; the count is read
         }
       }
+    }
+    if (few && timing) {
+      read_state();
+      const int64_t entries = (int64_t)h_counters->lp_entries;
+      lp_bytes_acc += entries * (4 + (g.unit ? 0 : g.wbytes) + 4);
+      lp_nnz_acc += entries;
     }
     *out_labels = in;
   }

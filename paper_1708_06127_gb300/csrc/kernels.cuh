@@ -69,11 +69,12 @@ struct Bins {
 };
 
 // Binning only the marked vertices: the others keep their label (out[v] = in[v]); the marks
-// are cleared.
+// are cleared.  *entries (may be null) += the length of the marked vertices' lists.
 struct KeepLabels {
   unsigned char* mark = nullptr;
   const int32_t* in = nullptr;
   int32_t* out = nullptr;
+  unsigned long long* entries = nullptr;
 };
 // list_n not null: bins the vertices list[0, *list_n) (at most g.n of them) instead of all.
 void bins_build(const GraphView& g, Bins& b, cudaStream_t s, const int32_t* list = nullptr,

@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(256) bins_k(int64_t n, int64_t chunk, const in
   __syncthreads();
   int c[kBinClasses] = {0, 0, 0, 0, 0};
   int dmax = 0;
+  unsigned long long len = 0;
   for (int64_t i = lo + tid; i < hi; i += 256) {
     const int64_t v = vert(i);
     const int64_t d = off[v + 1] - off[v];
@@ -71,6 +72,11 @@ __global__ void __launch_bounds__(256) bins_k(int64_t n, int64_t chunk, const in
 #pragma unroll
     for (int q = 0; q < kBinClasses; ++q) c[q] += k == q;
     if (k >= 2) dmax = max(dmax, (int)(d < INT_MAX ? d : INT_MAX));
+    if (k >= 0) len += (unsigned long long)d;
+  }
+  if (keep.entries) {
+    len = warp_sum(len);
+    if (lane == 0 && len) atomicAdd(keep.entries, len);
   }
 #pragma unroll
   for (int q = 0; q < kBinClasses; ++q) {

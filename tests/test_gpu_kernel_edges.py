@@ -356,3 +356,33 @@ def test_converging_rounds_not_symmetric():
         cut, bits = mc.run(3, 25)
         assert mc.trace() == ref.trace
     assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+def test_converging_rounds_count_their_entries(weighted):
+    """The statistics of a level whose later rounds visit the neighbours of changed vertices
+    only: the entries those rounds read are counted, the others' are not."""
+    g = gg.core_lcc(gg.rhg(1 << 16, 32, 5), 0)
+    if weighted:
+        g = gg.with_pair_weights(g, 4, 1, 9)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    deg, src = np.diff(G.offsets), np.repeat(np.arange(G.n), np.diff(G.offsets))
+    label, moved, few = np.arange(G.n, dtype=np.int32), None, False
+    nnz, size, restricted = 0, 0, 0
+    for r in range(25):
+        entries = int(deg[np.unique(G.adj[moved[src]])].sum()) if few else G.nnz
+        nnz += entries
+        size += 8 * (G.n + 1) + entries * (4 + (4 if weighted else 0) + (4 if r else 0)) + 4 * G.n
+        restricted += few
+        after = oracle.lp_round(G, label, oracle.level_key(3, 0))
+        moved, label = after != label, after
+        if int(moved.sum()) * 10000 <= G.n:
+            break
+        few = few or int(moved.sum()) * 32 <= G.n
+    assert restricted > 0
+    with vc.MinCut(g.offsets, g.adj, g.w, n0=G.n - 1, lp_converge=True, timing=True) as mc:
+        for _ in range(2):
+            mc.run(3, 25)
+            st = mc.stats()
+            assert st["levels"] == 1 and st["lp_launches"] == r + 1
+            assert st["lp_nnz"] == nnz and st["lp_bytes"] == size
