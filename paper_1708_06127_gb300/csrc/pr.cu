@@ -111,12 +111,12 @@ __global__ void __launch_bounds__(256) partners_long_k(int64_t n, const int64_t*
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const int64_t e = e0 + 256 * q;
-          x[q] = e < end ? (long long)w[e] : -1;
-          u[q] = e < end ? adj[e] : INT_MAX;
+          x[q] = e < end ? (long long)w[e] : 0;
+          u[q] = e < end ? adj[e] : -1;
         }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
-          if (x[q] >= 0) partner_fold(s, bw, bu, x[q], u[q]);
+          if (u[q] >= 0) partner_fold(s, bw, bu, x[q], u[q]);
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {

@@ -386,3 +386,23 @@ def test_converging_rounds_count_their_entries(weighted):
             st = mc.stats()
             assert st["levels"] == 1 and st["lp_launches"] == r + 1
             assert st["lp_nnz"] == nnz and st["lp_bytes"] == size
+
+
+@pytest.mark.parametrize("entries", [8192, 8193, 9000])
+def test_partners_of_a_long_list_with_negative_weights(entries):
+    """Weights below 0 (an upload takes any) count in a long list's degree as in a short one's."""
+    ring = [(v, (v + 1) % entries, 90 if v in (6, 7) else 1) for v in range(entries)]
+    star = [(v, entries, 100 if v == 7 else 1) for v in range(entries)]
+    g = gg.from_edges(entries + 1, ring + star)
+    src = np.repeat(np.arange(g.n), np.diff(g.offsets))
+    hub = (src == entries) | (g.adj == entries)
+    w = np.where(hub & ((src + g.adj) % 2 == 1) & (g.w == 1), -1, g.w)
+    G = oracle.as_csr64(g.offsets, g.adj, w)
+    d = vc.viecut_graph_upload(G.offsets, G.adj, G.w)
+    try:
+        ref, cnt = oracle.pr_pass_a(G, 1000)
+        got, ch = vc.viecut_step_pr_a(d, 1000)
+        assert ref[entries] == ref[7]  # by the hub's degree of about 100 alone: vertex 7's is 280
+        assert np.array_equal(got, ref) and ch == (1 if cnt > 0 else 0)
+    finally:
+        vc.viecut_graph_free(d)
