@@ -970,7 +970,8 @@ static int step_labels(viecut_graph* g, int64_t lambda_hat, int32_t* labels, int
       vc::pr_pass_a(v, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), W.st(),
                     W.parent.as<int32_t>(), lab, chg, c.s);
     else
-      vc::pr_pass_b(v, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), W.st(), lab, chg, c.s);
+      vc::pr_pass_b(v, W.partner.as<int32_t>(), W.pw.as<long long>(), W.deg.as<long long>(), W.st(), lab, chg, c.s,
+                    nullptr, nullptr, W.pr_long(v.nnz));
   } else {
     // every entry reaches a bound below 1, one of weight 0 too: as unit weights reach 1
     if (lambda_hat < 1) {

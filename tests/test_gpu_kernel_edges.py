@@ -406,3 +406,137 @@ def test_partners_of_a_long_list_with_negative_weights(entries):
         assert np.array_equal(got, ref) and ch == (1 if cnt > 0 else 0)
     finally:
         vc.viecut_graph_free(d)
+
+
+def check_pass_b(G, lam):
+    d = vc.viecut_graph_upload(G.offsets, G.adj, G.w)
+    try:
+        got, ch = vc.viecut_step_pr_b(d, lam)
+    finally:
+        vc.viecut_graph_free(d)
+    ref, cnt = oracle.pr_pass_b(G, lam)
+    assert np.array_equal(got, ref) and ch == (1 if cnt > 0 else 0)
+    return ref
+
+
+@pytest.mark.parametrize("longer", [0, 1500])
+def test_pass_b_long_pairs(longer):
+    """Mutual partners whose shorter list is at the edge of what the grid's blocks share, one
+    unit to either side of conditions 3 and 4 (each alone decisive; the longer list of some
+    pairs first, of others second)."""
+    lam, n0, rng = 10000, 20000, np.random.default_rng(5)
+    blob = gg.er(n0, 56, 9)
+    src = np.repeat(np.arange(n0), np.diff(blob.offsets))
+    edges = [(int(a), int(b), 1) for a, b in zip(src, blob.adj) if a < b]
+    pairs, at = [], n0
+
+    def private(v, k, w, kw, avoid):  # neighbours of v alone and of w alone
+        own = rng.choice(np.setdiff1d(np.arange(n0), avoid), k + kw, replace=False)
+        edges.extend((int(u), v if i < k else w, 1) for i, u in enumerate(own))
+
+    for size in (2047, 2048, 2049, 2050, 4097):  # entries of the shorter list
+        for case in ("3", "not 3", "4", "not 4"):
+            v, w = (at, at + 1) if len(pairs) % 2 else (at + 1, at)
+            at += 2
+            if case.endswith("3"):  # one common neighbour: degree = 2 (c + y) or one more
+                p = size - 2
+                c = p // 2 + 1
+                y = p - c - (case != "3")
+                u = int(rng.integers(n0))
+                edges += [(u, v, y), (u, w, y), (v, w, c)]
+                private(v, p, w, p, [u])
+            else:  # 900 common neighbours of weight 10, c + 9000 = lam or one less
+                u = rng.choice(n0, 900, replace=False)
+                edges += [(int(x), v, 10) for x in u] + [(int(x), w, 10) for x in u]
+                edges.append((v, w, lam - 9000 - (case != "4")))
+                private(v, size - 901, w, size - 901 + longer, u)
+            pairs.append((v, w, case))
+    g = gg.from_edges(at, [(min(a, b), max(a, b), x) for a, b, x in edges])
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    assert G.nnz >= 1 << 20 and (np.diff(G.offsets)[n0:] > 2048).sum() >= 24
+    ref = check_pass_b(G, lam)
+    for v, w, case in pairs:
+        assert (ref[v] == ref[w]) == (case in ("3", "4")), (v, w, case)
+
+
+def test_run_of_passes_over_changed_lists():
+    """Passes that test only the lists the last contractions changed, and find merges that those
+    made: a and b are joined by an edge of the bound, then c and then d by two edges of half the
+    bound each, one to either part of what was joined before, and pass B joins p and q once
+    their common neighbour is one vertex."""
+    n, lam, rng = 36000, 10, np.random.default_rng(4)
+    blob = gg.er(n, 34, 2)
+    src = np.repeat(np.arange(n), np.diff(blob.offsets))
+    weight = {(int(a), int(b)): 1 for a, b in zip(src, blob.adj) if a < b}
+    pick = rng.permutation(np.flatnonzero(np.diff(blob.offsets) >= 26))[:20 * 6].reshape(20, 6)
+    for a, b, c, d, p, q in pick.tolist():
+        for x, y, wt in ((a, b, lam), (a, c, 5), (b, c, 5), (a, d, 5), (c, d, 5), (p, q, 6), (c, p, 4), (a, q, 4)):
+            weight[min(x, y), max(x, y)] = wt
+    for u in rng.choice(n, lam, replace=False):
+        weight[int(u), n] = 1  # the vertex of smallest degree
+    g = gg.from_edges(n + 1, [(a, b, wt) for (a, b), wt in sorted(weight.items())])
+    ref = oracle.viecut(g.offsets, g.adj, g.w, seed=2, lp_iters=0, n0=1000)
+    # a pass is restricted where the last one of its kind had the same bound and at most a quarter
+    # of the lists changed since: at most those of the vertices merged so far and their neighbours
+    widest = int(np.diff(g.offsets).max())
+    size, seen, restricted = n + 1, set(), {2: 0, 3: 0}
+    for kind, level, left, _, bound in ref.trace[2:7]:
+        assert kind in (2, 3) and level == 0 and bound == lam and left >= 1 << 15
+        restricted[kind] += kind in seen and 4 * 2 * (n + 1 - size) * (widest + 1) <= size
+        seen.add(kind)
+        size = left
+    assert restricted[2] >= 1 and restricted[3] >= 1
+    with vc.MinCut(g.offsets, g.adj, g.w, n0=1000) as mc:
+        for _ in range(2):
+            cut, bits = mc.run(2, 0)
+            assert mc.trace() == ref.trace
+            assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
+
+
+def test_contract_large_near_identity_unit():
+    """As test_contract_large_near_identity on unit weights, then with several hubs among the
+    merged vertices (their lists are shared by the grid's blocks)."""
+    g = gg.er(700_000, 50, 8)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    assert G.nnz >= 1 << 25
+    rng = np.random.default_rng(9)
+    labels = np.arange(G.n)
+    pick = rng.choice(G.n, 2000, replace=False)
+    labels[pick[:1000]] = labels[pick[1000:]]
+    check_contract(G, labels)
+    labels = np.arange(G.n)
+    members = rng.choice(G.n, 1200, replace=False).reshape(6, 200)
+    labels[members] = members[:, :1]
+    hubs = check_contract(G, labels)
+    wide = np.flatnonzero(np.diff(hubs.offsets) > 4096)
+    assert len(wide) == 6
+    labels = np.arange(hubs.n)
+    labels[wide[:3]] = rng.choice(hubs.n, 3, replace=False)
+    labels[wide[3]] = wide[4]
+    check_contract(hubs, labels)
+
+
+def test_exact_rounds_on_a_large_input():
+    """Exact rounds on an input of more than 2^25 entries with 32-bit weights that join one pair
+    of a regular circulant graph, so that nearly every list is renumbered by the run; the second
+    round reads what the first one's contraction wrote.  A triangle apart from it collapses in
+    two rounds and ends the run."""
+    n, half = 40_000, 420
+    step = np.concatenate([np.arange(1, half + 1), np.arange(n - half, n)])
+    wt = (1 + np.minimum(step, n - step) % 7).astype(np.int32)
+    adj = ((np.arange(n)[:, None] + step) % n).astype(np.int32)
+    order = np.argsort(adj, axis=1)
+    adj, w = np.take_along_axis(adj, order, 1).ravel(), wt[order].ravel()
+    degree = int(wt.sum())
+    side = degree // 2 + 1
+    adj = np.concatenate([adj, np.array([n + 1, n + 2, n, n + 2, n, n + 1], np.int32)])
+    w = np.concatenate([w, np.full(6, side, np.int32)])
+    off = np.concatenate([np.arange(n + 1) * 2 * half, n * 2 * half + np.array([2, 4, 6])]).astype(np.int64)
+    assert len(adj) >= 1 << 25
+    ref = oracle.viecut(off, adj, w, seed=1, lp_iters=2, n0=n + 3)
+    assert [t[0] for t in ref.trace] == [0, 4, 4] and ref.trace[2][3] >= 1 << 25
+    assert [t[2] for t in ref.trace] == [n + 3, n + 1, n - 1] and ref.cut == 0
+    with vc.MinCut(off, adj, w, n0=n + 3) as mc:
+        cut, bits = mc.run(1, 2)
+        assert mc.trace() == ref.trace
+    assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
