@@ -332,7 +332,10 @@ struct Workspace {
   // sparse contraction of a graph whose own arrays are valid (had), only changed lists are
   // read; pr_new (after the next read_state, pr_new_read) says how many lists are new for a
   // pass.  Graphs below kFlagMinN keep no flags: their passes cost launches, not lists.
-  static constexpr int64_t kFlagMinN = int64_t(1) << 15;
+  // Planted graphs by vertices, with flags and without: 4 x 30,000 9.24 and 8.89 ms,
+  // 8 x 16,384 10.38 and 10.06 ms, 8 x 60,013 25.5 and 25.5 ms, 8 x 131,072 59.9 and 63.2 ms,
+  // 8 x 524,288 116.2 and 123.7 ms; a line at 2^19 loses 59.9 -> 62.7 ms on 8 x 131,072.
+  static constexpr int64_t kFlagMinN = int64_t(1) << 17;
   bool flags_ok = false;  // prflag describes the current graph
   bool carried = false;
   int64_t pr_new[2] = {0, 0};

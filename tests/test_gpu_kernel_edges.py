@@ -463,9 +463,10 @@ def test_run_of_passes_over_changed_lists():
     """Passes that test only the lists the last contractions changed, and find merges that those
     made: a and b are joined by an edge of the bound, then c and then d by two edges of half the
     bound each, one to either part of what was joined before, and pass B joins p and q once
-    their common neighbour is one vertex."""
-    n, lam, rng = 36000, 10, np.random.default_rng(4)
-    blob = gg.er(n, 34, 2)
+    their common neighbour is one vertex.  A chain apart from the rest collapses a vertex a pass
+    and ends the run with its last one."""
+    n, lam, rng = 140_000, 10, np.random.default_rng(4)
+    blob = gg.er(n, 36, 2)
     src = np.repeat(np.arange(n), np.diff(blob.offsets))
     weight = {(int(a), int(b)): 1 for a, b in zip(src, blob.adj) if a < b}
     pick = rng.permutation(np.flatnonzero(np.diff(blob.offsets) >= 26))[:20 * 6].reshape(20, 6)
@@ -474,18 +475,25 @@ def test_run_of_passes_over_changed_lists():
             weight[min(x, y), max(x, y)] = wt
     for u in rng.choice(n, lam, replace=False):
         weight[int(u), n] = 1  # the vertex of smallest degree
-    g = gg.from_edges(n + 1, [(a, b, wt) for (a, b), wt in sorted(weight.items())])
+    chain, e0 = 9, n + 1
+    weight[e0, e0 + 1] = lam
+    for k in range(2, chain):
+        weight[e0 + k - 1, e0 + k] = 5
+        for x in (e0, e0 + 1):
+            weight[x, e0 + k] = weight.get((x, e0 + k), 0) + 3
+    g = gg.from_edges(n + 1 + chain, [(a, b, wt) for (a, b), wt in sorted(weight.items())])
     ref = oracle.viecut(g.offsets, g.adj, g.w, seed=2, lp_iters=0, n0=1000)
     # a pass is restricted where the last one of its kind had the same bound and at most a quarter
     # of the lists changed since: at most those of the vertices merged so far and their neighbours
     widest = int(np.diff(g.offsets).max())
-    size, seen, restricted = n + 1, set(), {2: 0, 3: 0}
-    for kind, level, left, _, bound in ref.trace[2:7]:
-        assert kind in (2, 3) and level == 0 and bound == lam and left >= 1 << 15
-        restricted[kind] += kind in seen and 4 * 2 * (n + 1 - size) * (widest + 1) <= size
+    size, seen, restricted = g.n, set(), {2: 0, 3: 0}
+    assert [t[4] for t in ref.trace[2:]] == [lam] * (len(ref.trace) - 3) + [0]
+    for kind, level, left, *_ in ref.trace[2:]:
+        assert kind in (2, 3) and level == 0 and left >= 1 << 17
+        restricted[kind] += kind in seen and 4 * 2 * (g.n - size) * (widest + 1) <= size
         seen.add(kind)
         size = left
-    assert restricted[2] >= 1 and restricted[3] >= 1
+    assert restricted[2] >= 2 and restricted[3] >= 1 and ref.cut == 0
     with vc.MinCut(g.offsets, g.adj, g.w, n0=1000) as mc:
         for _ in range(2):
             cut, bits = mc.run(2, 0)
@@ -540,3 +548,16 @@ def test_exact_rounds_on_a_large_input():
         cut, bits = mc.run(1, 2)
         assert mc.trace() == ref.trace
     assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
+
+
+def test_run_of_changed_lists_many_passes():
+    """Degrees, partners and flags carried over many passes on a graph whose hubs grow from merges
+    (planted blocks, 2^19 vertices)."""
+    g = gg.planted(8, 1 << 16, 24, 8, 3)
+    ref = oracle.viecut(g.offsets, g.adj, g.w, seed=2, lp_iters=2, n0=1000)
+    assert sum(t[0] in (2, 3) and t[2] >= 1 << 17 for t in ref.trace) >= 8
+    with vc.MinCut(g.offsets, g.adj, g.w, n0=1000) as mc:
+        for _ in range(2):
+            cut, bits = mc.run(2, 2)
+            assert mc.trace() == ref.trace
+            assert cut == ref.cut and np.array_equal(bits, ref.side_bits)
