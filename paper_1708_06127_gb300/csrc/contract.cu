@@ -2,12 +2,14 @@
 // every block of a labelling becomes one vertex, intra-block edges vanish and
 // parallel edges between two blocks merge with summed weight.  Block ids are the
 // ranks of the label values.  Steps: relabel (flag + scan), the optional correcting
-// step, pre-merge per fine vertex (lp.cu), then either
+// step, pre-merge per fine vertex (lp.cu), then one of
+//   * the table (few clusters and many pairs): the pairs are added up in c x c sums, which are
+//     read row by row into the coarse lists,
 //   * the cluster merge: a counting sort of the pre-merged pairs by source cluster,
 //     then a warp per cluster of at most kMergeMax pairs (registers, or a bitonic sort
 //     in shared memory), a block per cluster of at most kMergeBlockMax, and one radix
 //     sort for all larger ("giant") clusters together; each writes its distinct
-//     targets in ascending order at the front of its segment, or
+//     targets in ascending order at the front of its segment,
 //   * pair build, LSD radix sort on (cid v, cid u) and a run reduction (when the giant
 //     clusters hold more than half of the pairs).
 #include <limits.h>
@@ -101,11 +103,14 @@ void build_pairs(const GraphView& g, const int32_t* cid, const ContractScratch& 
                  const LongLists& longs, unsigned long long* keys, long long* vals, cudaStream_t s) {
   const PairOut in{cs.tmp_key, cs.tmp_val, cs.cmp_key, cs.cmp_val};
   if (pairs <= 2 * g.n)
-    build_pairs_k<1><<<grid_for(g.n, 256, kSMs * 8), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals, longs);
+    build_pairs_k<1><<<grid_for(g.n, 256, kSMs * 8), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys,
+                                                                  vals, longs);
   else if (pairs <= 16 * g.n)
-    build_pairs_k<8><<<grid_for(g.n, 32, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals, longs);
+    build_pairs_k<8><<<grid_for(g.n, 32, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys,
+                                                                  vals, longs);
   else
-    build_pairs_k<32><<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys, vals, longs);
+    build_pairs_k<32><<<grid_for(g.n, 8, kSMs * 16), 256, 0, s>>>(g.n, g.off, cid, cs.cnt, cs.pos, in, bits, keys,
+                                                                  vals, longs);
   count_launch();
   if (longs.item) {
     build_pairs_long_k<<<kSMs * 4, 256, 0, s>>>(g.off, cid, cs.cnt, in, bits, keys, vals, longs);
@@ -199,7 +204,6 @@ void reduce_pairs(const unsigned long long* keys, const long long* vals, int64_t
 // pair of weight 0 or below went into it (inputs that nothing checked): those are noted in a
 // bit per sum (zero, 32 columns a word).
 __host__ __device__ inline int64_t table_words(int64_t c) { return (c + 31) >> 5; }
-
 
 // W lanes per fine vertex add its pre-merged list to its cluster's row.
 template <int W>
@@ -699,7 +703,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32) cluster_merge_k(int64_t c, c
 // Clusters of kMergeMax < T <= kMergeBlockMax pairs: a block per cluster sorts the pairs by
 // target (sort_elements, 4 to 16 elements per thread), then every run head sums its run; the
 // distinct targets are written back in ascending order at the front of the segment.
-// With a list (list_count not null) only the listed clusters are visited.
+// The clusters are the listed ones, list[0, *list_count).
 constexpr int kMergeBlockSmem = (kMergeBlockMax + kMergeBlockMax / 16 + kMergeBlockMax) * 8;  // elements, sums
 
 template <int E>
@@ -759,22 +763,21 @@ __device__ __forceinline__ int merge_block(long long b, int T, int32_t* __restri
   return total;
 }
 
-__global__ void __launch_bounds__(256) cluster_merge_block_k(int64_t c, const long long* __restrict__ cbase,
+__global__ void __launch_bounds__(256) cluster_merge_block_k(const long long* __restrict__ cbase,
                                                              int32_t* __restrict__ seg_key,
                                                              long long* __restrict__ seg_val,
                                                              int32_t* __restrict__ dcount,
-                                                             const int32_t* __restrict__ list = nullptr,
-                                                             const int* __restrict__ list_count = nullptr) {
+                                                             const int32_t* __restrict__ list,
+                                                             const int* __restrict__ list_count) {
   extern __shared__ __align__(16) unsigned char mb_dyn[];
   unsigned long long* se = (unsigned long long*)mb_dyn;
   long long* sv = (long long*)(se + kMergeBlockMax + kMergeBlockMax / 16);
   __shared__ int s_warp[8];
-  const int64_t total = list_count ? (int64_t)*list_count : c;
-  for (int64_t xi = blockIdx.x; xi < total; xi += gridDim.x) {
-    const int64_t x = list_count ? (int64_t)list[xi] : xi;
+  const int total = *list_count;
+  for (int xi = blockIdx.x; xi < total; xi += gridDim.x) {
+    const int32_t x = list[xi];
     const long long b = cbase[x];
-    const int T = (int)(cbase[x + 1] - b);
-    if (T <= kMergeMax || T > kMergeBlockMax) continue;  // the same in every thread of the block
+    const int T = (int)(cbase[x + 1] - b);  // kMergeMax < T <= kMergeBlockMax
     int d;
     if (T <= 1024) d = merge_block<4>(b, T, seg_key, seg_val, se, sv, s_warp);
     else if (T <= 2048) d = merge_block<8>(b, T, seg_key, seg_val, se, sv, s_warp);
@@ -818,7 +821,6 @@ __global__ void __launch_bounds__(256) cluster_place_k(int64_t c, const long lon
   }
 }
 
-
 // The lists cluster_place_k left out.
 __global__ void cluster_place_long_k(const long long* __restrict__ cbase, const int64_t* __restrict__ coff,
                                      const int32_t* __restrict__ seg_key, const long long* __restrict__ seg_val,
@@ -847,8 +849,9 @@ __global__ void cluster_place_long_k(const long long* __restrict__ cbase, const 
 // a lone vertex is its fine list renumbered, except for the few entries that point into
 // the other ("merged") clusters: those may repeat a target and sit out of order.
 // A warp per lone vertex sums them per target in shared memory and merges the distinct
-// ones into the renumbered list -- one pass to count the coarse degree, one to write.  Only the members of merged groups (and lone vertices with more than
-// kScMaxM such entries) go through the pre-merge and the cluster merge.
+// ones into the renumbered list -- one pass to count the coarse degree, one to write.  Only
+// the members of merged groups (and lone vertices with more than kScMaxM such entries) go
+// through the pre-merge and the cluster merge.
 constexpr int kScMaxM = 32;  // entries into merged groups per lone vertex
 
 // mflag[cid[v]] = 1 for every v not labelled by its own id (its cluster has another
@@ -913,13 +916,14 @@ __device__ __forceinline__ int sc_collect(int64_t beg, int64_t end, int lane, co
 
 // A contraction that merges few vertices touches few lists: the neighbours of the merged
 // groups' members (every edge is in both lists: GraphView::symmetric), found from the
-// members' own.  They are
-// marked so (touched) while at most a sixteenth of the vertices disappears, and pass 1 then
-// reads only those lists; otherwise it reads every list.  Planted 8 x 2^20, 392 million
-// entries: 1.25 ms a pass over every list, whatever the pass merged (one random gather per
-// entry, at 0.8 of one per SM and cycle); 31.0 -> 17.2 ms for its 25 contractions.  Below
-// kScPushMin entries a pass costs less than the marking: 8 x 60,000 (18.7 million entries)
-// took 1.6 ms with it, 1.4 ms without.
+// members' own.  They are marked so (touched) while at most a sixteenth of the vertices
+// disappears, and pass 1 then reads only those lists; otherwise it reads every list.  Planted
+// 8 x 2^20, 392 million entries: 1.25 ms a pass over every list, whatever the pass merged (one
+// random gather per entry, at 0.8 of one per SM and cycle); 31.0 -> 17.2 ms for its 25
+// contractions.  Below kScPushMin entries a pass costs less than the marking: whole planted
+// runs by entries, with the marks and sc_copy_k and without both, 6.3 million 14.6 and 13.8 ms,
+// 25 million 28.4 and 27.7, 50 million 60.6 and 60.7, 101 million 90.5 and 93.0, 201 million
+// 173 and 177.  An eighth or a thirty-second of the vertices instead: the same within 1 %.
 constexpr int64_t kScPushMin = int64_t(1) << 25;
 __device__ __forceinline__ bool sc_few(int64_t n, const int* nclust) { return 16 * (n - __ldg(nclust)) <= n; }
 
@@ -955,7 +959,8 @@ __global__ void __launch_bounds__(256) sc_push_long_k(const int64_t* __restrict_
   for (int i = G.first; i < n; i += G.step) {
     const int64_t beg = off[longs[i]], end = off[longs[i] + 1];
 #pragma unroll 4
-    for (int64_t e = beg + G.part * 256 + threadIdx.x; e < end; e += (int64_t)G.parts * 256) touched[__ldg(adj + e)] = 1;
+    for (int64_t e = beg + G.part * 256 + threadIdx.x; e < end; e += (int64_t)G.parts * 256)
+      touched[__ldg(adj + e)] = 1;
   }
 }
 
@@ -1017,7 +1022,9 @@ __global__ void __launch_bounds__(256) sc_count_k(int64_t n, const int* __restri
 // memory, and only entries into the other runs gather their new id.  What is left is a
 // stream: 12 bytes read and 16 written per entry (392 million entries, 1800 of 4.4 million
 // vertices gone: 3.5 ms -> 2.4 ms here and 0.4 ms in sc_write_k; 15,800 gone, over one in
-// 512: too few whole runs).  From kScPushMin entries on: at 18.7 million it gained nothing.
+// 512: too few whole runs).  From kScPushMin entries on (alone, whole planted runs: 25 million
+// 28.3 against 27.7 ms, 101 million 92.6 against 93.0).  One vertex in 128 or in 2048 instead:
+// within 1 % at 101 and 134 million entries.
 constexpr int kScTab = 16384;  // runs at most
 constexpr int kScCopyThreads = 512;
 static int sc_shift(int64_t n) { return std::max(8, ceil_log2(n) - 14); }
@@ -1628,7 +1635,7 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
     // like the other lists' here, starts from zero)
     block_class_list_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, blist, blist_n);
     set_smem(cluster_merge_block_k, kMergeBlockSmem);
-    cluster_merge_block_k<<<kSMs * 3, 256, kMergeBlockSmem, s>>>(c, cbase, seg_key, seg_val, ccount, blist, blist_n);
+    cluster_merge_block_k<<<kSMs * 3, 256, kMergeBlockSmem, s>>>(cbase, seg_key, seg_val, ccount, blist, blist_n);
     count_launch(2);
     VC_CHECK_LAUNCH();
   }
@@ -1636,7 +1643,7 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
   if (sp) sparse_finish_degrees(g, cid, sp->sdeg, ccount, sp->clean, c, s);
   exclusive_scan<int, long long>(ccount, (long long*)coff, c, (long long*)coff + c, cs.scan_scr, s, nullptr, nnz_dev);
   LongLists place = longs;
-  place.n = longs.n + 1;  // a count of its own, the items no longer needed
+  if (longs.n) place.n = longs.n + 1;  // a count of its own, the items no longer needed
   cluster_place_k<<<grid_for(c, 256, kSMs * 8), 256, 0, s>>>(c, cbase, coff, seg_key, seg_val, cadj, cw, csrc,
                                                                sp ? sp->clean : nullptr, place);
   if (longs.item) {
@@ -1647,6 +1654,5 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
   VC_CHECK_LAUNCH();
   if (sp) sparse_copy(g, c, *sp, coff, cadj, cw, csrc, s);
 }
-
 
 }  // namespace vc

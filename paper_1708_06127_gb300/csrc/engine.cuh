@@ -94,7 +94,8 @@ struct Workspace {
   cudaStream_t s = nullptr;
   // vertex-sized
   Buf deg, labA, labB, map0, cidT, cur1, side1, flags, rank, cnt, pos, scan64, scan32, hv;
-  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, longV, longAt, longHit, mergeS, mergeL, slist, rlist, mlist, blist, glist, bl1, noi_r;
+  Buf partner, pw, parent, partner2, pw2, deg2, prflag, prflag2, prlist, longV, longAt, longHit, mergeS, mergeL;
+  Buf slist, rlist, mlist, blist, glist, bl1, noi_r;
   // entry-sized
   Buf tmpK, tmpV, cmpK, cmpV;
   // pair-sized
@@ -277,7 +278,7 @@ struct Workspace {
     tune.emit_group = pick_group([&](int G) {
       LpTuning t = tune;
       t.emit_group = G;
-      emit_cross(g, bins, gt, cid, po, c, s, t);
+      emit_cross(g, bins, cid, po, c, s, t);
     });
   }
 
@@ -605,7 +606,7 @@ struct Workspace {
     if (sparse) VC_CUDA(cudaMemsetAsync(cs.cnt, 0, sizeof(int32_t) * g.n, s));  // clean vertices: no pairs
     po.ccount = ccount;
     cudaEvent_t e0 = mark();
-    emit_cross(g, B, gt, cid_out, po, cs.cnt, s, tune);
+    emit_cross(g, B, cid_out, po, cs.cnt, s, tune);
     if (timing && !sparse) pm_spans.push_back({e0, mark()});  // the whole graph's pre-merge only
     VC_CUDA(cudaMemsetAsync(&ctr()->maxt, 0, offsetof(Counters, nflag) - offsetof(Counters, maxt), s));
     cluster_stats(g.n, ccount, &ctr()->maxt, &ctr()->pairs, &ctr()->ngiant, &ctr()->gpairs, s);
@@ -617,7 +618,7 @@ struct Workspace {
     if (timing) {
       // pre-merge: offsets, ids, weights (none when all are 1), the cluster id of every
       // neighbour and of v, the pair count of v and the pairs (int32 key + int64 sum)
-      if (!sparse) pm_bytes_acc += 8 * (g.n + 1) + g.nnz * (4 + (g.unit ? 0 : g.wbytes) + 4) + 4 * g.n + 4 * g.n + 12 * P;
+      if (!sparse) pm_bytes_acc += 8 * (g.n + 1) + g.nnz * (4 + (g.unit ? 0 : g.wbytes) + 4) + 8 * g.n + 12 * P;
       ct_count += 1;
     }
     // coarse entries: at most the pairs, plus (sparse) the clean vertices' copied lists;

@@ -175,8 +175,8 @@ struct PairOut {
 
 // Pre-merge for contraction: for each vertex v, the distinct coarse neighbours cu =
 // cid[u] != cid[v] with summed weights, cnt[v] pairs placed as PairOut says.
-void emit_cross(const GraphView& g, const Bins& b, const GlobalTables& gt, const int32_t* cid, const PairOut& out,
-                int32_t* cnt, cudaStream_t s, const LpTuning& tune = LpTuning());
+void emit_cross(const GraphView& g, const Bins& b, const int32_t* cid, const PairOut& out, int32_t* cnt,
+                cudaStream_t s, const LpTuning& tune = LpTuning());
 
 // ------------------------------------------------------------------ contraction
 struct ContractScratch {
@@ -292,12 +292,13 @@ void cluster_merge(const GraphView& g, const int32_t* cid, const ContractScratch
                    const GiantScratch* giant, int32_t* blist, int* blist_n, const MergeLists& lists, cudaStream_t s,
                    const SparseCtx* sparse = nullptr, const LongLists& longs = LongLists());
 
-// Builds (cid[v] << bits | cu, weight) pairs from the pre-merged lists.
 // Whether the pairs are merged in a table of c x c sums, which this picks where the table is
 // at most as large as the arrays that the other merges sort the pairs in (16 bytes a pair)
 // and no sum takes more than 64 additions on average (few clusters: additions to one address
-// run one after another), or all pairs are so few that the other merges' launches cost more.
-// 16,001 vertices, 18 million pairs to 2326 clusters: sorting 1.35 ms, the table 0.18 ms;
+// run one after another), or there are at most 2^16 pairs, where the other merges' launches
+// cost more than any run of additions: pairs to two clusters, the table and the others, 7,853:
+// 17 and 270 us, 31,420: 28 and 46, 62,842: 40 and 50; beyond, 117,808: 60 and 57, 196,469: 92
+// and 56.  16,001 vertices, 18 million pairs to 2326 clusters: sorting 1.35 ms, the table 0.18 ms;
 // 2326 vertices, 3 million pairs to 2270: the cluster merge 0.9 ms, the table 0.05 ms; 1367
 // vertices, 2732 pairs to 2: the cluster merge 0.12 ms, the table 0.02 ms.
 bool table_merge_fits(int64_t c, int64_t pairs);
@@ -307,6 +308,7 @@ void table_merge(const GraphView& g, const int32_t* cid, const ContractScratch& 
                  long long* sums, int32_t* ccount, int64_t* coff, int32_t* cadj, long long* cw, int32_t* csrc,
                  long long* nnz_dev, cudaStream_t s);
 
+// Builds (cid[v] << bits | cu, weight) pairs from the pre-merged lists.
 void build_pairs(const GraphView& g, const int32_t* cid, const ContractScratch& cs, int bits, int64_t pairs,
                  const LongLists& longs, unsigned long long* keys, long long* vals, cudaStream_t s);
 

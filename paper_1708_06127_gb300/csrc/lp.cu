@@ -480,13 +480,13 @@ __global__ void __launch_bounds__(kAggThreads) lp_warp_k(
 
 // ------------------------------------------------------------ register class
 // Lists of at most kWarpMaxDeg = 128 entries (and, in other launches, of at most
-// kMidMaxDeg).  A group of G lanes (see RegShape) holds the whole list in registers (slot r of group lane i holds entry G r + i) and visits its
-// distinct keys one at a time, slot by slot: the first lane whose slot r is still
-// unvisited broadcasts its key, every lane marks its entries holding it (only slots
-// >= r can), and a group reduction gives the key's count (unit weights) or weight
-// sum.  No table and no shared memory: one short step per distinct key.  The groups
-// of a warp step in lockstep (the loops run while any group has work; a group
-// without work idles), so every warp-wide vote and shuffle has all lanes present.
+// kMidMaxDeg).  A group of G lanes (see RegShape) holds the whole list in registers (slot r
+// of group lane i holds entry G r + i) and visits its distinct keys one at a time, slot by
+// slot: the first lane whose slot r is still unvisited broadcasts its key, every lane marks
+// its entries holding it (only slots >= r can), and a group reduction gives the key's count
+// (unit weights) or weight sum.  No table and no shared memory: one short step per distinct
+// key.  The groups of a warp step in lockstep (the loops run while any group has work; a
+// group without work idles), so every warp-wide vote and shuffle has all lanes present.
 //
 // A vertex needs three dependent reads (its offsets, its neighbour ids, their keys),
 // so the warp software-pipelines its vertices: while it works on one vertex per
@@ -1485,9 +1485,8 @@ void lp_round(const GraphView& g, const Bins& b, const GlobalTables& gt, const i
   }
 }
 
-void emit_cross(const GraphView& g, const Bins& b, const GlobalTables& gt, const int32_t* cid, const PairOut& out,
-                int32_t* cnt, cudaStream_t s, const LpTuning& tune) {
-  (void)gt;
+void emit_cross(const GraphView& g, const Bins& b, const int32_t* cid, const PairOut& out, int32_t* cnt,
+                cudaStream_t s, const LpTuning& tune) {
   if (g.n <= 0) return;
   const int G = tune.emit_group;
   if (g.unit) launch_emit<UnitW>(g, b, cid, out, cnt, G, s);

@@ -641,7 +641,8 @@ __global__ void __launch_bounds__(kNoiThreads) noi_dense_batch_k(const int32_t* 
     const int32_t base = (int32_t)vbase[g];
     NoiIO io{bn.lam + g, bn.best_kind + g, bn.n_out + g, bn.nnz_out + g, bn.dmin + g, bn.argmin + g,
              bn.trace_len + g, bn.trace + (int64_t)g * bn.trace_cap, bn.trace_cap, bn.level[g]};
-    noi_dense_body<WT>((int)nv[g], off + base, adj, w, base, noi_dyn, scap, M0, M1, ck, sideK + (int64_t)g * kDenseMax, io);
+    noi_dense_body<WT>((int)nv[g], off + base, adj, w, base, noi_dyn, scap, M0, M1, ck,
+                       sideK + (int64_t)g * kDenseMax, io);
     __syncthreads();
   }
 }

@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(256) partners_long_k(int64_t n, const int64_t*
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     const int64_t v0 = base + threadIdx.x;
-    if (v0 < n && (!flag || (flag[v0] & kListNew)) && off[v0 + 1] - off[v0] > kPartnerBlockMin) s_list[atomicAdd(&s_n, 1)] = (int32_t)v0;
+    if (v0 < n && (!flag || (flag[v0] & kListNew)) && off[v0 + 1] - off[v0] > kPartnerBlockMin)
+      s_list[atomicAdd(&s_n, 1)] = (int32_t)v0;
     __syncthreads();
     const int cnt = s_n;
     for (int i = 0; i < cnt; ++i) {
@@ -353,7 +354,8 @@ __global__ void uf_init_min_k(int64_t n, const int64_t* __restrict__ off, const 
 // hundreds of links), and a walk per vertex shortens them once for all entries: RHG n = 2^22,
 // two passes over the coarse graphs, 100 us -> 13 us here and 16 us in pr_a_edge_k.  From
 // kShortenMin vertices on: chains of fewer cost less than the launch (a run with four passes
-// on at most 2326 vertices: 2928 us without it, 2948 us with).
+// on at most 2326 vertices: 2928 us without it, 2948 us with).  Whole runs without it and with
+// it: RHG n = 2^17 (degree 64) 0.67 and 0.67 ms, 2^20 (64) 1.26 and 1.22, 2^21 (32) 1.79 and 1.73.
 constexpr int64_t kShortenMin = 4096;
 __global__ void uf_shorten_k(int32_t* parent, int64_t n) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
