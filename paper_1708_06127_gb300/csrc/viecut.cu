@@ -136,8 +136,7 @@ static void device_validate(Handle& H, bool with_weights = true) {
   Workspace& W = *H.ws;
   int* err = &W.ctr()->changed;
   unsigned long long* asym = relies_on_symmetry(H.m, H.lp_converge) ? &W.ctr()->asym : nullptr;
-  VC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), H.stream));
-  VC_CUDA(cudaMemsetAsync(&W.ctr()->asym, 0, sizeof(unsigned long long), H.stream));
+  VC_CUDA(cudaMemsetAsync(err, 0, offsetof(Counters, lp_entries) - offsetof(Counters, changed), H.stream));  // and asym
   validate_k<<<grid_for(H.n, 256, kSMs * 8), 256, 0, H.stream>>>(H.n, H.m, H.off0, H.adj0,
                                                                 with_weights ? H.w0 : nullptr, err, asym);
   count_launch();
