@@ -100,6 +100,25 @@ def test_exact_round_unchecked_weights(n):
             vc.viecut_graph_free(d)
 
 
+@pytest.mark.parametrize("n", [2, 40, 513, 4000, 16384, 16390])
+def test_exact_round_negative_weights_large_bounds(n):
+    """Few small weights, some below 0, under bounds near 2^63: an entry that counts as the bound
+    carries its vertex across, and the next ones carry the value past the end of its range."""
+    g = ring_graph(n, 9 + n, 1, 9)
+    G = oracle.as_csr64(g.offsets, g.adj, g.w)
+    src = np.repeat(np.arange(n), np.diff(G.offsets))
+    w = np.where((src * 7 + G.adj * 7) % 5 < 3, -G.w, G.w)
+    d = vc.viecut_graph_upload(G.offsets, G.adj, w)
+    try:
+        for lam in (1 << 61, (1 << 62) + 5, (1 << 63) - 1):
+            ref = any_round(oracle.CsrGraph(G.offsets, G.adj, np.where(w < 0, lam, w)), lam)
+            got, ch = vc.viecut_step_noi_round(d, lam)
+            assert np.array_equal(got, ref), lam
+            assert ch == int(any(ref[v] != v for v in range(n)))
+    finally:
+        vc.viecut_graph_free(d)
+
+
 @pytest.mark.parametrize("n", [2, 40, 513, 3000, 16390])
 def test_exact_round_zero_weights(n):
     """Entries of weight 0: they join their ends where the bound is below 1, and only there."""
