@@ -217,7 +217,8 @@ int viecut_step_contract(viecut_graph* g, const int32_t* labels, viecut_graph** 
  * group); *changed = 1 if anything merged.  The graph must have merged, sorted lists. */
 int viecut_step_pr_a(viecut_graph* g, int64_t lambda_hat, int32_t* labels, int32_t* changed);
 int viecut_step_pr_b(viecut_graph* g, int64_t lambda_hat, int32_t* labels, int32_t* changed);
-/* One Nagamochi-Ono-Ibaraki round (Sec. 3) with bound lambda_hat: labels[n] as above. */
+/* One Nagamochi-Ono-Ibaraki round (Sec. 3) with bound lambda_hat: labels[n] as above.
+ * Entries of negative weight count as 0. */
 int viecut_step_noi_round(viecut_graph* g, int64_t lambda_hat, int32_t* labels, int32_t* changed);
 
 /* One Nagamochi-Ono-Ibaraki round, like viecut_step_noi_round, that allocates no

@@ -19,8 +19,7 @@ struct GraphView {
   // Every entry has its reverse.  False only where something relies on it (sparse_touches,
   // converging label rounds) and the input was found otherwise; those then read every list.
   bool symmetric = true;
-  // 64-bit weights nothing checked: some are below 0, or their sums may leave 64 bits
-  bool wraps = false;
+  bool wraps = false;   // 64-bit weights nothing checked: their sums may leave 64 bits
   // batches: label propagation touches only vertices v with vact[v] != 0 (null: all)
   const unsigned char* vact = nullptr;
   // source vertex of every entry (contracted graphs; null when not built)

@@ -455,7 +455,7 @@ struct StepGraph {
   bool simple = false;
   bool symmetric = true;
   bool unit = false;  // every weight is 1: the kernels that can then read no weights
-  bool wraps = false; // a round's sums may leave 64 bits (GraphView::wraps)
+  bool wraps = false; // sums of the weights may leave 64 bits
   Buf off, adj, w;
   GraphView view() const {
     GraphView g;
@@ -782,10 +782,11 @@ int viecut_graph_upload(viecut_graph** g, const int64_t* offsets, const int32_t*
         if (adj[e + 1] <= adj[e]) { x->g.simple = false; break; }
     x->g.unit = true;
     for (int64_t e = 0; e < nnz && x->g.unit; ++e) x->g.unit = weights[e] == 1;
-    // a weight below 0 counts as a round's bound there, which may be any size
-    uint64_t sum = 0;  // of the weights, until it passes 2^61
-    for (int64_t e = 0; e < nnz && !x->g.unit && !x->g.wraps; ++e)
-      x->g.wraps = weights[e] < 0 || weights[e] >> 61 || (sum += (uint64_t)weights[e]) >> 61;
+    uint64_t sum = 0;  // of the weights' magnitudes, until it passes 2^61
+    for (int64_t e = 0; e < nnz && !x->g.unit && !x->g.wraps; ++e) {
+      const uint64_t a = weights[e] < 0 ? 0 - (uint64_t)weights[e] : (uint64_t)weights[e];
+      x->g.wraps = a >> 61 || (sum += a) >> 61;
+    }
     VC_CUDA(cudaMemcpy(x->g.off.ensure_n<int64_t>(n + 1), offsets, sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice));
     x->g.adj.ensure_n<int32_t>(nnz);
     x->g.w.ensure_n<long long>(nnz);

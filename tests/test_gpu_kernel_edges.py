@@ -81,8 +81,8 @@ def any_round(G, lam):
 
 @pytest.mark.parametrize("n", [2, 40, 513, 4000, 16384, 16390])
 def test_exact_round_unchecked_weights(n):
-    """A step takes any 64-bit weights: those below 0 count as the bound, sums may pass 2^63,
-    and every vertex is still taken exactly once."""
+    """A step takes any 64-bit weights: those below 0 count as 0, sums may pass 2^63, and every
+    vertex is still taken exactly once."""
     g = ring_graph(n, 3 + n, 1, 9)
     G = oracle.as_csr64(g.offsets, g.adj, g.w)
     src = np.repeat(np.arange(n), np.diff(G.offsets))
@@ -92,7 +92,7 @@ def test_exact_round_unchecked_weights(n):
         d = vc.viecut_graph_upload(G.offsets, G.adj, w)
         try:
             for lam in bounds:
-                ref = any_round(oracle.CsrGraph(G.offsets, G.adj, np.where(w < 0, lam, w)), lam)
+                ref = any_round(oracle.CsrGraph(G.offsets, G.adj, np.maximum(w, 0)), lam)
                 got, ch = vc.viecut_step_noi_round(d, lam)
                 assert np.array_equal(got, ref), lam
                 assert ch == int(any(ref[v] != v for v in range(n)))
@@ -102,8 +102,8 @@ def test_exact_round_unchecked_weights(n):
 
 @pytest.mark.parametrize("n", [2, 40, 513, 4000, 16384, 16390])
 def test_exact_round_negative_weights_large_bounds(n):
-    """Few small weights, some below 0, under bounds near 2^63: an entry that counts as the bound
-    carries its vertex across, and the next ones carry the value past the end of its range."""
+    """Few small weights, some below 0, under bounds near 2^63, at which two entries of the bound
+    would already leave 64 bits."""
     g = ring_graph(n, 9 + n, 1, 9)
     G = oracle.as_csr64(g.offsets, g.adj, g.w)
     src = np.repeat(np.arange(n), np.diff(G.offsets))
@@ -111,7 +111,7 @@ def test_exact_round_negative_weights_large_bounds(n):
     d = vc.viecut_graph_upload(G.offsets, G.adj, w)
     try:
         for lam in (1 << 61, (1 << 62) + 5, (1 << 63) - 1):
-            ref = any_round(oracle.CsrGraph(G.offsets, G.adj, np.where(w < 0, lam, w)), lam)
+            ref = any_round(oracle.CsrGraph(G.offsets, G.adj, np.maximum(w, 0)), lam)
             got, ch = vc.viecut_step_noi_round(d, lam)
             assert np.array_equal(got, ref), lam
             assert ch == int(any(ref[v] != v for v in range(n)))
