@@ -45,7 +45,8 @@ struct BinOut {
 };
 
 // With a vertex list (list_n not null), the listed vertices list[0, *list_n) are binned
-// instead of [0, n) (n is then only the list's capacity).
+// instead of [0, n) (n is then only the list's capacity).  ENTRIES: *keep.entries is added to.
+template <bool ENTRIES>
 __global__ void __launch_bounds__(256) bins_k(int64_t n, int64_t chunk, const int64_t* __restrict__ off, BinOut out,
                                               int* __restrict__ counts, const int32_t* __restrict__ list,
                                               const int* __restrict__ list_n, KeepLabels keep) {
@@ -72,9 +73,9 @@ __global__ void __launch_bounds__(256) bins_k(int64_t n, int64_t chunk, const in
 #pragma unroll
     for (int q = 0; q < kBinClasses; ++q) c[q] += k == q;
     if (k >= 2) dmax = max(dmax, (int)(d < INT_MAX ? d : INT_MAX));
-    if (k >= 0) len += (unsigned long long)d;
+    if (ENTRIES && k >= 0) len += (unsigned long long)d;
   }
-  if (keep.entries) {
+  if (ENTRIES) {
     len = warp_sum(len);
     if (lane == 0 && len) atomicAdd(keep.entries, len);
   }
@@ -127,7 +128,8 @@ void bins_build(const GraphView& g, Bins& b, cudaStream_t s, const int32_t* list
   const int64_t blocks = std::min<int64_t>((g.n + 255) / 256, (int64_t)kSMs * 8);
   const int64_t chunk = (g.n + blocks - 1) / blocks;
   BinOut out{{b.small_list, b.reg_list, b.mid_list, b.block_list, b.global_list}, {4, 5, 0, 1, 2}};
-  bins_k<<<(int)blocks, 256, 0, s>>>(g.n, chunk, g.off, out, b.counts, list, list_n, keep);
+  auto kfn = keep.entries ? bins_k<true> : bins_k<false>;
+  kfn<<<(int)blocks, 256, 0, s>>>(g.n, chunk, g.off, out, b.counts, list, list_n, keep);
   count_launch();
   VC_CHECK_LAUNCH();
 }
