@@ -89,10 +89,10 @@ __device__ __forceinline__ int warp_argmax_unseen(const long long* r, const int*
 // the untaken vertex of largest attachment holds the largest r read as unsigned.
 //
 // A vertex is taken at most once whatever the weights, so the queue (n places) never
-// overflows: a weight above lam counts as lam (which crosses it as the weight itself does), a
-// negative one, which only an input that nothing checked can hold, as 0, so that r never
-// falls; and on graphs whose sums may leave 64 bits (GraphView::wraps) a taken vertex is not
-// added to any more, so that r cannot come back below 0 around the end of its range either.
+// overflows: a negative weight, which only an input that nothing checked can hold, counts as
+// 0, so that r never falls; and on graphs whose sums may leave 64 bits (GraphView::wraps) a
+// taken vertex is not added to any more, so that r cannot come back below 0 around the end of
+// its range either (-lam plus one weight stays inside it).
 //
 // Measured (RHG n = 8191, average degree 32, unit weights: 612 runs, 2174 levels): 1.66 ms a
 // round, about 1400 cycles a level (450 of them the lists' L2 access) and 1100 a choice,
@@ -108,8 +108,8 @@ struct NoiShared {
 };
 
 // The state in shared memory.  R = int serves graphs in which lam x entries stays below
-// 2^31, so no sum of weights of at most lam wraps.  kOff: the list offsets are kept too
-// (they are read from goff otherwise).
+// 2^31: weights are cut to lam (which crosses it as the weight itself does), so no sum
+// wraps.  kOff: the list offsets are kept too (they are read from goff otherwise).
 template <typename RT, typename OT, bool kOff>
 struct ClosureSmem {
   using R = RT;
@@ -298,7 +298,7 @@ __device__ __forceinline__ bool noi_closure_block(int32_t lo, int n, const int32
             if (e < len) {
               y[q] = __ldg(a + e) - lo;
               const long long x64 = ldw(w, e0 + beg + e);
-              c[q] = x64 < 0 ? 0 : x64 > (long long)lam ? lam : (R)x64;
+              c[q] = x64 < 0 ? 0 : (sizeof(R) == 4 && x64 > (long long)lam) ? lam : (R)x64;
             }
           }
 #pragma unroll
